@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace soft {
 
 // Barrier of the threads that own one transform: the whole CTA
@@ -12,9 +14,17 @@ namespace soft {
 // transforms side by side (named barrier `id`, `n` threads).
 struct BarCTA {
     __device__ __forceinline__ void sync() const { __syncthreads(); }
+    // barrier; true where any thread's p is
+    __device__ __forceinline__ bool any(bool p) const { return __syncthreads_or(p) != 0; }
 };
 struct BarGroup {
     int id, n;
+    __device__ __forceinline__ bool any(bool p) const {
+        int r;
+        asm volatile("{\n .reg .pred a, b;\n setp.ne.s32 a, %1, 0;\n bar.red.or.pred b, %2, %3, a;\n"
+                     " selp.s32 %0, 1, 0, b;\n}\n" : "=r"(r) : "r"((int)p), "r"(id), "r"(n) : "memory");
+        return r != 0;
+    }
     __device__ __forceinline__ void sync() const {
         asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
     }
@@ -135,11 +145,14 @@ __device__ __forceinline__ C twc(C a) {
     }
 }
 
+template <int R, int SIGN, int t> __device__ __forceinline__ longlong2 fx_twc(longlong2 a);   // fix64.cuh
+
 template <typename C, int R, int SIGN, int SPAN, int BLK, int J>
 __device__ __forceinline__ void dif_bfly(C* v) {
     C a = v[BLK + J], b = v[BLK + J + SPAN];
     v[BLK + J] = cadd(a, b);
-    v[BLK + J + SPAN] = twc<C, 2 * SPAN, SIGN, J>(csub(a, b));
+    if constexpr (std::is_same<C, longlong2>::value) v[BLK + J + SPAN] = fx_twc<2 * SPAN, SIGN, J>(csub(a, b));
+    else v[BLK + J + SPAN] = twc<C, 2 * SPAN, SIGN, J>(csub(a, b));
 }
 
 template <typename C, int R, int SIGN, int SPAN, int BLK, int J>

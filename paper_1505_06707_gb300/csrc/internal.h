@@ -18,11 +18,13 @@ using cd = std::complex<double>;
 // Device descriptor of one 1D instance (read by the 1D step kernel).
 struct Inst1D {
     int64_t off;          // element offset of the instance in the packed state
-    const void* TK;       // e^{-i k^2 tau/2}/N, forward FFT output order, last-pass transposed
-    const void* TKh;      // e^{-i k^2 tau/4}/N, same order (first/last half step)
-    const void* TV;       // e^{-iU0 tau} off the strip block, e^{-iU0 tau/2} on it (minus 1 for complex64)
-    const void* W;        // per-pass twiddle bases (see soft1d.cuh)
-    const void* cn;       // strip CN coefficients, chunk-transposed (soft1d.cuh, strip_cn_1d)
+    const void* TK;       // e^{-i k^2 tau/2}, forward FFT output order, last-pass transposed (complex64: over N)
+    const void* TKh;      // e^{-i k^2 tau/4}, same order (first/last half step)
+    const void* TV;       // e^{-iU0 tau} off the strip block, e^{-iU0 tau/2} on it (minus 1 for complex64;
+                          // complex128: FxV in soft1d_fix.cuh)
+    const void* W;        // per-pass twiddles (complex64: bases, soft1d.cuh; complex128: FxGeom, soft1d_fix.cuh)
+    const void* cn;       // strip CN coefficients, chunk-transposed (soft1d.cuh, strip_cn_1d; complex128:
+                          // FxCn in soft1d_fix.cuh)
     const void* TVs;      // TV on the strip rows, same transposed order
     int nb;               // strip block length (0: no absorbing term)
     int blk0;             // first grid index of the block (cyclic)
@@ -39,6 +41,7 @@ struct Inst1D {
 struct Tables1D {
     int prec = 0, logn = 0, loge = 0, logrm = 0;
     int nb = 0, blk0 = 0, iL = 0, iR = 0;
+    bool cn_gen = false;          // complex128: the strip solve is not fit for fixed point
     double R0 = 0, theta = 0;
     Axis1D ax;                    // host FP64 grid, contour, C
     std::vector<cd> U0;           // potential at z(x_j)
@@ -51,9 +54,28 @@ struct Tables1D {
     void* TVs = nullptr;
 };
 
-// Complex128 1D step plans store every pass twiddle W^{M off} for passes of
-// stride up to this (the bases above it), see soft1d.cuh.
+// Passes of stride up to this store every twiddle W^{M off}, the others a few
+// bases: the complex128 line passes of the 2D and 3D steps (soft1d.cuh,
+// TwFull) and the complex128 1D step (soft1d_fix.cuh, FxGeom).
 constexpr int TWFULL_MAXS = 256;
+constexpr int FXFULL_MAXS = 256;
+
+// Centre of the complex128 1D step (soft1d_fix.cuh).  The centre (last forward pass of r bits, k-space factor, first inverse
+// pass) must leave its outputs as an inverse pass of LOGRM bits would,
+// 2^(LOGRM/2) above unitary: the factor takes 2^-(r - LOGRM/2 + cs), stored
+// outputs are shifted left by the smallest cs that keeps the factor's product
+// in range.  The host scales the table by sqrt(2) if s2.
+struct FxCenter { int K, cs; bool s2; };
+__host__ __device__ constexpr FxCenter fx_center(int r, int logrm) {
+    for (int cs = 0; cs < 8; ++cs) {
+        const int y2 = 2 * r - logrm + 2 * cs;            // half bits
+        if (y2 < 0) continue;
+        const bool s2 = y2 & 1;
+        const int K = 2 - (y2 + 1) / 2;
+        if (K >= 0 && r + 2 * K <= (s2 ? 3 : 4)) return FxCenter{K, cs, s2};
+    }
+    return FxCenter{-1, 0, false};
+}
 
 // Work item of the persistent batch kernel: up to G instances of one size.
 struct Pack1D {

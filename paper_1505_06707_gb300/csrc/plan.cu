@@ -7,6 +7,7 @@
 #include <map>
 #include <tuple>
 
+#include "fix64_host.h"
 #include "nn.h"
 #include "plan_internal.h"
 
@@ -105,6 +106,161 @@ int upload_tw_comp(void** dst, const std::vector<cd>& v, int prec) {
     return upload_tab(dst, v, prec);
 }
 
+static void fx_fill(int32_t* out, const std::vector<cd>& v, double scale) {
+    for (size_t i = 0; i < v.size(); ++i) {
+        fx_halves_host(std::llrint(v[i].real() * scale * 0x1p62), out + 4 * i);
+        fx_halves_host(std::llrint(v[i].imag() * scale * 0x1p62), out + 4 * i + 2);
+    }
+}
+int upload_fx(void** dst, const std::vector<cd>& v) {
+    std::vector<int32_t> buf(4 * v.size());
+    fx_fill(buf.data(), v, 1.0);
+    return upload(dst, buf.data(), buf.size() * sizeof(int32_t));
+}
+
+// e^{i ph} as factors, times sqrt(2) if s2 (soft1d_fix.cuh: passes of odd radix)
+static int upload_fx_phases(void** dst, const std::vector<double>& ph, bool s2) {
+    std::vector<int32_t> buf(4 * ph.size());
+    for (size_t i = 0; i < ph.size(); ++i) {
+        int64_t c, s;
+        fx_cis_host(fx_turns_host(ph[i]), &c, &s);
+        fx_halves_host(s2 ? fx_sqrt2_host(c) : c, &buf[4 * i]);
+        fx_halves_host(s2 ? fx_sqrt2_host(s) : s, &buf[4 * i + 2]);
+    }
+    return upload(dst, buf.data(), buf.size() * sizeof(int32_t));
+}
+
+// potential table of the fixed-point step (soft1d_fix.cuh, FxV) from the
+// factors' logarithms: the factors times 2^-p, p = 0 (|v| <= 1.01) or 1 (<= 2),
+// and sqrt(2) if s2 (the last inverse pass's share), then the entry
+// (p, gen, 0, 0) and the factors as double2, which plans with gen use
+static std::vector<int32_t> fxv_table(const std::vector<cd>& lv, bool gen, bool s2) {
+    const size_t n = lv.size();
+    std::vector<int32_t> buf(8 * n + 4, 0);
+    double m = 0;
+    for (const cd& x : lv) m = std::max(m, std::exp(x.real()));
+    const int p = !gen && m > 1.01 ? 1 : 0;
+    for (size_t i = 0; i < n && !gen; ++i) {
+        int64_t c, s;
+        fx_cis_host(fx_turns_host(lv[i].imag()), &c, &s);
+        const int64_t mod = std::llrint(std::exp(lv[i].real()) * (p ? 0x1p60 : 0x1p61));
+        c = (int64_t)(((__int128)c * mod + (1LL << 60)) >> 61);
+        s = (int64_t)(((__int128)s * mod + (1LL << 60)) >> 61);
+        fx_halves_host(s2 ? fx_sqrt2_host(c) : c, &buf[4 * i]);
+        fx_halves_host(s2 ? fx_sqrt2_host(s) : s, &buf[4 * i + 2]);
+    }
+    buf[4 * n] = p;
+    buf[4 * n + 1] = gen;
+    for (size_t i = 0; i < n; ++i) {
+        const cd v = std::exp(lv[i]);
+        std::memcpy(buf.data() + 4 * n + 4 + 4 * i, &v, 16);
+    }
+    return buf;
+}
+// a gain above 2 or a non-finite factor
+static bool fxv_gen(const std::vector<cd>& lv) {
+    for (const cd& x : lv)
+        if (!(std::exp(x.real()) <= 2.0) || !std::isfinite(x.imag())) return true;
+    return false;
+}
+
+// Strip tables of the fixed-point step (soft1d_fix.cuh, FxCn) from the LU of
+// the block: thr threads of ch rows each.  gen: a multiplier above 1, a g
+// above 1.9 (its halves still fit, and the rows it scales are below 2^59.5)
+// or a growth of the sweeps above 2^10; the kernel then solves in FP64.
+static std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vector<cd>& mb,
+                                            const std::vector<cd>& g, int nb, int thr, bool* gen) {
+    const int ch = (nb + thr - 1) / thr, nw = thr / 32;
+    const double tiny = 0x1p-70;
+    double grow = 1.0, gy = 0.0;
+    std::vector<double> y(nb);
+    *gen = false;
+    for (int i = 0; i < nb; ++i) {
+        gy = std::abs(mf[i]) * gy + 1.0;
+        y[i] = gy;
+        grow = std::max(grow, gy);
+        if (!(std::abs(mf[i]) <= 1.0 + 1e-12 && std::abs(g[i]) <= 1.9)) *gen = true;
+    }
+    double gx = 0.0;
+    for (int i = nb - 1; i >= 0; --i) {
+        gx = std::abs(mb[i]) * gx + std::abs(g[i]) * y[i];
+        grow = std::max(grow, gx);
+    }
+    const int lg = (int)std::ceil(std::log2(grow));
+    if (!(lg >= 0 && lg <= 10)) *gen = true;
+    std::vector<cd> m((size_t)(ch + 1) * thr, 0.0), gg((size_t)ch * thr, 0.0), scan[2];
+    for (int t = 0; t < thr; ++t)
+        for (int c = 0; c <= ch; ++c) {
+            const int i = t * ch + c;
+            if (i < nb) m[(size_t)c * thr + t] = mf[i];
+            if (c < ch && i < nb) gg[(size_t)c * thr + t] = g[i];
+        }
+    int rounds[2], span[2];
+    for (int d = 0; d < 2; ++d) {
+        std::vector<cd> tot(thr, 1.0);
+        for (int t = 0; t < thr; ++t)
+            for (int c = 0; c < ch && t * ch + c < nb; ++c) tot[t] *= m[(size_t)(c + d) * thr + t];
+        std::vector<cd>& s = scan[d];
+        s.assign((size_t)6 * thr + nw, 1.0);
+        std::vector<cd> prod = tot;              // of the 2^r totals ending (starting) at t
+        rounds[d] = 0;
+        for (int r = 0; r < 5; ++r) {
+            const int D = 1 << r;
+            double big = 0.0;
+            for (int t = 0; t < thr; ++t) {
+                s[(size_t)r * thr + t] = prod[t];
+                const int l = t & 31;
+                if (d ? l + D < 32 : l >= D) big = std::max(big, std::abs(prod[t]));
+            }
+            if (big > tiny) rounds[d] = r + 1;
+            std::vector<cd> nx = prod;
+            for (int t = 0; t < thr; ++t) {
+                const int o = d ? t + D : t - D;
+                if (o >= 0 && o < thr) nx[t] = prod[t] * prod[o];
+            }
+            prod = nx;
+        }
+        for (int w = 0; w < nw; ++w) {
+            cd p = 1.0;
+            for (int l = 0; l < 32; ++l) {
+                const int t = 32 * w + (d ? 31 - l : l);
+                s[(size_t)5 * thr + t] = p;
+                p *= tot[t];
+            }
+            s[(size_t)6 * thr + w] = p;
+        }
+        span[d] = nw;                            // warps whose totals still reach
+        for (int k = 1; k < nw; ++k) {
+            double big = 0.0;
+            for (int w = 0; w + k <= nw; ++w) {
+                cd p = 1.0;
+                for (int q = 0; q < k; ++q) p *= s[(size_t)6 * thr + w + q];
+                big = std::max(big, std::abs(p));
+            }
+            if (big <= tiny) { span[d] = k; break; }
+        }
+    }
+    std::vector<cd> all = m;
+    all.insert(all.end(), gg.begin(), gg.end());
+    all.insert(all.end(), scan[0].begin(), scan[0].end());
+    all.insert(all.end(), scan[1].begin(), scan[1].end());
+    std::vector<int32_t> buf(4 + 4 * (all.size() + m.size() + gg.size()), 0);
+    buf[0] = *gen ? 0 : lg;
+    buf[1] = rounds[0];
+    buf[2] = rounds[1];
+    buf[3] = span[0] | span[1] << 16;
+    if (!*gen) {
+        std::vector<int32_t> f(4 * all.size());
+        fx_fill(f.data(), all, 1.0);
+        std::memcpy(buf.data() + 4, f.data(), 16 * all.size());
+    }
+    std::memcpy(buf.data() + 4 + 4 * all.size(), m.data(), 16 * m.size());
+    std::memcpy(buf.data() + 4 + 4 * (all.size() + m.size()), gg.data(), 16 * gg.size());
+    return buf;
+}
+
+static int upload_i32(void** dst, const std::vector<int32_t>& v) { return upload(dst, v.data(), v.size() * 4); }
+
 // the upload_* conversions into a temporary device buffer, then one copy
 // into dst
 static int refill_with(int (*up)(void**, const std::vector<cd>&, int), void* dst,
@@ -120,29 +276,33 @@ static int refill_with(int (*up)(void**, const std::vector<cd>&, int), void* dst
 int refill_c(void* dst, const std::vector<cd>& v, int prec) { return refill_with(upload_c, dst, v, prec); }
 int refill_vtab(void* dst, const std::vector<cd>& v, int prec) { return refill_with(upload_vtab, dst, v, prec); }
 
-// Potential factors of one step from U0 (Sec. II, the scheme after Eq. C_FD):
-// tv[j] = e^{-iU0 tau} off the strip block (both half factors merged),
-// e^{-iU0 tau/2} on it (the strip CN sits between the halves); tvs holds
-// the block rows' factors in the chunk layout of the strip CN (thread t of
-// the n >> loge threads owns rows t*ch .. t*ch + ch - 1, entry c*T + t).
-static void potential_tables_1d(const Tables1D& T, int n, double tau, std::vector<cd>& tv,
-                                std::vector<cd>& tvs) {
+// Logarithms of the potential factors of one step from U0 (Sec. II, the
+// scheme after Eq. C_FD): e^{tv[j]} = e^{-iU0 tau} off the strip block (both
+// half factors merged), e^{-iU0 tau/2} on it (the strip CN sits between the
+// halves); tvs holds the block rows' in the chunk layout of the strip CN
+// (thread t of the n >> loge threads owns rows t*ch .. t*ch + ch - 1, entry
+// c*T + t).
+static void potential_logs_1d(const Tables1D& T, int n, double tau, std::vector<cd>& tv, std::vector<cd>& tvs) {
     tv.resize(n);
     for (int j = 0; j < n; ++j) {
         const bool inblk = ((j - T.blk0 + n) % n) < T.nb;
-        tv[j] = std::exp(cd(0.0, -1.0) * T.U0[j] * tau * (inblk ? 0.5 : 1.0));
+        tv[j] = cd(0.0, -1.0) * T.U0[j] * tau * (inblk ? 0.5 : 1.0);
     }
     tvs.clear();
     if (T.nb > 0) {
         const int thr = n >> T.loge, nb = T.nb;
         const int ch = (nb + thr - 1) / thr;
-        tvs.assign((size_t)ch * thr, 1.0);
+        tvs.assign((size_t)ch * thr, 0.0);
         for (int t = 0; t < thr; ++t)
             for (int c = 0; c < ch; ++c) {
                 const int i = t * ch + c;
                 if (i < nb) tvs[(size_t)c * thr + t] = tv[(T.blk0 + i) % n];
             }
     }
+}
+static std::vector<cd> vexp(std::vector<cd> v) {
+    for (cd& x : v) x = std::exp(x);
+    return v;
 }
 
 static int ilog2(int64_t n) {
@@ -179,9 +339,11 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
         T->U0[j] = soft_coulomb(&A.z[j], 1, o.soft_a2, o.charge) + T->Uabs[j];
     }
     // kinetic tables in the forward FFT's output order, 1/N folded in
+    // (complex128: the fixed-point passes carry the 1/N)
     const std::vector<int> perm = dif_output_order(logn, logrm);
     std::vector<cd> tk(n), tkh(n), tv, tvs;
-    const std::vector<cd> w = pass_twiddles(logn, logrm);
+    std::vector<double> ph(n), phh(n);        // complex128: their phases
+    const std::vector<cd> w = o.prec == SOFT_C64 ? pass_twiddles(logn, logrm) : std::vector<cd>();
     // The step kernel reads them in its last forward pass, whose butterflies
     // hold R consecutive positions b*R + m (R its radix): entry (b, m) is
     // stored at m*(n/R) + b, so that a warp's reads are contiguous.
@@ -190,16 +352,19 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
     for (int p = 0; p < n; ++p) {
         const double k = A.k[perm[p]];
         const int q = (p % Rl) * nbf + p / Rl;
-        tk[q] = std::polar(1.0 / n, -0.5 * k * k * tau);
-        tkh[q] = std::polar(1.0 / n, -0.25 * k * k * tau);
+        ph[q] = -0.5 * k * k * tau;
+        phh[q] = -0.25 * k * k * tau;
+        tk[q] = std::polar(1.0 / n, ph[q]);
+        tkh[q] = std::polar(1.0 / n, phh[q]);
     }
-    potential_tables_1d(*T, n, tau, tv, tvs);
+    potential_logs_1d(*T, n, tau, tv, tvs);
     // Strip CN coefficients for the kernel's chunked solve: thread t of the
     // T = n >> loge threads owns rows t*ch .. t*ch + ch - 1 (ch = ceil(nb/T)).
     // M is complex symmetric, so mb_i = mf_{i+1}: the kernel reads mf of rows
     // t*ch + c, c <= ch, at c*T + t (0 past the block), then g of row t*ch + c
     // at (ch+1)*T + c*T + t (tvs holds the rows' potential factors).
     std::vector<cd> mf, mb, g, cnv;
+    std::vector<int32_t> cnfx;
     if (T->nb > 0) {
         double err = 0;
         rc = strip_factor(A, T->blk0, T->nb, mf, mb, g, &err);
@@ -207,6 +372,7 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
         const int thr = n >> loge, nb = T->nb;
         for (int i = 0; i + 1 < nb; ++i)
             if (std::abs(mb[i] - mf[i + 1]) > 1e-12 * (std::abs(mb[i]) + 1e-300)) return SOFT_ERR_SETUP;
+        if (o.prec == SOFT_C128) cnfx = strip_tables_fx(mf, mb, g, nb, thr, &T->cn_gen);
         const int ch = (nb + thr - 1) / thr, P1 = (ch + 1) * thr;
         cnv.assign((size_t)P1 + (size_t)ch * thr, 0.0);
         for (int t = 0; t < thr; ++t)
@@ -216,16 +382,22 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
                 if (c < ch && i < nb) cnv[P1 + (size_t)c * thr + t] = g[i];
             }
     }
+    if (o.prec == SOFT_C128) {
+        const bool gen = T->cn_gen || fxv_gen(tv);
+        if ((rc = upload_i32(&T->cn, cnfx))) return rc;
+        const bool s2 = fx_center(lrl, logrm).s2;
+        if ((rc = upload_fx_phases(&T->TK, ph, s2))) return rc;
+        if ((rc = upload_fx_phases(&T->TKh, phh, s2))) return rc;
+        if ((rc = upload_i32(&T->W, pass_twiddles_fx(logn, logrm, FXFULL_MAXS)))) return rc;
+        if ((rc = upload_i32(&T->TV, fxv_table(tv, gen, logrm & 1)))) return rc;
+        return tvs.empty() ? SOFT_OK : upload_i32(&T->TVs, fxv_table(tvs, gen, false));
+    }
+    if ((rc = upload_c(&T->cn, cnv, o.prec))) return rc;
     if ((rc = upload_tab(&T->TK, tk, o.prec))) return rc;
     if ((rc = upload_tab(&T->TKh, tkh, o.prec))) return rc;
-    if ((rc = upload_vtab(&T->TV, tv, o.prec))) return rc;
-    if (o.prec == SOFT_C128)   // every twiddle of the small-stride passes (see soft1d.cuh, TwFullD)
-        rc = upload_c(&T->W, pass_twiddles_full(logn, logrm, TWFULL_MAXS), o.prec);
-    else
-        rc = upload_tw_comp(&T->W, w, o.prec);
-    if (rc) return rc;
-    if ((rc = upload_c(&T->cn, cnv, o.prec))) return rc;
-    if ((rc = upload_vtab(&T->TVs, tvs, o.prec))) return rc;
+    if ((rc = upload_vtab(&T->TV, vexp(tv), o.prec))) return rc;
+    if ((rc = upload_tw_comp(&T->W, w, o.prec))) return rc;
+    if ((rc = upload_vtab(&T->TVs, vexp(tvs), o.prec))) return rc;
     return SOFT_OK;
 }
 
@@ -544,9 +716,20 @@ static int soft_set_potential_impl(soft_plan* P, const double* U, int64_t n) {
     if (rc) return rc;
     for (int j = 0; j < nn; ++j) T->U0[j] = cd(U[2 * j], U[2 * j + 1]) + T->Uabs[j];
     std::vector<cd> tv, tvs;
-    potential_tables_1d(*T, nn, P->dt, tv, tvs);
-    if ((rc = refill_vtab(T->TV, tv, T->prec))) return rc;
-    if ((rc = refill_vtab(T->TVs, tvs, T->prec))) return rc;
+    potential_logs_1d(*T, nn, P->dt, tv, tvs);
+    if (T->prec == SOFT_C128) {
+        const bool gen = T->cn_gen || fxv_gen(tv);
+        for (int i = 0; i < 2; ++i) {
+            const std::vector<cd>& v = i ? tvs : tv;
+            if (v.empty()) continue;
+            const std::vector<int32_t> b = fxv_table(v, gen, !i && (T->logrm & 1));
+            rc = cuda_status(cudaMemcpy(i ? T->TVs : T->TV, b.data(), b.size() * 4, cudaMemcpyHostToDevice));
+            if (rc) return rc;
+        }
+        return sse1d_refill_potential(P);
+    }
+    if ((rc = refill_vtab(T->TV, vexp(tv), T->prec))) return rc;
+    if ((rc = refill_vtab(T->TVs, vexp(tvs), T->prec))) return rc;
     return sse1d_refill_potential(P);
 }
 int soft_set_potential(soft_plan* P, const double* U, int64_t n) {

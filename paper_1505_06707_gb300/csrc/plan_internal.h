@@ -30,6 +30,8 @@ int upload_tw(void** dst, const std::vector<cd>& v, int prec);
 int upload_tw_comp(void** dst, const std::vector<cd>& v, int prec);
 // rewrite an existing device buffer in place (same size and format as the
 // matching upload_*), so that pointers held by kernels and graphs stay valid
+// fixed-point factors |v| <= 1 (fix64.cuh)
+int upload_fx(void** dst, const std::vector<cd>& v);
 int refill_c(void* dst, const std::vector<cd>& v, int prec);
 int refill_vtab(void* dst, const std::vector<cd>& v, int prec);
 struct Plan2D;

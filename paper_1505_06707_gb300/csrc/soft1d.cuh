@@ -64,20 +64,19 @@ __device__ __forceinline__ float2 tmulc(float2 x, float4 t) {
 // same position, that modulus error returns unchanged in every step and the
 // state drifts linearly in time.  With compensated factors the modulus is
 // exact to ~2^-48 and only the data's own roundings remain.
-// Complex128 plans of the 1D step store, for passes with a stride of at
-// most TWFULL_MAXS, every twiddle W^{M off} (M = 1 .. R-1) instead of the
-// four bases: the products of bases cost 16 of the ~100 FP64 instructions
-// of a radix-8 butterfly, and the kernel is bound by the FP64 pipe.  Passes
-// with a larger stride keep the bases (their full table would not fit in
-// shared memory).  The complex64 line passes of the 2D and 3D steps use the
-// same layout with float2 entries.
+// Complex128 plans of the 1D step store fixed-point factors (TwFix,
+// soft1d_fix.cuh).  The complex128 line passes of the 2D and 3D steps store,
+// for passes with a stride of at most TWFULL_MAXS, every twiddle W^{M off}
+// (M = 1 .. R-1) instead of the four bases: the products of bases cost 16 of
+// the ~100 FP64 instructions of a radix-8 butterfly, and those kernels are
+// bound by the FP64 pipe.
 template <typename C> struct TwFull { C v; };
-using TwFullD = TwFull<double2>;
-using TwFullF = TwFull<float2>;
+struct TwFix { int4 v; };
+constexpr int FX_FR = 68;       // field factors of the fixed-point step behind its 2 E per-row ones
 
 template <typename R> struct TwT;
 template <> struct TwT<float> { using T = float4; };
-template <> struct TwT<double> { using T = TwFullD; };
+template <> struct TwT<double> { using T = TwFix; };
 
 template <typename R, int LOGN, int LOGE, int LOGRM>
 struct Cfg1D {
@@ -94,7 +93,7 @@ struct Cfg1D {
     static constexpr int MINB = T >= 512 ? 1 : 512 / T;   // CTAs per SM the registers must allow (128 regs)
     // state larger than a CTA's shared memory (complex128, N = 16384): the
     // step kernel works on the instance's own buffer in global memory (L2
-    // resident while the CTA runs; such plans are bound by FP64 arithmetic)
+    // resident while the CTA runs)
     static constexpr bool GM = sizeof(C) * N > 160 * 1024;
 };
 
@@ -252,6 +251,17 @@ struct TwCountT<TwFull<C>, LOGN, LOGRM> {
     static constexpr int value = TwGeomFull<LOGN, LOGRM, NP - 1>::TOFF +
                                  TwGeomFull<LOGN, LOGRM, NP - 1>::ROWS * PassGeom<LOGN, LOGRM, NP - 1>::S;
 };
+
+template <typename R, int LOGN, int LOGRM>
+struct Step1D {
+    static constexpr int NPASS = LOGN / LOGRM + ((LOGN % LOGRM) ? 1 : 0);
+    static constexpr int LOGR0 = PassGeom<LOGN, LOGRM, 0>::LOGR;   // radix of pass 0
+    static constexpr int R0 = 1 << LOGR0;
+};
+
+}  // namespace soft
+#include "soft1d_fix.cuh"
+namespace soft {
 
 // forward DIF pass P (radix 2^LOGR on sub-transforms of length 2^LOGL)
 template <typename R, int LOGN, int LOGE, int LOGRM, int P, bool SH = false, typename TW = typename CT<R>::C>
@@ -474,7 +484,6 @@ __device__ __forceinline__ void strip_cn_1d(C* S, const C* __restrict__ cn, cons
 }
 
 __device__ __forceinline__ void sincos_r(float a, float* s, float* c) { sincosf(a, s, c); }
-__device__ __forceinline__ void sincos_r(double a, double* s, double* c) { sincos(a, s, c); }
 
 // ---------------------------------------------------------------------------
 // Pieces of the resident step kernel.  Twiddles are read from a shared-memory
@@ -482,21 +491,21 @@ __device__ __forceinline__ void sincos_r(double a, double* s, double* c) { sinco
 // run as one in-register butterfly; the potential factor is applied as the
 // last inverse pass stores its outputs.
 
-template <typename R, int LOGN, int LOGRM>
-struct Step1D {
-    static constexpr int NPASS = LOGN / LOGRM + ((LOGN % LOGRM) ? 1 : 0);
-    static constexpr int TWN = TwCountT<typename TwT<R>::T, LOGN, LOGRM>::value;
-    static constexpr int LOGR0 = PassGeom<LOGN, LOGRM, 0>::LOGR;   // radix of pass 0
-    static constexpr int R0 = 1 << LOGR0;
-};
+// shared-memory bytes of one instance's private part: the state (unless
+// GM), 64 complex of scan scratch and the field phases (complex64: E
+// per-butterfly, 16 per-output, 4 clamped, 16 strip rows inside R0, 16
+// per-output squares; complex128: 2 E + FX_FR factors and 32 words of sums)
+template <typename R, int LOGN, int LOGE, int LOGRM>
+__host__ __device__ constexpr size_t soft1d_inst_smem() {
+    return sizeof(typename CT<R>::C) *
+           ((Cfg1D<R, LOGN, LOGE, LOGRM>::GM ? 0 : (size_t(1) << LOGN)) + 64 + (size_t(1) << LOGE) +
+            (sizeof(R) == 8 ? (size_t(1) << LOGE) + FX_FR + 8 : 52));
+}
 
-// shared-memory bytes of soft1d_kernel: state, twiddles, scan scratch, field
-// phases (E per-butterfly, 16 per-output, 4 clamped, 16 strip rows inside R0,
-// 16 per-output squares)
+// shared-memory bytes of soft1d_kernel: the instance's part and the twiddles
 template <typename R, int LOGN, int LOGE, int LOGRM>
 __host__ __device__ constexpr size_t soft1d_smem() {
-    return sizeof(typename CT<R>::C) *
-               ((Cfg1D<R, LOGN, LOGE, LOGRM>::GM ? 0 : (size_t(1) << LOGN)) + 64 + (size_t(1) << LOGE) + 52) +
+    return soft1d_inst_smem<R, LOGN, LOGE, LOGRM>() +
            sizeof(typename TwT<R>::T) * TwCountT<typename TwT<R>::T, LOGN, LOGRM>::value + 64;
 }
 
@@ -521,15 +530,10 @@ __device__ __forceinline__ void inv_passes(typename CT<R>::C* S, const TW* Ws, i
 // inverse pass: butterfly b owns the R consecutive points b*R + m of the
 // digit-reversed spectrum, whose factors the table holds at m*(N/R) + b
 //
-// With SURF, the spectrum entering the k-space factor is also contracted with
-// four weight rows sw[r * N + q] (same transposed index q as the table) into
-// acc[r] (surface sampling, soft1d_surf_kernel).
-//
 // TSH: the table has been copied to shared memory (plain loads).
-template <typename R, int LOGN, int LOGE, int LOGRM, bool SURF = false, bool TSH = false>
+template <typename R, int LOGN, int LOGE, int LOGRM, bool TSH = false>
 __device__ __forceinline__ void kcenter(typename CT<R>::C* S, const typename TabT<R>::T* __restrict__ tab,
-                                        int tid, const typename CT<R>::C* __restrict__ sw = nullptr,
-                                        typename CT<R>::C* acc = nullptr) {
+                                        int tid) {
     using K = Cfg1D<R, LOGN, LOGE, LOGRM>;
     using C = typename K::C;
     using G = PassGeom<LOGN, LOGRM, K::NPASS - 1>;
@@ -570,14 +574,6 @@ __device__ __forceinline__ void kcenter(typename CT<R>::C* S, const typename Tab
 #pragma unroll
         for (int j = 0; j < RR; ++j) v[j] = S[sb ^ swz<C>(j)];
         dft_reg<C, RR, -1>(v);
-        if constexpr (SURF) {
-#pragma unroll
-            for (int m = 0; m < RR; ++m) {
-                const int q = m * (K::N / RR) + tid + u * K::T;
-#pragma unroll
-                for (int r = 0; r < 4; ++r) acc[r] = cfma(v[bitrev_c(m, LOGR)], __ldg(&sw[r * K::N + q]), acc[r]);
-            }
-        }
         C w[RR];
 #pragma unroll
         for (int m = 0; m < RR; ++m) w[m] = tmul(v[bitrev_c(m, LOGR)], tc[m]);
@@ -676,26 +672,14 @@ __device__ __forceinline__ void inv_pass0_v(typename CT<R>::C* S, const TW* __re
             C x = vmul(v[bitrev_c(m, LOGR)], __ldg(&TV[n]));
             if (fld) {
                 // off the block exp(-2i alpha x_n) from the squared tables; on it
-                // the half factor exp(-i alpha x_n), clamped beyond +-R0.  FP64
-                // (pipe-bound) branches, so that only one factor is formed (a
-                // warp diverges only where it straddles the block's edge); FP32
-                // (issue-bound) forms both, branch-free, so that the table
-                // loads of all m issue early.
+                // the half factor exp(-i alpha x_n), clamped beyond +-R0.  Both
+                // are formed, branch-free, so that the table loads of all m
+                // issue early (the kernel is issue-bound).
                 const bool inb = ((n - blk0) & (N - 1)) < nb;
-                C f;
-                if constexpr (sizeof(R) == 8) {
-                    if (inb) {
-                        const C fh = cmul(fb, fr[K::E + m]);
-                        f = n >= iR ? fcR : (n < iL ? fcL : fh);
-                    } else {
-                        f = cmul(fb2, fr[K::E + 36 + m]);
-                    }
-                } else {
-                    const C fh = cmul(fb, fr[K::E + m]);
-                    const C ff = cmul(fb2, fr[K::E + 36 + m]);
-                    const C fk = n >= iR ? fcR : (n < iL ? fcL : fh);
-                    f = inb ? fk : ff;
-                }
+                const C fh = cmul(fb, fr[K::E + m]);
+                const C ff = cmul(fb2, fr[K::E + 36 + m]);
+                const C fk = n >= iR ? fcR : (n < iL ? fcL : fh);
+                const C f = inb ? fk : ff;
                 x = cmul(x, f);
             }
             S[sb ^ swz<C>(m * s)] = x;
@@ -723,32 +707,6 @@ __device__ __forceinline__ C strip_field(const C* fr, R al, const Inst1D& I, int
     return field_direct<R, C>(al, I.x0, I.h, n);
 }
 
-// Sum of four complex values over the group; thread 0 writes them to out.
-// scratch: 4 * (T/32) complex (the scan scratch, free at this point).
-template <typename C, int T, class B>
-__device__ __forceinline__ void surf_reduce(C (&acc)[4], C* scratch, int tid, B bar, C* __restrict__ out) {
-    static_assert(T / 32 <= 16, "scratch of 64 complex");
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, o);
-            acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, o);
-        }
-    if ((tid & 31) == 0)
-#pragma unroll
-        for (int r = 0; r < 4; ++r) scratch[4 * (tid >> 5) + r] = acc[r];
-    bar.sync();
-    if (tid == 0) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            C t = cmk<C>(0, 0);
-            for (int w = 0; w < (T + 31) / 32; ++w) t = cadd(t, scratch[4 * w + r]);
-            out[r] = t;
-        }
-    }
-}
-
 // n 16-byte table entries from global to shared memory by nt threads
 template <typename TT>
 __device__ __forceinline__ void copy16(TT* dst, const TT* __restrict__ src, int n, int t, int nt) {
@@ -757,32 +715,31 @@ __device__ __forceinline__ void copy16(TT* dst, const TT* __restrict__ src, int 
         reinterpret_cast<float4*>(dst)[i] = __ldg(reinterpret_cast<const float4*>(src) + i);
 }
 
-// shared-memory bytes of one instance's private part: the state (unless
-// GM), 64 complex of scan scratch and E + 52 field phases
-template <typename R, int LOGN, int LOGE, int LOGRM>
-__host__ __device__ constexpr size_t soft1d_inst_smem() {
-    return sizeof(typename CT<R>::C) *
-           ((Cfg1D<R, LOGN, LOGE, LOGRM>::GM ? 0 : (size_t(1) << LOGN)) + 64 + (size_t(1) << LOGE) + 52);
-}
-
 // All nsteps steps of one instance, run by the T threads of a group (tid =
 // index in the group, bar = its barrier).  Ss: the state in shared memory
-// (unused with GM); scan: 64 complex of scan scratch followed by E + 52
-// field phases; Ws: the twiddle bases, already in shared memory and visible
-// to the group by its first barrier.
+// (unused with GM); scan: 64 complex of scan scratch followed by the field
+// phases; Ws: the twiddles, already in shared memory and visible
+// to the group by its first barrier.  Complex128 runs in fixed point
+// (soft1d_fix.cuh); the code below is complex64's.
 //
 // SURF: sample psi and psi' at the two surfaces into samples[0 ..
-// nsteps][4] (soft1d_surf_kernel; sw holds two sets of four weight rows:
-// for the state at the call's start and, with the half kinetic factor
+// nsteps][4] (complex128; soft1d_surf_kernel; sw holds two sets of four weight
+// rows: for the state at the call's start and, with the half kinetic factor
 // e^{-iK tau/2} folded in, for the state after each step).
 template <typename R, int LOGN, int LOGE, int LOGRM, class B, bool SURF = false>
 __device__ __forceinline__ void soft1d_run(const Inst1D& I, void* __restrict__ psi_base, int64_t nsteps,
                                            const double* __restrict__ ftab_base, int64_t ftab_stride,
                                            int* __restrict__ status, typename CT<R>::C* Ss,
                                            typename CT<R>::C* scan, const typename TwT<R>::T* Ws, int tid,
-                                           B bar, const typename CT<R>::C* __restrict__ sw = nullptr,
-                                           typename CT<R>::C* __restrict__ samples = nullptr)
+                                           B bar, const void* __restrict__ sw = nullptr,
+                                           double2* __restrict__ samples = nullptr)
 {
+    if constexpr (sizeof(R) == 8) {
+        soft1d_run_fx<LOGN, LOGE, LOGRM, B, SURF>(I, psi_base, nsteps, ftab_base, ftab_stride, status,
+                                                  reinterpret_cast<fx2*>(Ss), scan,
+                                                  reinterpret_cast<const int4*>(Ws), tid, bar, sw, samples);
+    } else {
+    static_assert(!SURF, "surface sampling is complex128");
     using K = Cfg1D<R, LOGN, LOGE, LOGRM>;
     using C = typename K::C;
     constexpr int N = K::N, T = K::T, E = K::E;
@@ -791,8 +748,8 @@ __device__ __forceinline__ void soft1d_run(const Inst1D& I, void* __restrict__ p
     C* fr = scan + 64;               // E + 52 complex: field phases (field_setup)
 
     C* __restrict__ g_psi = reinterpret_cast<C*>(psi_base) + I.off;
-    // the state: shared memory, or (GM) the instance's buffer itself
-    C* S = K::GM ? g_psi : Ss;
+    static_assert(!K::GM, "complex64 states fit in shared memory");
+    C* S = Ss;
     using TT = typename K::TT;
     const TT* __restrict__ TK = reinterpret_cast<const TT*>(I.TK);
     const TT* __restrict__ TKh = reinterpret_cast<const TT*>(I.TKh);
@@ -803,19 +760,10 @@ __device__ __forceinline__ void soft1d_run(const Inst1D& I, void* __restrict__ p
     const int nb = I.nb, blk0 = I.blk0;
     if (nsteps <= 0) return;
 
-    // load the state (GM: permute the buffer into the swizzled order in place;
-    // swz is an involution, so it is a product of disjoint swaps)
-    if constexpr (K::GM) {
-        for (int j = 0; j < E; ++j) {
-            const int n = tid + j * T, p = swz<C>(n);
-            if (n < p) { const C a = S[n]; S[n] = S[p]; S[p] = a; }
-        }
-    } else {
 #pragma unroll
-        for (int j = 0; j < E; ++j) {
-            const int n = tid + j * T;
-            S[swz<C>(n)] = g_psi[n];
-        }
+    for (int j = 0; j < E; ++j) {
+        const int n = tid + j * T;
+        S[swz<C>(n)] = g_psi[n];
     }
     bar.sync();
 
@@ -841,16 +789,7 @@ __device__ __forceinline__ void soft1d_run(const Inst1D& I, void* __restrict__ p
         //      and last pass of the call), inverse FFT, potential of the next step
         const bool more = step + 1 < nsteps;
         fwd_passes<R, LOGN, LOGE, LOGRM, 0, K::NPASS - 1>(S, Ws, tid, bar);
-        if constexpr (SURF) {
-            C acc[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) acc[r] = cmk<C>(0, 0);
-            kcenter<R, LOGN, LOGE, LOGRM, true>(S, (step >= 0 && more) ? TK : TKh, tid,
-                                                sw + (step >= 0 ? 4 * N : 0), acc);
-            surf_reduce<C, T>(acc, scan, tid, bar, samples + 4 * (step + 1));
-        } else {
-            kcenter<R, LOGN, LOGE, LOGRM>(S, (step >= 0 && more) ? TK : TKh, tid);
-        }
+        kcenter<R, LOGN, LOGE, LOGRM>(S, (step >= 0 && more) ? TK : TKh, tid);
         if (more && I.has_field) {
             al = alpha(step + 1);
             field_setup<R, LOGN, LOGE, LOGRM>(fr, al, I, tid);
@@ -861,23 +800,16 @@ __device__ __forceinline__ void soft1d_run(const Inst1D& I, void* __restrict__ p
         bar.sync();
     }
 
-    // store
-    if constexpr (K::GM) {
-        for (int j = 0; j < E; ++j) {
-            const int n = tid + j * T, p = swz<C>(n);
-            if (n < p) { const C a = S[n]; S[n] = S[p]; S[p] = a; }
-        }
-    } else {
 #pragma unroll
-        for (int j = 0; j < E; ++j) {
-            const int n = tid + j * T;
-            g_psi[n] = S[swz<C>(n)];
-        }
+    for (int j = 0; j < E; ++j) {
+        const int n = tid + j * T;
+        g_psi[n] = S[swz<C>(n)];
     }
     if (tid == 0 && status) {
         const C v = S[0];
         if (!(isfinite((double)v.x) && isfinite((double)v.y))) atomicOr(status, 1);
     }
+    }   // complex64
 }
 
 // One CTA per instance: blockIdx.x indexes insts.
@@ -887,7 +819,6 @@ soft1d_kernel(const Inst1D* __restrict__ insts, void* __restrict__ psi_base, int
               const double* __restrict__ ftab_base, int64_t ftab_stride, int* __restrict__ status)
 {
     using K = Cfg1D<R, LOGN, LOGE, LOGRM>;
-    using Q = Step1D<R, LOGN, LOGRM>;
     using C = typename K::C;
     static_assert(soft1d_smem<R, LOGN, LOGE, LOGRM>() <= 227 * 1024, "shared memory");
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -898,10 +829,10 @@ soft1d_kernel(const Inst1D* __restrict__ insts, void* __restrict__ psi_base, int
     const Inst1D I = insts[blockIdx.x];
     const TWT* __restrict__ W = reinterpret_cast<const TWT*>(I.W);
     if (nsteps <= 0) return;
-    copy16(Ws, W, Q::TWN, threadIdx.x, K::T);
+    copy16(Ws, W, TwCountT<TWT, LOGN, LOGRM>::value, threadIdx.x, K::T);
     // the run's first barrier (after its state load) also covers the twiddles
     soft1d_run<R, LOGN, LOGE, LOGRM>(I, psi_base, nsteps, ftab_base, ftab_stride, status, Ss,
-                                     reinterpret_cast<C*>(Ws + Q::TWN), Ws, (int)threadIdx.x, BarCTA());
+                                     reinterpret_cast<C*>(Ws + TwCountT<TWT, LOGN, LOGRM>::value), Ws, (int)threadIdx.x, BarCTA());
 }
 
 // One instance (blockIdx.x 0) with surface sampling: samples[s][r] for the
@@ -914,7 +845,6 @@ soft1d_surf_kernel(const Inst1D* __restrict__ insts, void* __restrict__ psi_base
                    const void* __restrict__ sw, void* __restrict__ samples)
 {
     using K = Cfg1D<R, LOGN, LOGE, LOGRM>;
-    using Q = Step1D<R, LOGN, LOGRM>;
     using C = typename K::C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using TWT = typename TwT<R>::T;
@@ -923,11 +853,10 @@ soft1d_surf_kernel(const Inst1D* __restrict__ insts, void* __restrict__ psi_base
     const Inst1D I = insts[0];
     const TWT* __restrict__ W = reinterpret_cast<const TWT*>(I.W);
     if (nsteps <= 0) return;
-    copy16(Ws, W, Q::TWN, threadIdx.x, K::T);
+    copy16(Ws, W, TwCountT<TWT, LOGN, LOGRM>::value, threadIdx.x, K::T);
     soft1d_run<R, LOGN, LOGE, LOGRM, BarCTA, true>(I, psi_base, nsteps, ftab_base, ftab_stride, status, Ss,
-                                                   reinterpret_cast<C*>(Ws + Q::TWN), Ws, (int)threadIdx.x,
-                                                   BarCTA(), reinterpret_cast<const C*>(sw),
-                                                   reinterpret_cast<C*>(samples));
+                                                   reinterpret_cast<C*>(Ws + TwCountT<TWT, LOGN, LOGRM>::value), Ws, (int)threadIdx.x,
+                                                   BarCTA(), sw, reinterpret_cast<double2*>(samples));
 }
 
 template <typename R, int LOGN, int LOGE, int LOGRM>

@@ -36,7 +36,6 @@ void soft1d_default_cfg(int prec, int logn, int* loge, int* logrm) {
     else e = logn >= 14 ? 5 : logn >= 12 ? 4 : 3;   // N = 16384: state in global memory, 512 threads
     *loge = e;
     *logrm = e > 4 ? 4 : e;
-    if (prec == SOFT_C128 && *logrm > 3) *logrm = 3;   // radix 16 in FP64 does not fit 128 registers
 }
 
 // every built (elements per thread, radix) variant of a size

@@ -15,7 +15,7 @@ constexpr int PERSIST_THREADS = 512;
 // (LOGN, LOGE, LOGRM) of the kernel's variants, [0] complex64, [1] complex128,
 // largest N first (the queue order)
 constexpr int PERSIST_CFG[2][4][3] = {{{14, 5, 4}, {13, 5, 4}, {12, 4, 4}, {11, 4, 4}},
-                                      {{14, 5, 3}, {13, 4, 3}, {12, 4, 3}, {11, 3, 3}}};
+                                      {{14, 5, 4}, {13, 4, 4}, {12, 4, 4}, {11, 3, 3}}};
 
 // variant index of a size (-1: not in the persistent kernel), its
 // (LOGE, LOGRM) and the instances per CTA

@@ -34,13 +34,13 @@ SurfLaunch find_surf(int logn, int loge, int logrm) {
 #define SURF_CASE(LN, LE, LRM) \
     if (logn == LN && loge == LE && logrm == LRM) return &launch_soft1d_surf_t<double, LN, LE, LRM>;
     SURF_CASE(8, 3, 3) SURF_CASE(9, 3, 3) SURF_CASE(10, 3, 3) SURF_CASE(11, 3, 3)
-    SURF_CASE(12, 4, 3) SURF_CASE(13, 4, 3)
+    SURF_CASE(12, 4, 4) SURF_CASE(13, 4, 4)
 #undef SURF_CASE
     return nullptr;
 }
 
 struct SurfTabs {
-    void* sw = nullptr;      // 8 rows x N: the kernel's spectral weights (two sets)
+    void* sw = nullptr;      // 8 rows x N: the kernel's spectral weights (two sets) as factors, 8 scales
     void* xw = nullptr;      // 4 rows x N: x-space weights of the same interpolant
     ~SurfTabs() { cudaFree(sw); cudaFree(xw); }
 };
@@ -92,7 +92,20 @@ int build_surf(soft_plan* P, SurfTabs* S) {
         }
     }
     int rc;
-    if ((rc = upload_c(&S->sw, sw, SOFT_C128))) return rc;
+    // rows as fixed-point factors (largest modulus 1) and their scales
+    std::vector<double> scale(8, 0.0);
+    for (int r = 0; r < 8; ++r) {
+        for (int q = 0; q < n; ++q) scale[r] = std::max(scale[r], std::abs(sw[(size_t)r * n + q]));
+        for (int q = 0; q < n; ++q) sw[(size_t)r * n + q] /= scale[r];
+        if ((logn - lrl) & 1) scale[r] *= std::sqrt(2.0);    // half bit of the passes before the centre
+    }
+    void* rows = nullptr;
+    if ((rc = upload_fx(&rows, sw))) { cudaFree(rows); return rc; }
+    rc = cuda_status(cudaMalloc(&S->sw, 16 * sw.size() + 64));
+    if (rc == SOFT_OK) rc = cuda_status(cudaMemcpy(S->sw, rows, 16 * sw.size(), cudaMemcpyDeviceToDevice));
+    if (rc == SOFT_OK) rc = cuda_status(cudaMemcpy((char*)S->sw + 16 * sw.size(), scale.data(), 64, cudaMemcpyHostToDevice));
+    cudaFree(rows);
+    if (rc) return rc;
     return upload_c(&S->xw, xw, SOFT_C128);
 }
 
