@@ -54,10 +54,8 @@ struct Tables1D {
     void* TVs = nullptr;
 };
 
-// Passes of stride up to this store every twiddle W^{M off}, the others a few
-// bases: the complex128 line passes of the 2D and 3D steps (soft1d.cuh,
-// TwFull) and the complex128 1D step (soft1d_fix.cuh, FxGeom).
-constexpr int TWFULL_MAXS = 256;
+// Fixed-point passes of stride up to this store every twiddle W^{M off}, the
+// others eight rows (soft1d_fix.cuh, FxGeom).
 constexpr int FXFULL_MAXS = 256;
 
 // Centre of the complex128 1D step (soft1d_fix.cuh).  The centre (last forward pass of r bits, k-space factor, first inverse

@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <thread>
 #include <tuple>
 
 #include "fix64_host.h"
@@ -118,14 +119,14 @@ int upload_fx(void** dst, const std::vector<cd>& v) {
     return upload(dst, buf.data(), buf.size() * sizeof(int32_t));
 }
 
-// e^{i ph} as factors, times sqrt(2) if s2 (soft1d_fix.cuh: passes of odd radix)
-static int upload_fx_phases(void** dst, const std::vector<double>& ph, bool s2) {
+int upload_fx_phases(void** dst, const std::vector<double>& ph, int half) {
     std::vector<int32_t> buf(4 * ph.size());
+    auto sc = [&](int64_t w) { return half == 0 ? w : half > 0 ? fx_sqrt2_host(w) : (fx_sqrt2_host(w) + 1) >> 1; };
     for (size_t i = 0; i < ph.size(); ++i) {
         int64_t c, s;
         fx_cis_host(fx_turns_host(ph[i]), &c, &s);
-        fx_halves_host(s2 ? fx_sqrt2_host(c) : c, &buf[4 * i]);
-        fx_halves_host(s2 ? fx_sqrt2_host(s) : s, &buf[4 * i + 2]);
+        fx_halves_host(sc(c), &buf[4 * i]);
+        fx_halves_host(sc(s), &buf[4 * i + 2]);
     }
     return upload(dst, buf.data(), buf.size() * sizeof(int32_t));
 }
@@ -168,7 +169,7 @@ static bool fxv_gen(const std::vector<cd>& lv) {
 // the block: thr threads of ch rows each.  gen: a multiplier above 1, a g
 // above 1.9 (its halves still fit, and the rows it scales are below 2^59.5)
 // or a growth of the sweeps above 2^10; the kernel then solves in FP64.
-static std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vector<cd>& mb,
+std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vector<cd>& mb,
                                             const std::vector<cd>& g, int nb, int thr, bool* gen) {
     const int ch = (nb + thr - 1) / thr, nw = thr / 32;
     const double tiny = 0x1p-70;
@@ -259,7 +260,64 @@ static std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std
     return buf;
 }
 
-static int upload_i32(void** dst, const std::vector<int32_t>& v) { return upload(dst, v.data(), v.size() * 4); }
+int upload_i32(void** dst, const std::vector<int32_t>& v) { return upload(dst, v.data(), v.size() * 4); }
+
+void host_parallel(int64_t n, const std::function<void(int64_t, int64_t)>& fn) {
+    const int64_t nt = std::max<int64_t>(1, std::min<int64_t>({(int64_t)std::thread::hardware_concurrency(), 32, n / 4096}));
+    std::vector<std::thread> pool;
+    int64_t done = 0;              // handed to threads; the rest runs here
+    try {
+        for (int64_t t = 0; t + 1 < nt; ++t) {
+            const int64_t b = n * t / nt, e = n * (t + 1) / nt;
+            pool.emplace_back([&fn, b, e] { fn(b, e); });
+            done = e;
+        }
+    } catch (...) {                // no thread could be started: no exception crosses the C ABI
+    }
+    if (done < n) fn(done, n);
+    for (auto& th : pool) th.join();
+}
+
+// FxMeta of soft2d_fix.cuh
+struct FxMetaHost { int p, gen; const void* d; };
+static int fx_potential_fill(FxPotential& P, const std::vector<cd>& lv) {
+    const int64_t n = (int64_t)lv.size();
+    double m = 0;
+    bool fin = true;
+    for (const cd& x : lv) {
+        m = std::max(m, x.real());
+        fin = fin && std::isfinite(x.real()) && std::isfinite(x.imag());
+    }
+    FxMetaHost h{0, P.cn_gen || !fin || std::exp(m) > 2.0, nullptr};
+    h.p = !h.gen && std::exp(m) > 1.01;
+    std::vector<int32_t> buf(4 * n);
+    host_parallel(n, [&](int64_t b, int64_t e) {
+        for (int64_t i = b; i < e; ++i) {
+            if (h.gen) {
+                const cd v = std::exp(lv[i]);
+                std::memcpy(&buf[4 * i], &v, 16);
+                continue;
+            }
+            int64_t c, s;
+            fx_cis_host(fx_turns_host(lv[i].imag()), &c, &s);
+            const int64_t mod = std::llrint(std::exp(lv[i].real()) * (h.p ? 0x1p60 : 0x1p61));
+            fx_halves_host((int64_t)(((__int128)c * mod + (1LL << 60)) >> 61), &buf[4 * i]);
+            fx_halves_host((int64_t)(((__int128)s * mod + (1LL << 60)) >> 61), &buf[4 * i + 2]);
+        }
+    });
+    // gen plans read the same buffer as double2
+    if (h.gen) h.d = P.tab;
+    int rc = cuda_status(cudaMemcpy(P.tab, buf.data(), 16 * (size_t)n, cudaMemcpyHostToDevice));
+    return rc ? rc : cuda_status(cudaMemcpy(P.meta, &h, sizeof(h), cudaMemcpyHostToDevice));
+}
+int FxPotential::build(const std::vector<cd>& lv) {
+    int rc = cuda_status(cudaMalloc(&tab, 16 * lv.size()));
+    if (rc) { tab = nullptr; return rc; }
+    if ((rc = cuda_status(cudaMalloc(&meta, sizeof(FxMetaHost))))) { meta = nullptr; return rc; }
+    return fx_potential_fill(*this, lv);
+}
+int FxPotential::refill(const std::vector<cd>& lv) { return fx_potential_fill(*this, lv); }
+FxPotential::~FxPotential() { cudaFree(tab); cudaFree(meta); }
 
 // the upload_* conversions into a temporary device buffer, then one copy
 // into dst

@@ -23,12 +23,13 @@ int Plan2D::set_potential(const double* Uin) {
     int rc = cuda_status(cudaDeviceSynchronize());      // no step may still read the tables
     if (rc) return rc;
     const size_t n = (size_t)nx * ny;
-    std::vector<cd> tvh(n);
+    std::vector<cd> tvh(n);        // e^{-iU tau/2} (complex128: its logarithm)
     for (size_t i = 0; i < n; ++i) {
         U[i] = cd(Uin[2 * i], Uin[2 * i + 1]) + Uabs[i];
-        tvh[i] = std::exp(cd(0.0, -0.5 * tau) * U[i]);
+        tvh[i] = cd(0.0, -0.5 * tau) * U[i];
+        if (prec == SOFT_C64) tvh[i] = std::exp(tvh[i]);
     }
-    if ((rc = refill_vtab(TVh, tvh, prec))) return rc;
+    if ((rc = prec == SOFT_C64 ? refill_vtab(TVh, tvh, prec) : fxv.refill(tvh))) return rc;
     return pcg_refill_potential(this);
 }
 
@@ -46,7 +47,7 @@ int Plan2D::row(int mode, void* psi, const void* tkx, cudaStream_t st) {
 }
 int Plan2D::col(int mode, void* psi, const void* tky, cudaStream_t st) {
     ++launches;
-    const LineGeo lg{geo.Wy, geo.nx, 0, geo.cny, geo.TVh, geo.nby, geo.blk0y, 0, 1, 0, 0};
+    const LineGeo lg{geo.Wy, geo.nx, 0, geo.cny, geo.TVh, geo.nby, geo.blk0y, 0, 1, 0, 0, geo.vmeta};
     if (prec == SOFT_C64) return soft2d_col_c64(ly, ley, lry, mode, lg, 1, psi, tky, st);
     return soft2d_col_c128(ly, ley, lry, mode, lg, 1, psi, tky, st);
 }
@@ -100,7 +101,7 @@ int create_2d(const soft_grid* grid, const double* box, double R0, double theta,
     const int capy = o.prec == SOFT_C64 ? soft2d_col_strip_capacity_c64(ly, Q->ley, Q->lry)
                                         : soft2d_col_strip_capacity_c128(ly, Q->ley, Q->lry);
     if (nby > capy) return SOFT_ERR_UNSUPPORTED;
-    // potential at (z(x), z(y)) and e^{-iU tau/2}
+    // potential at (z(x), z(y)) and e^{-iU tau/2} (complex128: its logarithm)
     Q->U.resize((size_t)nx * ny);
     Q->Uabs.resize((size_t)nx * ny);
     std::vector<cd> tvh((size_t)nx * ny);
@@ -111,22 +112,27 @@ int create_2d(const soft_grid* grid, const double* box, double R0, double theta,
             const cd u = soft_coulomb(z, 2, o.soft_a2, o.charge) + ua;
             Q->Uabs[yy * nx + xx] = ua;
             Q->U[yy * nx + xx] = u;
-            tvh[yy * nx + xx] = std::exp(cd(0.0, -0.5 * dt) * u);
+            tvh[yy * nx + xx] = cd(0.0, -0.5 * dt) * u;
+            if (o.prec == SOFT_C64) tvh[yy * nx + xx] = std::exp(tvh[yy * nx + xx]);
         }
-    // kinetic factors per axis, 1/n folded in, read by the fused center of
-    // each line FFT (butterflies of R consecutive positions b*R + m of the
-    // digit-reversed spectrum, stored at m*(n/R) + b)
-    auto ktab = [&](const Axis1D& A, int logn, int logrm, double frac) {
+    // kinetic factors per axis, read by the fused center of each line FFT
+    // (butterflies of R consecutive positions b*R + m of the digit-reversed
+    // spectrum, stored at m*(n/R) + b); complex64: 1/n folded in; complex128:
+    // the passes' half bits (soft2d_fix.cuh)
+    const int pr = o.prec;
+    auto ktab = [&](void** dst, const Axis1D& A, int logn, int logrm, double frac) {
         const std::vector<int> perm = dif_output_order(logn, logrm);
         const int lrl = (logn % logrm) ? logn % logrm : logrm;
         const int Rl = 1 << lrl, nbf = A.n >> lrl;
-        std::vector<cd> t(A.n);
+        std::vector<double> ph(A.n);
         for (int p = 0; p < A.n; ++p) {
             const double k = A.k[perm[p]];
-            const int q = (p % Rl) * nbf + p / Rl;
-            t[q] = std::polar(1.0 / A.n, -0.5 * k * k * dt * frac);
+            ph[(p % Rl) * nbf + p / Rl] = -0.5 * k * k * dt * frac;
         }
-        return t;
+        if (pr == SOFT_C128) return upload_fx_phases(dst, ph, (int)fx_center(lrl, logrm).s2 - (logrm & 1));
+        std::vector<cd> t(A.n);
+        for (int q = 0; q < A.n; ++q) t[q] = std::polar(1.0 / A.n, ph[q]);
+        return upload_tab(dst, t, pr);
     };
     std::vector<cd> mfx, mbx, gx, mfy, mby, gy, cnx, cny;
     double err;
@@ -138,24 +144,31 @@ int create_2d(const soft_grid* grid, const double* box, double R0, double theta,
         if ((rc = strip_factor(Q->ay, by0, nby, mfy, mby, gy, &err))) return rc;
         cny = mfy; cny.insert(cny.end(), mby.begin(), mby.end()); cny.insert(cny.end(), gy.begin(), gy.end());
     }
-    const int pr = o.prec;
-    // pass twiddles: the four bases per pass (complex64); every W^{M off} of
-    // the small-stride passes (complex128)
+    // pass twiddles: the four bases per pass (complex64), fixed-point factors (complex128)
     auto twid = [&](void** d, int logn, int logrm) {
-        return upload_tw(d, pr == SOFT_C128 ? pass_twiddles_full(logn, logrm, TWFULL_MAXS)
-                                            : pass_twiddles(logn, logrm), pr);
+        return pr == SOFT_C128 ? upload_i32(d, pass_twiddles_fx(logn, logrm, FXFULL_MAXS))
+                               : upload_tw(d, pass_twiddles(logn, logrm), pr);
     };
     if ((rc = twid(&Q->Wx, lx, Q->lrx))) return rc;
     if ((rc = twid(&Q->Wy, ly, Q->lry))) return rc;
-    if ((rc = upload_tab(&Q->TKx, ktab(Q->ax, lx, Q->lrx, 1.0), pr))) return rc;
-    if ((rc = upload_tab(&Q->TKhx, ktab(Q->ax, lx, Q->lrx, 0.5), pr))) return rc;
-    if ((rc = upload_tab(&Q->TKy, ktab(Q->ay, ly, Q->lry, 1.0), pr))) return rc;
-    if ((rc = upload_tab(&Q->TKhy, ktab(Q->ay, ly, Q->lry, 0.5), pr))) return rc;
-    if ((rc = upload_vtab(&Q->TVh, tvh, pr))) return rc;
-    if ((rc = upload_c(&Q->cnx, cnx, pr))) return rc;
-    if ((rc = upload_c(&Q->cny, cny, pr))) return rc;
+    if ((rc = ktab(&Q->TKx, Q->ax, lx, Q->lrx, 1.0))) return rc;
+    if ((rc = ktab(&Q->TKhx, Q->ax, lx, Q->lrx, 0.5))) return rc;
+    if ((rc = ktab(&Q->TKy, Q->ay, ly, Q->lry, 1.0))) return rc;
+    if ((rc = ktab(&Q->TKhy, Q->ay, ly, Q->lry, 0.5))) return rc;
+    if (pr == SOFT_C128) {
+        bool gx_ = false, gy_ = false;
+        if (nbx > 0 && (rc = upload_i32(&Q->cnx, strip_tables_fx(mfx, mbx, gx, nbx, thr, &gx_)))) return rc;
+        if (nby > 0 && (rc = upload_i32(&Q->cny, strip_tables_fx(mfy, mby, gy, nby, (int)(ny >> Q->ley), &gy_)))) return rc;
+        Q->fxv.cn_gen = gx_ || gy_;
+        if ((rc = Q->fxv.build(tvh))) return rc;
+    } else {
+        if ((rc = upload_vtab(&Q->TVh, tvh, pr))) return rc;
+        if ((rc = upload_c(&Q->cnx, cnx, pr))) return rc;
+        if ((rc = upload_c(&Q->cny, cny, pr))) return rc;
+    }
     Geo2D& g = Q->geo;
-    g.Wx = Q->Wx; g.Wy = Q->Wy; g.TVh = Q->TVh; g.cnx = Q->cnx; g.cny = Q->cny;
+    g.Wx = Q->Wx; g.Wy = Q->Wy; g.TVh = pr == SOFT_C128 ? Q->fxv.tab : Q->TVh; g.cnx = Q->cnx; g.cny = Q->cny;
+    g.vmeta = Q->fxv.meta;
     g.nx = (int)nx; g.ny = (int)ny;
     g.nbx = nbx; g.blk0x = bx0; g.nby = nby; g.blk0y = by0;
     g.v2 = 1; g.ny1 = (int)ny; g.nz1 = 1; g.nbz1 = 0; g.blk0z1 = 0;

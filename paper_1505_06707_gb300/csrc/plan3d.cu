@@ -40,7 +40,7 @@ Plan3D::~Plan3D() {
     if (graph_exec) cudaGraphExecDestroy(graph_exec);
 }
 
-// e^{-iU tau/2} from U (host [nz][ny][nx]) plus the axes' absorber terms;
+// e^{-iU tau/2} (complex128: its logarithm) from U (host [nz][ny][nx]) plus the axes' absorber terms;
 // z planes are split over host threads (512^3 points take seconds alone)
 static std::vector<cd> half_factors(const Plan3D& Q, const double* Uin) {
     const int nx = Q.n[0], ny = Q.n[1], nz = Q.n[2];
@@ -58,7 +58,8 @@ static std::vector<cd> half_factors(const Plan3D& Q, const double* Uin) {
                         u = soft_coulomb(zz, 3, Q.a2, Q.charge);
                     }
                     u += Q.ua[0][x] + Q.ua[1][y] + Q.ua[2][z];
-                    tvh[i] = std::exp(cd(0.0, -0.5 * Q.tau) * u);
+                    tvh[i] = cd(0.0, -0.5 * Q.tau) * u;
+                    if (Q.prec == SOFT_C64) tvh[i] = std::exp(tvh[i]);
                 }
     };
     const int nt = std::max(1, std::min({(int)std::thread::hardware_concurrency(), 32, nz}));
@@ -80,7 +81,8 @@ static std::vector<cd> half_factors(const Plan3D& Q, const double* Uin) {
 int Plan3D::set_potential(const double* Uin) {
     int rc = cuda_status(cudaDeviceSynchronize());      // no step may still read the table
     if (rc) return rc;
-    return refill_vtab(TVh, half_factors(*this, Uin), prec);
+    const std::vector<cd> v = half_factors(*this, Uin);
+    return prec == SOFT_C64 ? refill_vtab(TVh, v, prec) : fxv.refill(v);
 }
 
 int Plan3D::row(int mode, void* psi, const void* tkx, cudaStream_t st) {
@@ -97,8 +99,8 @@ int Plan3D::line(int d, int mode, void* psi, const void* tk, cudaStream_t st) {
     const int64_t nx = n[0], ny = n[1];
     // z lines (c = y nx + x): V/2 off the z-strip block only on lines with y
     // in the y-strip block (the row pass applied it on the others)
-    const LineGeo lg{W[d], d == 1 ? nx : nx * ny, d == 1 ? nx * ny : 0, cn[d], TVh, nb[d], blk0[d],
-                     d == 2 ? nx : 0, n[1], nb[1], blk0[1]};
+    const LineGeo lg{W[d], d == 1 ? nx : nx * ny, d == 1 ? nx * ny : 0, cn[d], geo.TVh, nb[d], blk0[d],
+                     d == 2 ? nx : 0, n[1], nb[1], blk0[1], geo.vmeta};
     const int planes = d == 1 ? n[2] : 1;
     if (prec == SOFT_C64) return soft2d_col_c64(l[d], le[d], lr[d], mode, lg, planes, psi, tk, st);
     return soft2d_col_c128(l[d], le[d], lr[d], mode, lg, planes, psi, tk, st);
@@ -176,42 +178,56 @@ int create_3d(const soft_grid* grid, const double* box, double R0, double theta,
     if ((Q->nb[0] + thr - 1) / thr > (1 << Q->le[0]) / 4 + 2) return SOFT_ERR_UNSUPPORTED;
     if ((o.prec == SOFT_C64 ? 8 : 16) * (size_t)Q->nb[1] * 35 > 227 * 1024) return SOFT_ERR_UNSUPPORTED;
     if (Q->nb[2] > Q->col_capacity(2)) return SOFT_ERR_UNSUPPORTED;
-    // kinetic factors per axis, 1/n folded in, in the transposed order of
-    // the fused center of each line FFT
-    auto ktab = [&](int d, double frac) {
+    // kinetic factors per axis in the transposed order of the fused center of
+    // each line FFT (complex64: 1/n folded in; complex128: the passes' half
+    // bits, soft2d_fix.cuh)
+    const int pr = o.prec;
+    auto ktab = [&](void** dst, int d, double frac) {
         const Axis1D& A = Q->ax[d];
         const int logn = Q->l[d], logrm = Q->lr[d];
         const std::vector<int> perm = dif_output_order(logn, logrm);
         const int lrl = (logn % logrm) ? logn % logrm : logrm;
         const int Rl = 1 << lrl, nbf = A.n >> lrl;
-        std::vector<cd> t(A.n);
+        std::vector<double> ph(A.n);
         for (int p = 0; p < A.n; ++p) {
             const double k = A.k[perm[p]];
-            const int q = (p % Rl) * nbf + p / Rl;
-            t[q] = std::polar(1.0 / A.n, -0.5 * k * k * dt * frac);
+            ph[(p % Rl) * nbf + p / Rl] = -0.5 * k * k * dt * frac;
         }
-        return t;
+        if (pr == SOFT_C128) return upload_fx_phases(dst, ph, (int)fx_center(lrl, logrm).s2 - (logrm & 1));
+        std::vector<cd> t(A.n);
+        for (int q = 0; q < A.n; ++q) t[q] = std::polar(1.0 / A.n, ph[q]);
+        return upload_tab(dst, t, pr);
     };
-    const int pr = o.prec;
     for (int d = 0; d < 3; ++d) {
-        if ((rc = upload_tw(&Q->W[d], pr == SOFT_C128 ? pass_twiddles_full(Q->l[d], Q->lr[d], TWFULL_MAXS)
-                                                     : pass_twiddles(Q->l[d], Q->lr[d]), pr)))
-            return rc;
-        if ((rc = upload_tab(&Q->TK[d], ktab(d, 1.0), pr))) return rc;
-        if ((rc = upload_tab(&Q->TKh[d], ktab(d, 0.5), pr))) return rc;
+        rc = pr == SOFT_C128 ? upload_i32(&Q->W[d], pass_twiddles_fx(Q->l[d], Q->lr[d], FXFULL_MAXS))
+                             : upload_tw(&Q->W[d], pass_twiddles(Q->l[d], Q->lr[d]), pr);
+        if (rc) return rc;
+        if ((rc = ktab(&Q->TK[d], d, 1.0))) return rc;
+        if ((rc = ktab(&Q->TKh[d], d, 0.5))) return rc;
         if (Q->nb[d] > 0) {
             std::vector<cd> mf, mb, g;
             double err;
             if ((rc = strip_factor(Q->ax[d], Q->blk0[d], Q->nb[d], mf, mb, g, &err))) return rc;
+            if (pr == SOFT_C128 && d != 1) {       // (the y-strip pass is cn_lines_kernel)
+                bool gen = false;
+                rc = upload_i32(&Q->cn[d], strip_tables_fx(mf, mb, g, Q->nb[d], Q->n[d] >> Q->le[d], &gen));
+                if (rc) return rc;
+                Q->fxv.cn_gen = Q->fxv.cn_gen || gen;
+                continue;
+            }
             mf.insert(mf.end(), mb.begin(), mb.end());
             mf.insert(mf.end(), g.begin(), g.end());
             if ((rc = upload_c(&Q->cn[d], mf, pr))) return rc;
         }
     }
-    if ((rc = upload_vtab(&Q->TVh, half_factors(*Q, nullptr), pr))) return rc;
+    {
+        const std::vector<cd> tvh = half_factors(*Q, nullptr);
+        if ((rc = pr == SOFT_C128 ? Q->fxv.build(tvh) : upload_vtab(&Q->TVh, tvh, pr))) return rc;
+    }
     Geo2D& g = Q->geo;
     std::memset(&g, 0, sizeof(g));
-    g.Wx = Q->W[0]; g.TVh = Q->TVh; g.cnx = Q->cn[0];
+    g.Wx = Q->W[0]; g.TVh = pr == SOFT_C128 ? Q->fxv.tab : Q->TVh; g.cnx = Q->cn[0];
+    g.vmeta = Q->fxv.meta;
     g.nx = Q->n[0]; g.ny = Q->n[1] * Q->n[2];
     g.nbx = Q->nb[0]; g.blk0x = Q->blk0[0];
     g.nby = Q->nb[1]; g.blk0y = Q->blk0[1];

@@ -1,5 +1,6 @@
 // The opaque plan object behind the C ABI.
 #pragma once
+#include <functional>
 #include <memory>
 #include <vector>
 
@@ -30,8 +31,24 @@ int upload_tw(void** dst, const std::vector<cd>& v, int prec);
 int upload_tw_comp(void** dst, const std::vector<cd>& v, int prec);
 // rewrite an existing device buffer in place (same size and format as the
 // matching upload_*), so that pointers held by kernels and graphs stay valid
-// fixed-point factors |v| <= 1 (fix64.cuh)
+// fixed-point factors (fix64.cuh): values, and phases e^{i ph} times 2^(half/2)
 int upload_fx(void** dst, const std::vector<cd>& v);
+int upload_fx_phases(void** dst, const std::vector<double>& ph, int half);
+int upload_i32(void** dst, const std::vector<int32_t>& v);
+std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vector<cd>& mb, const std::vector<cd>& g,
+                                     int nb, int thr, bool* gen);
+// fn(begin, end) over 0 .. n - 1 on host threads (the calling one if none can start)
+void host_parallel(int64_t n, const std::function<void(int64_t, int64_t)>& fn);
+// Potential factors of a complex128 2D or 3D plan: factors e^{lv} 2^-p
+// (fix64.cuh) or, for gen plans, double2 in the same buffer, and the device
+// FxMeta record (soft2d_fix.cuh).  build allocates; refill rewrites in place.
+struct FxPotential {
+    void *tab = nullptr, *meta = nullptr;
+    bool cn_gen = false;           // a strip solve of the plan is not fit for fixed point
+    int build(const std::vector<cd>& lv);
+    int refill(const std::vector<cd>& lv);
+    ~FxPotential();
+};
 int refill_c(void* dst, const std::vector<cd>& v, int prec);
 int refill_vtab(void* dst, const std::vector<cd>& v, int prec);
 struct Plan2D;
@@ -76,6 +93,7 @@ struct Plan2D {
     std::vector<cd> Uabs;          // its comparison-absorber part, [ny][nx]
     void *Wx = nullptr, *Wy = nullptr, *TKx = nullptr, *TKhx = nullptr, *TKy = nullptr,
          *TKhy = nullptr, *TVh = nullptr, *cnx = nullptr, *cny = nullptr;
+    FxPotential fxv;               // complex128 (instead of TVh)
     Geo2D geo{};
     int64_t launches = 0, graph_launches = 0;
     cudaGraphExec_t graph_exec = nullptr;
@@ -102,6 +120,7 @@ struct Plan3D {
     Axis1D ax[3];
     std::vector<cd> ua[3];         // comparison-absorber potential of each axis
     void *W[3] = {}, *TK[3] = {}, *TKh[3] = {}, *TVh = nullptr, *cn[3] = {};
+    FxPotential fxv;               // complex128 (instead of TVh)
     Geo2D geo{};
     int64_t launches = 0, graph_launches = 0;
     cudaGraphExec_t graph_exec = nullptr;

@@ -65,12 +65,8 @@ __device__ __forceinline__ float2 tmulc(float2 x, float4 t) {
 // state drifts linearly in time.  With compensated factors the modulus is
 // exact to ~2^-48 and only the data's own roundings remain.
 // Complex128 plans of the 1D step store fixed-point factors (TwFix,
-// soft1d_fix.cuh).  The complex128 line passes of the 2D and 3D steps store,
-// for passes with a stride of at most TWFULL_MAXS, every twiddle W^{M off}
-// (M = 1 .. R-1) instead of the four bases: the products of bases cost 16 of
-// the ~100 FP64 instructions of a radix-8 butterfly, and those kernels are
-// bound by the FP64 pipe.
-template <typename C> struct TwFull { C v; };
+// soft1d_fix.cuh), and so do the complex128 line passes of the 2D and 3D steps
+// (soft2d_fix.cuh); the stationary solvers' FP64 passes use the bases.
 struct TwFix { int4 v; };
 constexpr int FX_FR = 68;       // field factors of the fixed-point step behind its 2 E per-row ones
 
@@ -129,29 +125,11 @@ __device__ __forceinline__ C tw_pow(const C* b) {
 // y * W^{M off} (fwd) and y * conj(W^{M off}) (inv) from the bases b[k] =
 // W^{2^k off}: plain bases (TW = C) through one product twiddle, compensated
 // FP32 bases (TW = float4) by one compensated multiply per set bit of M
-template <typename C, typename TW, int M, bool FULL = false> struct TwMul {
+template <typename C, typename TW, int M> struct TwMul {
     __device__ __forceinline__ static C fwd(C y, const C* b) { return cmul(y, tw_pow<C, M>(b)); }
     __device__ __forceinline__ static C inv(C y, const C* b) { return cmulc(y, tw_pow<C, M>(b)); }
 };
-// full tables: full passes hold b[M - 1] = W^{M off}; the other passes hold
-// W^{M off} for M = 1 .. 4, and W^{M off} = W^{4 off} W^{(M-4) off} above
-// (radix 8: one product instead of up to two)
-template <typename C, int M> __device__ __forceinline__ C tw_full(const TwFull<C>* b) {
-    static_assert(M >= 1 && M < 16, "radix <= 16");
-    if constexpr (M <= 4) return b[M - 1].v;
-    else return cmul(b[3].v, tw_full<C, M - 4>(b));
-}
-template <typename C, int M, bool FULL> struct TwMul<C, TwFull<C>, M, FULL> {
-    __device__ __forceinline__ static C fwd(C y, const TwFull<C>* b) {
-        if constexpr (FULL) return cmul(y, b[M - 1].v);
-        else return cmul(y, tw_full<C, M>(b));
-    }
-    __device__ __forceinline__ static C inv(C y, const TwFull<C>* b) {
-        if constexpr (FULL) return cmulc(y, b[M - 1].v);
-        else return cmulc(y, tw_full<C, M>(b));
-    }
-};
-template <int M, bool FULL> struct TwMul<float2, float4, M, FULL> {
+template <int M> struct TwMul<float2, float4, M> {
     __device__ __forceinline__ static float2 fwd(float2 y, const float4* b) {
         if constexpr ((M & 1) != 0) y = tmul(y, b[0]);
         if constexpr ((M & 2) != 0) y = tmul(y, b[1]);
@@ -170,23 +148,23 @@ template <int M, bool FULL> struct TwMul<float2, float4, M, FULL> {
 
 // The element M of a butterfly lives at base + M s; the callers pass
 // sb = swz(base) and the offset of element M is the constant swz(M s).
-template <typename C, typename TW, int RR, int SS, int M, bool FULL = false>
+template <typename C, typename TW, int RR, int SS, int M>
 struct StoreFwd {   // y_M = v[bitrev(M)] * W^{M off}, stored at base + M s
     __device__ __forceinline__ static void run(C* S, const C* v, const TW* b, int sb, bool tw) {
         constexpr int LOGR = (RR == 16) ? 4 : (RR == 8) ? 3 : (RR == 4) ? 2 : (RR == 2) ? 1 : 0;
         C y = v[bitrev_c(M, LOGR)];
-        if constexpr (M > 0) { if (tw) y = TwMul<C, TW, M, FULL>::fwd(y, b); }
+        if constexpr (M > 0) { if (tw) y = TwMul<C, TW, M>::fwd(y, b); }
         S[sb ^ swz<C>(M * SS)] = y;
-        if constexpr (M + 1 < RR) StoreFwd<C, TW, RR, SS, M + 1, FULL>::run(S, v, b, sb, tw);
+        if constexpr (M + 1 < RR) StoreFwd<C, TW, RR, SS, M + 1>::run(S, v, b, sb, tw);
     }
 };
-template <typename C, typename TW, int RR, int SS, int M, bool FULL = false>
+template <typename C, typename TW, int RR, int SS, int M>
 struct LoadInv {    // v_M = S[base + M s] * conj(W^{M off})
     __device__ __forceinline__ static void run(const C* S, C* v, const TW* b, int sb, bool tw) {
         C y = S[sb ^ swz<C>(M * SS)];
-        if constexpr (M > 0) { if (tw) y = TwMul<C, TW, M, FULL>::inv(y, b); }
+        if constexpr (M > 0) { if (tw) y = TwMul<C, TW, M>::inv(y, b); }
         v[M] = y;
-        if constexpr (M + 1 < RR) LoadInv<C, TW, RR, SS, M + 1, FULL>::run(S, v, b, sb, tw);
+        if constexpr (M + 1 < RR) LoadInv<C, TW, RR, SS, M + 1>::run(S, v, b, sb, tw);
     }
 };
 template <typename C, int RR, int SS, int M>
@@ -209,33 +187,6 @@ __device__ __forceinline__ void load_tw(C* b, const C* __restrict__ t) {
     }
 }
 
-// Twiddle table layout of a pass: offsets and whether the pass stores every
-// W^{M off} (FULL) or the four bases, for twiddle type TW.
-template <int LOGN, int LOGRM, int P>
-struct TwGeomFull {
-    using G = PassGeom<LOGN, LOGRM, P>;
-    static constexpr bool FULL = G::S > 1 && G::S <= TWFULL_MAXS;
-    static constexpr int ROWS = FULL ? (1 << G::LOGR) - 1 : 4;
-    static constexpr int TOFF = TwGeomFull<LOGN, LOGRM, P - 1>::TOFF +
-                                TwGeomFull<LOGN, LOGRM, P - 1>::ROWS * PassGeom<LOGN, LOGRM, P - 1>::S;
-};
-template <int LOGN, int LOGRM>
-struct TwGeomFull<LOGN, LOGRM, -1> { static constexpr bool FULL = false; static constexpr int ROWS = 0, TOFF = 0; };
-
-template <typename TW> struct TwLay {      // the four bases W^{2^k off} on every pass
-    template <int LOGN, int LOGRM, int P> static constexpr bool full() { return false; }
-    template <int LOGN, int LOGRM, int P> static constexpr int toff() { return PassGeom<LOGN, LOGRM, P>::TOFF; }
-    template <int LOGN, int LOGRM, int P> static constexpr int rows() { return PassGeom<LOGN, LOGRM, P>::LOGR; }
-};
-template <typename C> struct TwLay<TwFull<C>> {   // every W^{M off}, or M = 1 .. 4 (tw_full)
-    template <int LOGN, int LOGRM, int P> static constexpr bool full() { return TwGeomFull<LOGN, LOGRM, P>::FULL; }
-    template <int LOGN, int LOGRM, int P> static constexpr int toff() { return TwGeomFull<LOGN, LOGRM, P>::TOFF; }
-    template <int LOGN, int LOGRM, int P> static constexpr int rows() {
-        constexpr int R = 1 << PassGeom<LOGN, LOGRM, P>::LOGR;
-        return TwGeomFull<LOGN, LOGRM, P>::FULL ? R - 1 : (R - 1 < 4 ? R - 1 : 4);
-    }
-};
-
 // number of twiddle entries of all passes
 template <int LOGN, int LOGRM>
 struct TwCount {
@@ -245,13 +196,6 @@ struct TwCount {
 // the same for the table layout of twiddle type TW
 template <typename TW, int LOGN, int LOGRM>
 struct TwCountT { static constexpr int value = TwCount<LOGN, LOGRM>::value; };
-template <typename C, int LOGN, int LOGRM>
-struct TwCountT<TwFull<C>, LOGN, LOGRM> {
-    static constexpr int NP = LOGN / LOGRM + ((LOGN % LOGRM) ? 1 : 0);
-    static constexpr int value = TwGeomFull<LOGN, LOGRM, NP - 1>::TOFF +
-                                 TwGeomFull<LOGN, LOGRM, NP - 1>::ROWS * PassGeom<LOGN, LOGRM, NP - 1>::S;
-};
-
 template <typename R, int LOGN, int LOGRM>
 struct Step1D {
     static constexpr int NPASS = LOGN / LOGRM + ((LOGN % LOGRM) ? 1 : 0);
@@ -272,7 +216,6 @@ __device__ __forceinline__ void fwd_pass(typename CT<R>::C* S, const TW* __restr
     constexpr int RR = 1 << G::LOGR;
     constexpr int L = 1 << G::LOGL;
     constexpr int s = G::S;
-    constexpr int NB = G::LOGR;               // twiddle bases needed: 2^0 .. 2^(LOGR-1)
 #pragma unroll 1
     for (int u = 0; u < K::E / RR; ++u) {      // one butterfly live at a time
         const int b = tid + u * K::T;
@@ -282,12 +225,10 @@ __device__ __forceinline__ void fwd_pass(typename CT<R>::C* S, const TW* __restr
 #pragma unroll
         for (int j = 0; j < RR; ++j) v[j] = S[sb ^ swz<C>(j * s)];
         dft_reg<C, RR, -1>(v);
-        constexpr bool FULL = TwLay<TW>::template full<LOGN, LOGRM, P>();
-        TW tb[FULL ? RR - 1 : 4];
+        TW tb[4];
         if constexpr (s > 1)
-            load_tw<TW, TwLay<TW>::template rows<LOGN, LOGRM, P>(), s, SH>(
-                tb, W + TwLay<TW>::template toff<LOGN, LOGRM, P>() + off);
-        StoreFwd<C, TW, RR, s, 0, FULL>::run(S, v, tb, sb, s > 1);
+            load_tw<TW, G::LOGR, s, SH>(tb, W + G::TOFF + off);
+        StoreFwd<C, TW, RR, s, 0>::run(S, v, tb, sb, s > 1);
     }
 }
 
@@ -300,19 +241,16 @@ __device__ __forceinline__ void inv_pass(typename CT<R>::C* S, const TW* __restr
     constexpr int RR = 1 << G::LOGR;
     constexpr int L = 1 << G::LOGL;
     constexpr int s = G::S;
-    constexpr int NB = G::LOGR;
 #pragma unroll 1
     for (int u = 0; u < K::E / RR; ++u) {      // one butterfly live at a time
         const int b = tid + u * K::T;
         const int blk = b / s, off = b & (s - 1);
         const int sb = swz<C>(blk * L + off);
         C v[RR];
-        constexpr bool FULL = TwLay<TW>::template full<LOGN, LOGRM, P>();
-        TW tb[FULL ? RR - 1 : 4];
+        TW tb[4];
         if constexpr (s > 1)
-            load_tw<TW, TwLay<TW>::template rows<LOGN, LOGRM, P>(), s, SH>(
-                tb, W + TwLay<TW>::template toff<LOGN, LOGRM, P>() + off);
-        LoadInv<C, TW, RR, s, 0, FULL>::run(S, v, tb, sb, s > 1);
+            load_tw<TW, G::LOGR, s, SH>(tb, W + G::TOFF + off);
+        LoadInv<C, TW, RR, s, 0>::run(S, v, tb, sb, s > 1);
         dft_reg<C, RR, +1>(v);
         StoreNat<C, RR, s, 0>::run(S, v, sb);
     }
@@ -634,7 +572,6 @@ __device__ __forceinline__ void inv_pass0_v(typename CT<R>::C* S, const TW* __re
     constexpr int N = K::N;
     constexpr int LOGR = G::LOGR, RR = 1 << LOGR;
     constexpr int s = G::S;                    // = N / RR
-    constexpr int NB = G::LOGR;
     const int nb = I.nb, blk0 = I.blk0, iL = I.iL, iR = I.iR;
     const bool fld = V && I.has_field;
     C ft; ft.x = 1; ft.y = 0;
@@ -650,12 +587,10 @@ __device__ __forceinline__ void inv_pass0_v(typename CT<R>::C* S, const TW* __re
         const int off = tid + u * K::T;        // L = N: a single block
         const int sb = swz<C>(off);
         C v[RR];
-        constexpr bool FULL = TwLay<TW>::template full<LOGN, LOGRM, 0>();
-        TW tb[FULL ? RR - 1 : 4];
+        TW tb[4];
         if constexpr (s > 1)
-            load_tw<TW, TwLay<TW>::template rows<LOGN, LOGRM, 0>(), s, true>(
-                tb, Ws + TwLay<TW>::template toff<LOGN, LOGRM, 0>() + off);
-        LoadInv<C, TW, RR, s, 0, FULL>::run(S, v, tb, sb, s > 1);
+            load_tw<TW, G::LOGR, s, true>(tb, Ws + G::TOFF + off);
+        LoadInv<C, TW, RR, s, 0>::run(S, v, tb, sb, s > 1);
         dft_reg<C, RR, +1>(v);
         if (!V) {
             StoreNat<C, RR, s, 0>::run(S, v, sb);

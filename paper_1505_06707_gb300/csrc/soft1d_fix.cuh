@@ -334,14 +334,14 @@ __device__ __noinline__ void potential_gen(fx2* S, const double2* __restrict__ t
 }
 // the thread's own rows times 2^k (rows of the strip block) and 2^(k - kx)
 template <int LOGN, int LOGE, int LOGRM>
-__device__ __noinline__ void rescale_fx(fx2* S, int k, int kx, const Inst1D& I, int tid) {
+__device__ __noinline__ void rescale_fx(fx2* S, int k, int kx, int nb, int blk0, int tid) {
     using F = Fx1D<LOGN, LOGE, LOGRM>;
     const int ko = max(k - kx, -62);
 #pragma unroll 1
     for (int j = 0; j < F::E; ++j) {
         const int n = tid + j * F::T;
         fx2& r = S[swz<fx2>(n)];
-        r = fx_scale(r, ((n - I.blk0) & (F::N - 1)) < I.nb ? k : ko);
+        r = fx_scale(r, ((n - blk0) & (F::N - 1)) < nb ? k : ko);
     }
 }
 
@@ -467,8 +467,9 @@ __device__ __forceinline__ fx2 fx_carry(fx2 Y, const int4* __restrict__ tab, int
     return ex;
 }
 
-// Strip Crank-Nicolson (strip_cn_1d in soft1d.cuh) in fixed point, times the
-// second half potential and field factor.  Every multiplier and chunk product
+// Strip Crank-Nicolson (strip_cn_1d in soft1d.cuh) in fixed point, followed by
+// post(v, c, n) on row c of the thread, grid index n (|v| < 2^60.5): the second
+// half potential and field factor.  Every multiplier and chunk product
 // has modulus <= 1 and the sweeps grow the rows by at most 2^lg (host check;
 // other plans take strip_cn_gen), so rows below 2^(59 - lg) cannot overflow;
 // coarse: rows beyond that (a packet inside the strip) are shifted right by
@@ -479,14 +480,12 @@ __device__ __forceinline__ fx2 fx_carry(fx2 Y, const int4* __restrict__ tab, int
 // the rows r; r_c = y_c - mf_c y_{c-1}, the same integer product, returns them
 // exactly.  kx: the block is left in units 2^kx times as large; returns the
 // thread's sum of fx_abs2 in those units.
-template <int LOGN, int LOGE, int LOGRM, class B>
-__device__ __forceinline__ float strip_cn_fx(fx2* S, const FxCn<Fx1D<LOGN, LOGE, LOGRM>::T>& cn,
-                                             const FxV<LOGN>& TVs, const int4* fr, double al, const Inst1D& I,
-                                             int tid, fx2* scan, B bar, bool coarse, int& kx) {
+template <int LOGN, int LOGE, int LOGRM, class B, class Post>
+__device__ __forceinline__ float strip_cn_fx(fx2* S, const FxCn<Fx1D<LOGN, LOGE, LOGRM>::T>& cn, int nb, int blk0,
+                                             int tid, fx2* scan, B bar, bool coarse, int& kx, Post post) {
     using F = Fx1D<LOGN, LOGE, LOGRM>;
     constexpr int N = F::N, T = F::T;
     constexpr int U = 2;
-    const int nb = I.nb, blk0 = I.blk0;
     const int ch = (nb + T - 1) / T;             // host guarantees ch <= CMAX
     const int i0 = tid * ch;
     const int nv = max(0, min(ch, nb - i0));     // rows of this thread
@@ -530,11 +529,8 @@ __device__ __forceinline__ float strip_cn_fx(fx2* S, const FxCn<Fx1D<LOGN, LOGE,
     float t2 = 0.0f;
 #pragma unroll U
     for (int c = 0; c < nv; ++c) {
-        const int4 tv = __ldg(&TVs.t[c * T + tid]);
         fx2& r = row(c);
-        fx2 v = half ? make_longlong2(fx_shr<1>(r.x), fx_shr<1>(r.y)) : r;
-        v = fx_mul<2>(v, tv);
-        if (I.has_field) v = fx_mul<2>(v, strip_field_fx<F::E>(fr, al, I, (blk0 + i0 + c) & (N - 1)));
+        const fx2 v = post(half ? fx_shr<1>(r) : r, c, (blk0 + i0 + c) & (N - 1));
         r = v;
         t2 += fx_abs2(v);
     }
@@ -543,14 +539,13 @@ __device__ __forceinline__ float strip_cn_fx(fx2* S, const FxCn<Fx1D<LOGN, LOGE,
 }
 
 // The same on rows held as doubles, in FP64 (strip_cn_1d): plans with the
-// `gen` flag.
-template <int LOGN, int LOGE, int LOGRM, class B>
-__device__ __noinline__ void strip_cn_gen(fx2* S, const double2* __restrict__ cn, const double2* __restrict__ tvs,
-                                          const int4* fr, double al, const Inst1D& I, int tid, double2* scan, B bar) {
+// `gen` flag.  cn: mf and g in chunk order.
+template <int LOGN, int LOGE, int LOGRM, class B, class Post>
+__device__ __forceinline__ void strip_cn_gen(fx2* S, const double2* __restrict__ cn, int nb, int blk0, int tid,
+                                             double2* scan, B bar, Post post) {
     using F = Fx1D<LOGN, LOGE, LOGRM>;
     using C = double2;
     constexpr int N = F::N, T = F::T, CMAX = F::K::CMAX;
-    const int nb = I.nb, blk0 = I.blk0;
     const int ch = (nb + T - 1) / T, P1 = (ch + 1) * T, i0 = tid * ch;
     const int nv = min(ch, nb - i0);
     auto row = [&](int c) -> fx2& { return S[swz<fx2>((blk0 + i0 + c) & (N - 1))]; };
@@ -584,13 +579,19 @@ __device__ __noinline__ void strip_cn_gen(fx2* S, const double2* __restrict__ cn
             yl = cfma(__ldg(&cn[(c + 1) * T + tid]), yl, y[c]);
             fx2& r = row(c);
             const C rc = fx_asd(r);
-            C v = cmul(cmk<C>(2 * yl.x - rc.x, 2 * yl.y - rc.y), __ldg(&tvs[c * T + tid]));
-            if (I.has_field) {
-                const int4 f = strip_field_fx<F::E>(fr, al, I, (blk0 + i0 + c) & (N - 1));
-                v = cmul(v, cscale(fx_to_double(fx_lift(f)), 0x1p-62));
-            }
-            r = fx_bits(v);
+            r = fx_bits(post(cmk<C>(2 * yl.x - rc.x, 2 * yl.y - rc.y), c, (blk0 + i0 + c) & (N - 1)));
         }
+}
+// with the second half potential and field factor of the 1D step
+template <int LOGN, int LOGE, int LOGRM, class B>
+__device__ __noinline__ void strip_gen_1d(fx2* S, const double2* __restrict__ cn, const double2* __restrict__ tvs,
+                                          const int4* fr, double al, const Inst1D& I, int tid, double2* scan, B bar) {
+    using F = Fx1D<LOGN, LOGE, LOGRM>;
+    strip_cn_gen<LOGN, LOGE, LOGRM>(S, cn, I.nb, I.blk0, tid, scan, bar, [&](double2 v, int c, int n) {
+        v = cmul(v, __ldg(&tvs[c * F::T + tid]));
+        if (I.has_field) v = cmul(v, cscale(fx_to_double(fx_lift(strip_field_fx<F::E>(fr, al, I, n))), 0x1p-62));
+        return v;
+    });
 }
 
 // Sum of the four accumulators over the group, times 2^e scale[r]; thread
@@ -672,7 +673,7 @@ __device__ __forceinline__ void soft1d_run_fx(const Inst1D& I, void* __restrict_
         if (step >= 0) {
             if (TV.gen) {
                 if (nb > 0) {
-                    strip_cn_gen<LOGN, LOGE, LOGRM, B>(S, cn.cd, TVs.d(((nb + T - 1) / T) * T), fr, al, I, tid, scan,
+                    strip_gen_1d<LOGN, LOGE, LOGRM, B>(S, cn.cd, TVs.d(((nb + T - 1) / T) * T), fr, al, I, tid, scan,
                                                        bar);
                     bar.sync();
                 }
@@ -681,8 +682,13 @@ __device__ __forceinline__ void soft1d_run_fx(const Inst1D& I, void* __restrict_
             } else {
                 e += TV.p;
                 if (nb > 0) {
-                    const float ts = strip_cn_fx<LOGN, LOGE, LOGRM>(S, cn, TVs, fr, al, I, tid,
-                                                                    reinterpret_cast<fx2*>(scan), bar, coarse, kx);
+                    const float ts = strip_cn_fx<LOGN, LOGE, LOGRM>(
+                        S, cn, nb, blk0, tid, reinterpret_cast<fx2*>(scan), bar, coarse, kx,
+                        [&](fx2 v, int c, int n) {
+                            v = fx_mul<2>(v, __ldg(&TVs.t[c * T + tid]));
+                            if (I.has_field) v = fx_mul<2>(v, strip_field_fx<E>(fr, al, I, n));
+                            return v;
+                        });
                     kx += TVs.p;
                     t2 = kx ? ts + t2 * exp2f(-2.0f * (float)kx) : ts + t2;
                     e += kx;
@@ -697,7 +703,7 @@ __device__ __forceinline__ void soft1d_run_fx(const Inst1D& I, void* __restrict_
         for (int w = 1; w < NW; ++w) t2 += part[w];
         const int k = fx_norm_shift(t2, N);
         e -= k;
-        if (k != 0 || kx != 0) rescale_fx<LOGN, LOGE, LOGRM>(S, k, kx, I, tid);
+        if (k != 0 || kx != 0) rescale_fx<LOGN, LOGE, LOGRM>(S, k, kx, nb, blk0, tid);
         // ---- kinetic: forward FFT, e^{-iK tau} (e^{-iK tau/2} in the first
         //      and last pass of the call), inverse FFT, potential of the next step
         const bool more = step + 1 < nsteps;

@@ -26,16 +26,12 @@ namespace soft {
 enum RowMode { ROW_K = 0, ROW_KVC = 1 };
 enum ColMode { COL_K = 0, COL_CVK = 1, COL_CBK = 2 };
 
-// Pass twiddles of the line passes.  Complex128 plans, which are bound by
-// the FP64 pipe, store every W^{M off} for the passes with a stride of at
-// most TWFULL_MAXS and W^{M off}, M = 1 .. 4, for the others (TwFull, as the
-// complex128 1D step), so a butterfly forms no products of bases.
-// Complex64 plans store the four bases W^{2^k off} per pass: their kernels
-// are bound by instruction issue with shared memory busy, and the full
-// tables' 15 loads per radix-16 butterfly measured slower than the 4 loads
-// and the products.
-template <typename R> struct Tw2D { using T = TwFull<typename CT<R>::C>; };
-template <> struct Tw2D<float> { using T = float2; };
+// The row and column kernels below are the complex64 ones (complex128:
+// soft2d_fix.cuh).  Their twiddles are the four bases W^{2^k off} per pass: the
+// kernels are bound by instruction issue with shared memory busy, and full
+// tables' 15 loads per radix-16 butterfly measured slower than 4 loads and the
+// products.
+template <typename R> struct Tw2D { using T = typename CT<R>::C; };
 
 // Shared memory of the row pass: the row (swizzled) and the scan scratch of
 // the strip CN, the row's e^{-iU tau/2}, the twiddles.
@@ -62,17 +58,15 @@ __device__ __forceinline__ void inv_pass0_post(typename CT<R>::C* S, const TW* _
     using G = PassGeom<LOGN, LOGRM, 0>;
     constexpr int LOGR = G::LOGR, RR = 1 << LOGR;
     constexpr int s = G::S;
-    constexpr bool FULL = TwLay<TW>::template full<LOGN, LOGRM, 0>();
 #pragma unroll 1
     for (int u = 0; u < K::E / RR; ++u) {
         const int off = tid + u * K::T;
         const int sb = swz<C>(off);
         C v[RR];
-        TW tb[FULL ? RR - 1 : 4];
+        TW tb[4];
         if constexpr (s > 1)
-            load_tw<TW, TwLay<TW>::template rows<LOGN, LOGRM, 0>(), s, SH>(
-                tb, W + TwLay<TW>::template toff<LOGN, LOGRM, 0>() + off);
-        LoadInv<C, TW, RR, s, 0, FULL>::run(S, v, tb, sb, s > 1);
+            load_tw<TW, G::LOGR, s, SH>(tb, W + G::TOFF + off);
+        LoadInv<C, TW, RR, s, 0>::run(S, v, tb, sb, s > 1);
         dft_reg<C, RR, +1>(v);
 #pragma unroll
         for (int m = 0; m < RR; ++m) S[sb ^ swz<C>(m * s)] = post(off + m * s, v[bitrev_c(m, LOGR)]);

@@ -8,8 +8,8 @@ namespace soft {
 struct Geo2D {              // passed by value to every 2D kernel
     const void* Wx;         // pass twiddles of the row FFT (length nx)
     const void* Wy;         // pass twiddles of the column FFT (length ny)
-    const void* TVh;        // e^{-iU tau/2}, [ny][nx] (minus 1, float2, for complex64)
-    const void* cnx;        // x-strip LU (mf, mb, g) for the row pass
+    const void* TVh;        // e^{-iU tau/2}, [ny][nx] (minus 1, float2, for complex64; complex128: factors)
+    const void* cnx;        // x-strip LU (mf, mb, g) for the row pass (complex128: FxCn)
     const void* cny;        // y-strip LU (mf, mb, g) for the column pass
     int nx, ny;             // row length; number of rows (3D: ny nz)
     int nbx, blk0x;         // x-strip block (same for every row)
@@ -18,6 +18,7 @@ struct Geo2D {              // passed by value to every 2D kernel
     // y-strip block and outside the z-strip block, y = r mod ny1 and
     // z = r / ny1 (2D: ny1 = ny, no z block)
     int v2, ny1, nz1, nbz1, blk0z1;
+    const void* vmeta;      // complex128: FxMeta of TVh
 };
 
 // Lines along a strided axis: element i of line c of plane p sits at
@@ -26,7 +27,7 @@ struct Geo2D {              // passed by value to every 2D kernel
 struct LineGeo {
     const void* W;          // pass twiddles of the line FFT
     int64_t ld, plane;
-    const void* cn;         // strip CN LU (mf, mb, g) along the lines (COL_CVK)
+    const void* cn;         // strip CN LU (mf, mb, g) along the lines (COL_CVK; complex128: FxCn)
     const void* tv;         // e^{-iU tau/2}, laid out as the state (COL_CVK)
     int nb, blk0;           // strip block along the lines (COL_CVK)
     // COL_CVK: with sel_div > 0 only lines whose (c / sel_div) mod sel_n lies
@@ -34,6 +35,7 @@ struct LineGeo {
     // (the row pass applied it on the others)
     int64_t sel_div;
     int sel_n, sel_nb, sel_blk0;
+    const void* vmeta;      // complex128: FxMeta of tv
 };
 
 // The strip CN along a strided axis: the cyclic block blk0 .. blk0 + nb - 1
