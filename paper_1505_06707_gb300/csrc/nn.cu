@@ -13,6 +13,7 @@
 #include "conv.cuh"
 #include "conv_tc.cuh"
 #include "nn.h"
+#include "wgrad.cuh"
 #include "plan_internal.h"
 
 namespace soft {
@@ -66,78 +67,6 @@ __global__ void pack_kernel(const float* __restrict__ P, __nv_bfloat16* __restri
         if (k < 18) v = P[P_W3 + ((k % 2) * 32 + ii) * 9 + (8 - k / 2)];
         b3[i] = __float2bfloat16(v);
     }
-}
-
-// Weight and bias gradients of one layer as per-CTA partials:
-// dW[o][c][tap] += sum_p g[p][o] in[p + tap][c], db[o] += sum_p g[p][o].
-// CTA = (field, band of ROWS rows); each thread owns a set of (o, c, tap).
-template <int CIN, int COUT, int INK, int GK /*0 bf16 NHWC, 1 float2 [H][W][2]*/>
-__global__ void __launch_bounds__(256)
-wgrad_kernel(const void* __restrict__ in, const void* __restrict__ gout, int H, int W, int rows,
-             float* __restrict__ part /* [gridDim.x * gridDim.y][COUT*CIN*9 + COUT] */)
-{
-    constexpr int NW = COUT * CIN * 9, NP = NW + COUT;
-    constexpr int PER = (NP + 255) / 256;
-    const int f = blockIdx.y, r0 = blockIdx.x * rows;
-    extern __shared__ float sm[];
-    float* tin = sm;                        // [3][W+2][CIN]
-    float* tg = sm + 3 * (W + 2) * CIN;     // [W][COUT]
-    float acc[PER];
-#pragma unroll
-    for (int q = 0; q < PER; ++q) acc[q] = 0.f;
-    for (int y = r0; y < r0 + rows && y < H; ++y) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < 3 * (W + 2) * CIN; i += blockDim.x) {
-            const int c = i % CIN, px = (i / CIN) % (W + 2), r = i / (CIN * (W + 2));
-            const int yy = (y + r - 1 + H) % H, xx = (px - 1 + W) % W;
-            const int64_t pix = (int64_t)f * H * W + (int64_t)yy * W + xx;
-            float v;
-            if (INK == IN_BF16) v = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(in)[pix * CIN + c]);
-            else v = reinterpret_cast<const float*>(in)[pix * 2 + c];
-            tin[i] = v;
-        }
-        for (int i = threadIdx.x; i < W * COUT; i += blockDim.x) {
-            const int64_t pix = (int64_t)f * H * W + (int64_t)y * W + i / COUT;
-            float v;
-            if (GK == 0) v = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(gout)[pix * COUT + i % COUT]);
-            else v = reinterpret_cast<const float*>(gout)[pix * 2 + i % COUT];
-            tg[i] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            const int id = threadIdx.x + q * 256;
-            if (id >= NP) continue;
-            float s = 0.f;
-            if (id < NW) {
-                const int tap = id % 9, c = (id / 9) % CIN, o = id / (9 * CIN);
-                const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-                const float* src = tin + ((dy + 1) * (W + 2) + dx + 1) * CIN + c;
-                for (int x = 0; x < W; ++x) s += tg[x * COUT + o] * src[x * CIN];
-            } else {
-                const int o = id - NW;
-                for (int x = 0; x < W; ++x) s += tg[x * COUT + o];
-            }
-            acc[q] += s;
-        }
-    }
-    const int64_t cta = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int id = threadIdx.x + q * 256;
-        if (id < NP) part[cta * NP + id] = acc[q];
-    }
-}
-
-// sum the CTA partials of one layer into the gradient vector (fixed order)
-__global__ void wgrad_reduce_kernel(const float* __restrict__ part, int ncta, int np, int nw,
-                                    float* __restrict__ gW, float* __restrict__ gb) {
-    const int id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= np) return;
-    double s = 0;
-    for (int c = 0; c < ncta; ++c) s += part[(int64_t)c * np + id];
-    if (id < nw) gW[id] = (float)s;
-    else gb[id - nw] = (float)s;
 }
 
 // loss = mean |out - target|^2 over all elements; gout = 2 (out - target)/n
@@ -308,27 +237,30 @@ int NNState::forward_c64(const void* x, int F, int H, int W, cudaStream_t st) {
     return SOFT_OK;
 }
 
-template <int CIN, int COUT, int INK, int GK>
+// weight and bias gradient of one layer (wgrad.cuh): about one CTA per SM, at
+// most MAXROWS rows of 128 pixels each
+template <int AK, int BK>
 static int wgrad(NNState& S, const void* in, const void* g, int F, int H, int W, float* gW, float* gb,
                  cudaStream_t st) {
-    constexpr int NP = COUT * CIN * 9 + COUT;
-    const int rows = 16;
-    dim3 grid((H + rows - 1) / rows, F);
-    const int64_t ncta = (int64_t)grid.x * grid.y;
-    if (ncta * NP > S.part_cap) {
+    using Q = WgCfg<AK, BK>;
+    const int64_t nrows = (int64_t)F * H * (W / 128);
+    const int rows = (int)std::max<int64_t>(1, std::min<int64_t>(Q::MAXROWS, (nrows + 151) / 152));
+    const int64_t ncta = (nrows + rows - 1) / rows;
+    if (ncta > 0x7fffffff) return SOFT_ERR_TOO_LARGE;
+    if (ncta * Q::NP > S.part_cap) {
         cudaFree(S.part);
         S.part = nullptr;
-        int rc = nn_alloc((void**)&S.part, sizeof(float) * ncta * NP);
+        S.part_cap = 0;
+        int rc = nn_alloc((void**)&S.part, sizeof(float) * ncta * Q::NP);
         if (rc) return rc;
-        S.part_cap = ncta * NP;
+        S.part_cap = ncta * Q::NP;
     }
-    const size_t smem = sizeof(float) * (3 * (W + 2) * CIN + W * COUT);
-    auto k = wgrad_kernel<CIN, COUT, INK, GK>;
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    auto k = wgrad_tc_kernel<AK, BK>;
+    if (Q::SMEM > 48 * 1024 &&
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Q::SMEM) != cudaSuccess)
         return SOFT_ERR_CUDA;
-    k<<<grid, 256, smem, st>>>(in, g, H, W, rows, S.part);
-    wgrad_reduce_kernel<<<(NP + 255) / 256, 256, 0, st>>>(S.part, (int)ncta, NP, NP - COUT, gW, gb);
+    k<<<(unsigned)ncta, Q::THREADS, Q::SMEM, st>>>(in, g, H, W, nrows, rows, S.part);
+    wgrad_reduce_kernel<<<(Q::NP + 31) / 32, 256, 0, st>>>(S.part, (int)ncta, Q::NP, Q::NW, gW, gb);
     return cudaGetLastError() == cudaSuccess ? SOFT_OK : SOFT_ERR_CUDA;
 }
 
@@ -341,17 +273,17 @@ int NNState::grad(const void* x, const void* t, int F, int H, int W, cudaStream_
     loss_kernel<<<256, 256, 0, st>>>(out, (const float*)t, n, gout, lpart);
     loss_reduce_kernel<<<1, 1, 0, st>>>(lpart, 256, n, lval);
     // layer 3: weight gradient, then the data gradient through ReLU of h2
-    if ((rc = wgrad<32, 2, IN_BF16, 1>(*this, h2, gout, F, H, W, G + P_W3, G + P_B3, st))) return rc;
+    if ((rc = wgrad<WG_SPLIT, WG_BF16_32>(*this, h2, gout, F, H, W, G + P_W3, G + P_B3, st))) return rc;
     ConvArgs a = cargs(gout, b3, nullptr, g2, H, W);
     a.mask = h2;
     if ((rc = launch_conv<2, 32, IN_C64, OUT_BF16_MASK>(a, F, st))) return SOFT_ERR_CUDA;
     // layer 2
-    if ((rc = wgrad<32, 32, IN_BF16, 0>(*this, h1, g2, F, H, W, G + P_W2, G + P_B2, st))) return rc;
+    if ((rc = wgrad<WG_BF16_32, WG_BF16_32>(*this, h1, g2, F, H, W, G + P_W2, G + P_B2, st))) return rc;
     a = cargs(g2, b2, nullptr, g1, H, W, err);
     a.mask = h1;
     if ((rc = launch_conv32_tc<32, OUT_BF16_MASK>(a, F, st))) return SOFT_ERR_CUDA;
     // layer 1
-    return wgrad<2, 32, IN_C64, 0>(*this, x, g1, F, H, W, G + P_W1, G + P_B1, st);
+    return wgrad<WG_BF16_32, WG_SPLIT>(*this, x, g1, F, H, W, G + P_W1, G + P_B1, st);
 }
 
 // one Adam step on the batch
