@@ -101,9 +101,11 @@ typedef struct {
     int persistent;      /* batch plans: 1 advances the instances with
                             N = 2048 .. 16384 by one persistent kernel that
                             takes packs of same-size instances from a queue,
-                            largest N first; 0 launches one kernel per size
-                            group.  With autotune the plan times both on one
-                            16-step chunk and keeps the faster [1]           */
+                            largest N first, if there is at most one pack per
+                            SM, and else, as 0 always does, by one kernel per
+                            size group (faster for larger batches; the results
+                            are the same).  With autotune the plan times both
+                            on one 16-step chunk and keeps the faster [1]    */
 } soft_options;
 
 /* Laser pulse (length gauge, x-polarised), E(t) = E0 sin^2(pi t/T) sin(omega t)

@@ -54,9 +54,9 @@ struct Tables1D {
     void* TVs = nullptr;
 };
 
-// Fixed-point passes of stride up to this store every twiddle W^{M off}, the
-// others eight rows (soft1d_fix.cuh, FxGeom).
-constexpr int FXFULL_MAXS = 256;
+// Fixed-point passes of stride up to this hold every twiddle W^{M off} in shared
+// memory, the others eight rows (soft1d_fix.cuh, FxGeom).
+constexpr int FXFULL_MAXS = 128;
 
 // Centre of the complex128 1D step (soft1d_fix.cuh).  The centre (last forward pass of r bits, k-space factor, first inverse
 // pass) must leave its outputs as an inverse pass of LOGRM bits would,

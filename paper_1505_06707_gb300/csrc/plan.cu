@@ -891,7 +891,17 @@ int soft_plan::build_1d_device() {
         }
         std::stable_sort(packs.begin(), packs.end(), [](const Pack1D& a, const Pack1D& b) { return a.var < b.var; });
         npacks = (int)packs.size();
-        use_persist = npacks > 0;
+        // The persistent kernel keeps one 512-thread CTA per SM for every size;
+        // per-size kernels keep two or more CTAs of the smaller sizes, whose
+        // phases fill each other's waits.  With more packs than SMs the latter
+        // are faster (16 steps of the mixed laser batch, persistent / per size:
+        // complex64, 4096 instances 7.71 / 6.24 ms, complex128, 1216 instances
+        // 9.5 / 7.9 ms), so the queue runs batches of at most one pack per SM.
+        int dev = 0, nsm = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return SOFT_ERR_CUDA;
+        use_persist = npacks > 0 && npacks <= nsm;
         if (npacks > 0) {
             if ((rc = upload((void**)&d_pinst, pd.data(), pd.size() * sizeof(Inst1D)))) return rc;
             if ((rc = upload(&d_packs, packs.data(), packs.size() * sizeof(Pack1D)))) return rc;

@@ -29,10 +29,11 @@
 namespace soft {
 
 // Twiddle tables (factor format): passes of a stride of at most FXFULL_MAXS
-// store every W^{M off}, the others W^{M off} for M = 1 .. 8 (a full table of
-// N = 16384's first pass would take 245 KB of shared memory; the seven
-// products cost a butterfly 84 of its 350 wide multiplies); the last pass,
-// of stride 1, has none.
+// hold every W^{M off} in shared memory; a radix-16 first pass of a larger
+// stride (N >= 4096) holds M = 1 .. 8 there and reads the other seven from
+// global memory, where they follow the table (N = 16384's full table would
+// take 245 KB; N = 4096 keeps two CTAs per SM: 1216 instances x 16 steps
+// 4.29 -> 3.24 ms).  The last pass, of stride 1, has none.
 template <int LOGN, int LOGRM, int P>
 struct FxGeom {
     using G = PassGeom<LOGN, LOGRM, P>;
@@ -92,15 +93,17 @@ struct Fx1D {
     static constexpr int N = K::N, T = K::T, E = K::E, NPASS = K::NPASS;
     static constexpr int RR = 1 << LOGRM;
     static_assert(E % RR == 0, "whole butterflies per thread");
-    // the first pass's twiddles above 8 are products (stride > FXFULL_MAXS)
+    // the first pass's twiddles above 8 are read from ext (stride > FXFULL_MAXS)
     static constexpr bool PART = LOGRM == 4 && (N >> LOGRM) > FXFULL_MAXS;
+    static constexpr int TWN = TwCountT<TwFix, LOGN, LOGRM>::value;
 
-    __device__ __forceinline__ static int4 tw(const int4* t, int s, int m, bool part) {
-        if (PART && m > 8 && part) return fx_mulw(t[7 * s], t[(m - 9) * s]);
+    __device__ __forceinline__ static int4 tw(const int4* t, const int4* __restrict__ ext, int s, int m, bool part) {
+        if (PART && m > 8 && part) return __ldg(&ext[(m - 9) * s]);
         return t[(m - 1) * s];
     }
+    // W: the table in shared memory, Wg in global memory (used by PART only)
     template <class B>
-    __device__ __forceinline__ static void fwd_all(fx2* S, const int4* W, int tid, B bar) {
+    __device__ __forceinline__ static void fwd_all(fx2* S, const int4* W, const int4* __restrict__ Wg, int tid, B bar) {
         const int4* Wp = W;
 #pragma unroll 1
         for (int P = 0; P < NPASS - 1; ++P) {
@@ -118,15 +121,15 @@ struct Fx1D {
                 const int4* t = Wp + off;
 #pragma unroll
                 for (int m = 1; m < RR; ++m)
-                    S[at(m)] = fx_mul<FxPass<LOGRM>::K>(v[bitrev_c(m, LOGRM)], tw(t, s, m, part));
+                    S[at(m)] = fx_mul<FxPass<LOGRM>::K>(v[bitrev_c(m, LOGRM)], tw(t, Wg + TWN + off, s, m, part));
             }
             Wp += (part ? 8 : RR - 1) << logs;
             bar.sync();
         }
     }
     template <class B>
-    __device__ __forceinline__ static void inv_all(fx2* S, const int4* W, int tid, B bar) {
-        const int4* Wp = W + TwCountT<TwFix, LOGN, LOGRM>::value;
+    __device__ __forceinline__ static void inv_all(fx2* S, const int4* W, const int4* __restrict__ Wg, int tid, B bar) {
+        const int4* Wp = W + TWN;
 #pragma unroll 1
         for (int P = NPASS - 2; P >= 0; --P) {
             const int logs = LOGN - LOGRM * (P + 1), s = 1 << logs;
@@ -140,7 +143,7 @@ struct Fx1D {
                 fx2 v[RR];
                 v[0] = fx_unit<LOGRM>(S[at.sb]);
 #pragma unroll
-                for (int m = 1; m < RR; ++m) v[m] = fx_mul<FxPass<LOGRM>::K, true>(S[at(m)], tw(t, s, m, part));
+                for (int m = 1; m < RR; ++m) v[m] = fx_mul<FxPass<LOGRM>::K, true>(S[at(m)], tw(t, Wg + TWN + off, s, m, part));
                 dft_reg<fx2, RR, +1>(v);
 #pragma unroll
                 for (int m = 0; m < RR; ++m) S[at(m)] = v[bitrev_c(m, LOGRM)];
@@ -644,6 +647,7 @@ __device__ __forceinline__ void soft1d_run_fx(const Inst1D& I, void* __restrict_
     fx2* __restrict__ g_psi = reinterpret_cast<fx2*>(psi_base) + I.off;
     fx2* S = K::GM ? g_psi : Ss;
     const int nb = I.nb, blk0 = I.blk0;
+    const int4* __restrict__ Wg = reinterpret_cast<const int4*>(I.W);
     if (nsteps <= 0) return;
     const FxV<LOGN> TV(I.TV, N), TVs(nb > 0 ? I.TVs : I.TV, nb > 0 ? ((nb + T - 1) / T) * T : N);
 
@@ -707,7 +711,7 @@ __device__ __forceinline__ void soft1d_run_fx(const Inst1D& I, void* __restrict_
         // ---- kinetic: forward FFT, e^{-iK tau} (e^{-iK tau/2} in the first
         //      and last pass of the call), inverse FFT, potential of the next step
         const bool more = step + 1 < nsteps;
-        F::fwd_all(S, Ws, tid, bar);
+        F::fwd_all(S, Ws, Wg, tid, bar);
         const int4* __restrict__ tk = reinterpret_cast<const int4*>((step >= 0 && more) ? I.TK : I.TKh);
         if constexpr (SURF) {
             fx2 acc[4];
@@ -729,7 +733,7 @@ __device__ __forceinline__ void soft1d_run_fx(const Inst1D& I, void* __restrict_
             field_setup_fx<LOGN, LOGE, LOGRM>(fr, al, I, tid);
         }
         bar.sync();
-        F::inv_all(S, Ws, tid, bar);
+        F::inv_all(S, Ws, Wg, tid, bar);
         unsigned mr = 0;
         if (more) {
             if (TV.gen) potential_gen<LOGN, LOGE, LOGRM>(S, TV.d(N), fr, I, tid);

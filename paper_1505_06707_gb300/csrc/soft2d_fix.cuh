@@ -154,10 +154,10 @@ row_fx_kernel(Geo2D g, void* __restrict__ psi_v, const void* __restrict__ tkx_v)
     for (int j = 0; j < E; ++j) S[swz<fx2>(tid + j * T)] = fx_from_double(d[j], ed);
     cp_async_wait<0>();
     __syncthreads();
-    F::fwd_all(S, Ws, tid, bar);
+    F::fwd_all(S, Ws, W, tid, bar);
     F::template center<false>(S, reinterpret_cast<const int4*>(tkx_v), tid, nullptr, nullptr);
     __syncthreads();
-    F::inv_all(S, Ws, tid, bar);
+    F::inv_all(S, Ws, W, tid, bar);
     const int nb = MODE == ROW_KVC ? g.nbx : 0, blk0 = g.blk0x;
     // rows outside the y- and z-strip blocks take the second V/2 here
     const int ry = (int)(y % g.ny1), rz = (int)(y / g.ny1);
@@ -343,10 +343,10 @@ col_fx_kernel(LineGeo lg, void* __restrict__ psi_v, const void* __restrict__ tky
         }
     }
     bar.sync();
-    F::fwd_all(Sc, Ws, tid, bar);
+    F::fwd_all(Sc, Ws, W, tid, bar);
     F::template center<false>(Sc, reinterpret_cast<const int4*>(tky_v), tid, nullptr, nullptr);
     bar.sync();
-    F::inv_all(Sc, Ws, tid, bar);
+    F::inv_all(Sc, Ws, W, tid, bar);
     if (tid == 0) ecol[col] = bad ? BADE : e;
     __syncthreads();
 #pragma unroll 2

@@ -269,25 +269,30 @@ std::vector<cd> pass_twiddles(int logn, int logrm) {
 
 // The fixed-point passes' twiddles (soft1d_fix.cuh, FxGeom): every
 // W_L^{M off} for strides up to full_maxs and radices below 16, M = 1 .. 8
-// otherwise, none for the last pass; times sqrt(2) for radices of odd log2.
+// otherwise (the first pass only; its other rows follow the table), none for
+// the last pass; times sqrt(2) for radices of odd log2.
 std::vector<int32_t> pass_twiddles_fx(int logn, int logrm, int full_maxs) {
     std::vector<int32_t> out;
-    int logl = logn;
+    auto row = [&](int logl, int lr, int M) {
+        for (int off = 0; off < 1 << (logl - lr); ++off) {
+            int64_t c, sn;
+            fx_cis_host(0 - ((uint64_t)M * off << (64 - logl)), &c, &sn);      // -M off / 2^logl turns
+            int32_t h[4];
+            fx_halves_host(lr & 1 ? fx_sqrt2_host(c) : c, h);
+            fx_halves_host(lr & 1 ? fx_sqrt2_host(sn) : sn, h + 2);
+            out.insert(out.end(), h, h + 4);
+        }
+    };
+    int logl = logn, first = 0;
     for (int lr : pass_radices(logn, logrm)) {
         const int s = 1 << (logl - lr), R = 1 << lr;
         const int rows = s == 1 ? 0 : (s <= full_maxs || lr < 4) ? R - 1 : 8;
-        for (int r = 0; r < rows; ++r)
-            for (int off = 0; off < s; ++off) {
-                const uint64_t e = (uint64_t)(r + 1) * off;
-                int64_t c, sn;
-                fx_cis_host(0 - (e << (64 - logl)), &c, &sn);      // -e / 2^logl turns
-                int32_t h[4];
-                fx_halves_host(lr & 1 ? fx_sqrt2_host(c) : c, h);
-                fx_halves_host(lr & 1 ? fx_sqrt2_host(sn) : sn, h + 2);
-                out.insert(out.end(), h, h + 4);
-            }
+        for (int M = 1; M <= rows; ++M) row(logl, lr, M);
+        if (logl == logn) first = rows;
         logl -= lr;
     }
+    if (first == 8 && logrm == 4)
+        for (int M = 9; M < 16; ++M) row(logn, 4, M);
     return out;
 }
 
