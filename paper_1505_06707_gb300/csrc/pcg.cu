@@ -37,6 +37,7 @@ struct Pcg {
     int *upd = nullptr, *lastu = nullptr, *mode = nullptr, *act32 = nullptr, *act64 = nullptr;
     // A tables in FP64 and FP32, and the preconditioners
     void *U = nullptr, *Cx = nullptr, *Cy = nullptr, *Kx = nullptr, *Ky = nullptr;
+    void *fWx = nullptr, *fWy = nullptr;       // fixed-point twiddles (FP64 passes)
     void *U32 = nullptr, *Cx32 = nullptr, *Cy32 = nullptr, *Kx32 = nullptr, *Ky32 = nullptr;
     PcgTables pc[3];             // simple, banded, banded with FP32 tables (and the FP32 A)
     bool tables = false;
@@ -48,7 +49,7 @@ struct Pcg {
     int gcap = 0;
     ~Pcg() {
         void* v[] = {r, z, p, w, t, dE, part, part2, rho, alpha, beta, relres, fnorm2, active, iters,
-                     status, nactive, rref, upd, lastu, mode, act32, act64, U, Cx, Cy, Kx, Ky, U32, Cx32, Cy32, Kx32, Ky32,
+                     status, nactive, rref, upd, lastu, mode, act32, act64, U, Cx, Cy, Kx, Ky, fWx, fWy, U32, Cx32, Cy32, Kx32, Ky32,
                      gP, gQ, gbeta, gpart, gqn};
         for (void* b : v) cudaFree(b);
         for (auto& T : pc)
@@ -69,6 +70,25 @@ static std::vector<cd> ksq_tab(const Axis1D& A, int logn, int logrm) {
         t[p] = 0.5 * k * k / A.n;
     }
     return t;
+}
+
+// k^2/2 2^-pk <= 1 as fixed-point factors in the transposed order of the fused
+// centre, with the passes' half bits (pcg_fix.cuh)
+static int upload_ksq_fx(void** dst, const Axis1D& A, int logn, int logrm, int* pk) {
+    const std::vector<int> perm = dif_output_order(logn, logrm);
+    const int lrl = (logn % logrm) ? logn % logrm : logrm;
+    const int Rl = 1 << lrl, nbf = A.n >> lrl;
+    double m = 0;
+    for (double k : A.k) m = std::max(m, 0.5 * k * k);
+    *pk = m > 0 ? (int)std::ceil(std::log2(m)) : 0;
+    const int half = (int)fx_center(lrl, logrm).s2 - (logrm & 1);
+    const double sc = std::ldexp(half == 0 ? 1.0 : half > 0 ? std::sqrt(2.0) : std::sqrt(0.5), -*pk);
+    std::vector<cd> t(A.n);
+    for (int p = 0; p < A.n; ++p) {
+        const double k = A.k[perm[p]];
+        t[(p % Rl) * nbf + p / Rl] = 0.5 * k * k * sc;
+    }
+    return upload_fx(dst, t);
 }
 
 static int build_pc(Plan2D* Q, int type, PcgTables& T, int prec = SOFT_C128) {
@@ -112,10 +132,40 @@ static int build_pc(Plan2D* Q, int type, PcgTables& T, int prec = SOFT_C128) {
             for (int u = 0; u < B.width[nu]; ++u) t[(size_t)u * B.n + nu] = tab[(size_t)B.off[nu] + u];
         return t;
     };
-    g.xfx = uc(umajor(bx, bx.xf)); g.xfy = uc(umajor(by, by.xf));
-    g.xbx = uc(umajor(bx, bx.xb)); g.xby = uc(umajor(by, by.xb));
+    if (prec == SOFT_C128) {
+        // fixed-point factors (pcg_fix.cuh): without the 1/sqrt n, times 2^-p
+        // with 2^p a bound of the operator norm (row sums times column sums);
+        // back: the half bits of the inverse FFT that follows
+        auto ux = [&](const BandAxis& B, const std::vector<cd>& tab, int logn, int logrm, bool back, int* p) -> const void* {
+            std::vector<cd> t = umajor(B, tab);
+            const double sn = std::sqrt((double)B.n);
+            std::vector<double> rows(B.n, 0.0), cols(B.n, 0.0);
+            for (int nu = 0; nu < B.n; ++nu)
+                for (int u = 0; u < B.width[nu]; ++u) {
+                    const double a = sn * std::abs(t[(size_t)u * B.n + nu]);
+                    rows[nu] += a;
+                    cols[B.start[nu] + u] += a;
+                }
+            const double nrm = std::sqrt(*std::max_element(rows.begin(), rows.end()) *
+                                         *std::max_element(cols.begin(), cols.end()));
+            *p = std::max(0, (int)std::ceil(std::log2(nrm * (1 + 1e-9))));
+            const int lrl = (logn % logrm) ? logn % logrm : logrm;
+            const int half = back ? ((logrm - lrl) & 1) - (logrm & 1) : 0;
+            const double sc = sn * std::ldexp(half == 0 ? 1.0 : half > 0 ? std::sqrt(2.0) : std::sqrt(0.5), -*p);
+            for (cd& v : t) v *= sc;
+            void* d = nullptr;
+            if (upload_fx(&d, t)) return nullptr;
+            T.bufs[i++] = d;
+            return d;
+        };
+        g.xfx = ux(bx, bx.xf, Q->lx, Q->lrx, false, &g.pfx); g.xfy = ux(by, by.xf, Q->ly, Q->lry, false, &g.pfy);
+        g.xbx = ux(bx, bx.xb, Q->lx, Q->lrx, true, &g.pbx); g.xby = ux(by, by.xb, Q->ly, Q->lry, true, &g.pby);
+    } else {
+        g.xfx = uc(umajor(bx, bx.xf)); g.xfy = uc(umajor(by, by.xf));
+        g.xbx = uc(umajor(bx, bx.xb)); g.xby = uc(umajor(by, by.xb));
+    }
     g.lamx = uc(bx.lam); g.lamy = uc(by.lam);
-    {                            // FFT twiddles (the four bases per pass)
+    if (prec == SOFT_C64) {      // FFT twiddles (the four bases per pass)
         auto ut = [&](const std::vector<cd>& v) -> const void* {
             void* d = nullptr;
             if (upload_tw(&d, v, prec)) return nullptr;
@@ -146,8 +196,11 @@ static int ensure_tables(Plan2D* Q) {
     };
     if ((rc = upload_c(&S->Cx, cat(Q->ax), SOFT_C128))) return rc;
     if ((rc = upload_c(&S->Cy, cat(Q->ay), SOFT_C128))) return rc;
-    if ((rc = upload_tab(&S->Kx, ksq_tab(Q->ax, Q->lx, Q->lrx), SOFT_C128))) return rc;
-    if ((rc = upload_tab(&S->Ky, ksq_tab(Q->ay, Q->ly, Q->lry), SOFT_C128))) return rc;
+    int pkx, pky;
+    if ((rc = upload_ksq_fx(&S->Kx, Q->ax, Q->lx, Q->lrx, &pkx))) return rc;
+    if ((rc = upload_ksq_fx(&S->Ky, Q->ay, Q->ly, Q->lry, &pky))) return rc;
+    if ((rc = upload_i32(&S->fWx, pass_twiddles_fx(Q->lx, Q->lrx, FXFULL_MAXS)))) return rc;
+    if ((rc = upload_i32(&S->fWy, pass_twiddles_fx(Q->ly, Q->lry, FXFULL_MAXS)))) return rc;
     if ((rc = upload_c(&S->U32, Q->U, SOFT_C64))) return rc;
     if ((rc = upload_c(&S->Cx32, cat(Q->ax), SOFT_C64))) return rc;
     if ((rc = upload_c(&S->Cy32, cat(Q->ay), SOFT_C64))) return rc;
@@ -158,7 +211,9 @@ static int ensure_tables(Plan2D* Q) {
         if ((rc = build_pc(Q, f32 ? 1 : type, S->pc[type], f32 ? SOFT_C64 : SOFT_C128))) return rc;
         PcgGeo& g = S->pc[type].geo;
         g.nx = Q->nx; g.ny = Q->ny; g.N = S->N;
-        g.Kx = f32 ? S->Kx32 : S->Kx; g.Ky = f32 ? S->Ky32 : S->Ky; g.U = f32 ? S->U32 : S->U;
+        if (f32) { g.Kx = S->Kx32; g.Ky = S->Ky32; }
+        else { g.fKx = S->Kx; g.fKy = S->Ky; g.fWx = S->fWx; g.fWy = S->fWy; g.pkx = pkx; g.pky = pky; }
+        g.U = f32 ? S->U32 : S->U;
         g.Cx = f32 ? S->Cx32 : S->Cx; g.Cy = f32 ? S->Cy32 : S->Cy;
         g.nbx = Q->geo.nbx; g.blk0x = Q->geo.blk0x; g.nby = Q->geo.nby; g.blk0y = Q->geo.blk0y;
     }

@@ -9,6 +9,7 @@
 //                                     energies that fall back: A with R double,
 //                                     IO complex64
 #include "pcg.cuh"
+#include "pcg_fix.cuh"
 #include "pcg_launch.h"
 
 namespace soft {
@@ -89,6 +90,53 @@ int pc_col(const PcgGeo& g, void* t, const double* E, const int* act, int nE, cu
     return done();
 }
 
+// the FP64 passes in fixed point (pcg_fix.cuh)
+template <typename IO, int LN>
+int a_row_fx(const PcgGeo& g, const void* p, void* w, const double* E, const int* act, int nE, cudaStream_t st) {
+    using Q = PcgFx<LN>;
+    auto k = a_row_fx_kernel<IO, LN>;
+    if (!set_smem(k, Q::SMEM_A)) return SOFT_ERR_CUDA;
+    if (nE > 0) k<<<dim3(g.ny, nE), Q::T, Q::SMEM_A, st>>>(g, p, w, E, act);
+    return done();
+}
+template <typename IO, int LN>
+int a_col_fx(const PcgGeo& g, const void* p, void* w, const int* act, double2* part, int pstride, int nE,
+             cudaStream_t st) {
+    using Q = PcgFx<LN>;
+    constexpr size_t smem = Q::template smem_col<TWP>(1);
+    auto k = a_col_fx_kernel<IO, LN, TWP>;
+    if (!set_smem(k, smem)) return SOFT_ERR_CUDA;
+    const int nb = g.nx / TWP;
+    if (nE > 0) k<<<dim3(nb, nE), TWP * Q::T, smem, st>>>(g, p, w, act, part, pstride > nb ? pstride : nb);
+    return done();
+}
+template <int LN>
+int pc_row_fx(int which, const PcgGeo& g, const void* a, void* b, const void* r, const int* act, double2* part,
+              int nE, cudaStream_t st) {
+    using Q = PcgFx<LN>;
+    const dim3 grid(g.ny, nE);
+    if (which == 1) {
+        auto k = pc_row1_fx_kernel<LN>;
+        if (!set_smem(k, Q::SMEM_P)) return SOFT_ERR_CUDA;
+        if (nE > 0) k<<<grid, Q::T, Q::SMEM_P, st>>>(g, a, b, act);
+    } else {
+        auto k = pc_row2_fx_kernel<LN>;
+        if (!set_smem(k, Q::SMEM_P)) return SOFT_ERR_CUDA;
+        if (nE > 0) k<<<grid, Q::T, Q::SMEM_P, st>>>(g, a, b, r, act, part);
+    }
+    return done();
+}
+template <int LN>
+int pc_col_fx(const PcgGeo& g, void* t, const double* E, const int* act, int nE, cudaStream_t st) {
+    using Q = PcgFx<LN>;
+    constexpr size_t smem = Q::template smem_col<TWP>(2);
+    static_assert(smem <= 227 * 1024, "shared memory");
+    auto k = pc_col_fx_kernel<LN, TWP>;
+    if (!set_smem(k, smem)) return SOFT_ERR_CUDA;
+    if (nE > 0) k<<<dim3(g.nx / TWP, nE), TWP * Q::T, smem, st>>>(g, t, E, act);
+    return done();
+}
+
 }  // namespace
 
 // every pass runs with LOGE = LOGRM = 3 (radix 8, eight elements per thread)
@@ -103,16 +151,16 @@ int pc_col(const PcgGeo& g, void* t, const double* E, const int* act, int nE, cu
 
 int pcg_row(int logn, int which, const PcgGeo& g, const void* a, void* b, const void* c,
             const double* E, const int* act, double2* part, int nE, cudaStream_t st) {
-#define CALL(L) (which == 0 ? a_row<double, double2, L, 3, 3>(g, a, b, E, act, nE, st) \
-                            : pc_row<double, double2, L, 3, 3>(which, g, a, b, c, nullptr, act, part, nullptr, nE, st))
+#define CALL(L) (which == 0 ? a_row_fx<double2, L>(g, a, b, E, act, nE, st) \
+                            : pc_row_fx<L>(which, g, a, b, c, act, part, nE, st))
     PCG_SIZES(CALL)
 #undef CALL
 }
 
 int pcg_col(int logn, int which, const PcgGeo& g, const void* a, void* b, const double* E,
             const int* act, double2* part, int nE, cudaStream_t st) {
-#define CALL(L) (which == 0 ? a_col<double, double2, L, 3, 3, TWP, 1>(g, a, b, act, part, 0, nE, st) \
-                            : pc_col<double, L, 3, 3, TWP, 1>(g, b, E, act, nE, st))
+#define CALL(L) (which == 0 ? a_col_fx<double2, L>(g, a, b, act, part, 0, nE, st) \
+                            : pc_col_fx<L>(g, b, E, act, nE, st))
     PCG_SIZES(CALL)
 #undef CALL
 }
@@ -157,14 +205,14 @@ int pcg_a32_col(int logn, const PcgGeo& g, const void* p, void* w, const int* ac
 
 int pcg_a64f_row(int logn, const PcgGeo& g, const void* p, void* w, const double* E, const int* act,
                  int nE, cudaStream_t st) {
-#define CALL(L) a_row<double, float2, L, 3, 3>(g, p, w, E, act, nE, st)
+#define CALL(L) a_row_fx<float2, L>(g, p, w, E, act, nE, st)
     PCG_SIZES(CALL)
 #undef CALL
 }
 
 int pcg_a64f_col(int logn, const PcgGeo& g, const void* p, void* w, const int* act, double2* part,
                  int pstride, int nE, cudaStream_t st) {
-#define CALL(L) a_col<double, float2, L, 3, 3, TWP, 1>(g, p, w, act, part, pstride, nE, st)
+#define CALL(L) a_col_fx<float2, L>(g, p, w, act, part, pstride, nE, st)
     PCG_SIZES(CALL)
 #undef CALL
 }
