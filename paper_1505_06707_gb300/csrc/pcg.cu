@@ -72,22 +72,48 @@ static std::vector<cd> ksq_tab(const Axis1D& A, int logn, int logrm) {
     return t;
 }
 
-// k^2/2 2^-pk <= 1 as fixed-point factors in the transposed order of the fused
-// centre, with the passes' half bits (pcg_fix.cuh)
-static int upload_ksq_fx(void** dst, const Axis1D& A, int logn, int logrm, int* pk) {
+// k^2/2 in the transposed order of the fused centre (pcg_fix.cuh, center_k)
+int upload_ksq(void** dst, const Axis1D& A, int logn, int logrm) {
     const std::vector<int> perm = dif_output_order(logn, logrm);
     const int lrl = (logn % logrm) ? logn % logrm : logrm;
     const int Rl = 1 << lrl, nbf = A.n >> lrl;
-    double m = 0;
-    for (double k : A.k) m = std::max(m, 0.5 * k * k);
-    *pk = m > 0 ? (int)std::ceil(std::log2(m)) : 0;
-    const int half = (int)fx_center(lrl, logrm).s2 - (logrm & 1);
-    const double sc = std::ldexp(half == 0 ? 1.0 : half > 0 ? std::sqrt(2.0) : std::sqrt(0.5), -*pk);
-    std::vector<cd> t(A.n);
+    std::vector<double> t(A.n);
     for (int p = 0; p < A.n; ++p) {
         const double k = A.k[perm[p]];
-        t[(p % Rl) * nbf + p / Rl] = 0.5 * k * k * sc;
+        t[(p % Rl) * nbf + p / Rl] = 0.5 * k * k;
     }
+    return upload(dst, t.data(), t.size() * sizeof(double));
+}
+
+// band rows u-major
+static std::vector<cd> umajor(const BandAxis& B, const std::vector<cd>& tab) {
+    int wmax = 1;
+    for (int wd : B.width) wmax = std::max(wmax, wd);
+    std::vector<cd> t((size_t)wmax * B.n, 0.0);
+    for (int nu = 0; nu < B.n; ++nu)
+        for (int u = 0; u < B.width[nu]; ++u) t[(size_t)u * B.n + nu] = tab[(size_t)B.off[nu] + u];
+    return t;
+}
+// the same as fixed-point factors (pcg_fix.cuh): without the 1/sqrt n, times
+// 2^-p with 2^p a bound of the operator norm (row sums times column sums);
+// back: the half bits of the inverse FFT that follows
+int upload_band_fx(void** dst, const BandAxis& B, const std::vector<cd>& tab, int logn, int logrm, bool back, int* p) {
+    std::vector<cd> t = umajor(B, tab);
+    const double sn = std::sqrt((double)B.n);
+    std::vector<double> rows(B.n, 0.0), cols(B.n, 0.0);
+    for (int nu = 0; nu < B.n; ++nu)
+        for (int u = 0; u < B.width[nu]; ++u) {
+            const double a = sn * std::abs(t[(size_t)u * B.n + nu]);
+            rows[nu] += a;
+            cols[B.start[nu] + u] += a;
+        }
+    const double nrm = std::sqrt(*std::max_element(rows.begin(), rows.end()) *
+                                 *std::max_element(cols.begin(), cols.end()));
+    *p = std::max(0, (int)std::ceil(std::log2(nrm) - 1e-6));       // (a norm of 1 keeps p = 0)
+    const int lrl = (logn % logrm) ? logn % logrm : logrm;
+    const int half = back ? ((logrm - lrl) & 1) - (logrm & 1) : 0;
+    const double sc = sn * std::ldexp(half == 0 ? 1.0 : half > 0 ? std::sqrt(2.0) : std::sqrt(0.5), -*p);
+    for (cd& v : t) v *= sc;
     return upload_fx(dst, t);
 }
 
@@ -124,37 +150,10 @@ static int build_pc(Plan2D* Q, int type, PcgTables& T, int prec = SOFT_C128) {
     g.bsx = ub(bx.start); g.bsy = ub(by.start);
     g.bwx = ub(bx.width); g.bwy = ub(by.width);
     // band rows u-major (entry u of row nu at u * n + nu), zero past each width
-    auto umajor = [](const BandAxis& B, const std::vector<cd>& tab) {
-        int wmax = 0;
-        for (int wd : B.width) wmax = std::max(wmax, wd);
-        std::vector<cd> t((size_t)wmax * B.n, cd(0.0, 0.0));
-        for (int nu = 0; nu < B.n; ++nu)
-            for (int u = 0; u < B.width[nu]; ++u) t[(size_t)u * B.n + nu] = tab[(size_t)B.off[nu] + u];
-        return t;
-    };
     if (prec == SOFT_C128) {
-        // fixed-point factors (pcg_fix.cuh): without the 1/sqrt n, times 2^-p
-        // with 2^p a bound of the operator norm (row sums times column sums);
-        // back: the half bits of the inverse FFT that follows
         auto ux = [&](const BandAxis& B, const std::vector<cd>& tab, int logn, int logrm, bool back, int* p) -> const void* {
-            std::vector<cd> t = umajor(B, tab);
-            const double sn = std::sqrt((double)B.n);
-            std::vector<double> rows(B.n, 0.0), cols(B.n, 0.0);
-            for (int nu = 0; nu < B.n; ++nu)
-                for (int u = 0; u < B.width[nu]; ++u) {
-                    const double a = sn * std::abs(t[(size_t)u * B.n + nu]);
-                    rows[nu] += a;
-                    cols[B.start[nu] + u] += a;
-                }
-            const double nrm = std::sqrt(*std::max_element(rows.begin(), rows.end()) *
-                                         *std::max_element(cols.begin(), cols.end()));
-            *p = std::max(0, (int)std::ceil(std::log2(nrm * (1 + 1e-9))));
-            const int lrl = (logn % logrm) ? logn % logrm : logrm;
-            const int half = back ? ((logrm - lrl) & 1) - (logrm & 1) : 0;
-            const double sc = sn * std::ldexp(half == 0 ? 1.0 : half > 0 ? std::sqrt(2.0) : std::sqrt(0.5), -*p);
-            for (cd& v : t) v *= sc;
             void* d = nullptr;
-            if (upload_fx(&d, t)) return nullptr;
+            if (upload_band_fx(&d, B, tab, logn, logrm, back, p)) return nullptr;
             T.bufs[i++] = d;
             return d;
         };
@@ -196,9 +195,8 @@ static int ensure_tables(Plan2D* Q) {
     };
     if ((rc = upload_c(&S->Cx, cat(Q->ax), SOFT_C128))) return rc;
     if ((rc = upload_c(&S->Cy, cat(Q->ay), SOFT_C128))) return rc;
-    int pkx, pky;
-    if ((rc = upload_ksq_fx(&S->Kx, Q->ax, Q->lx, Q->lrx, &pkx))) return rc;
-    if ((rc = upload_ksq_fx(&S->Ky, Q->ay, Q->ly, Q->lry, &pky))) return rc;
+    if ((rc = upload_ksq(&S->Kx, Q->ax, Q->lx, Q->lrx))) return rc;
+    if ((rc = upload_ksq(&S->Ky, Q->ay, Q->ly, Q->lry))) return rc;
     if ((rc = upload_i32(&S->fWx, pass_twiddles_fx(Q->lx, Q->lrx, FXFULL_MAXS)))) return rc;
     if ((rc = upload_i32(&S->fWy, pass_twiddles_fx(Q->ly, Q->lry, FXFULL_MAXS)))) return rc;
     if ((rc = upload_c(&S->U32, Q->U, SOFT_C64))) return rc;
@@ -212,7 +210,7 @@ static int ensure_tables(Plan2D* Q) {
         PcgGeo& g = S->pc[type].geo;
         g.nx = Q->nx; g.ny = Q->ny; g.N = S->N;
         if (f32) { g.Kx = S->Kx32; g.Ky = S->Ky32; }
-        else { g.fKx = S->Kx; g.fKy = S->Ky; g.fWx = S->fWx; g.fWy = S->fWy; g.pkx = pkx; g.pky = pky; }
+        else { g.fKx = S->Kx; g.fKy = S->Ky; g.fWx = S->fWx; g.fWy = S->fWy; }
         g.U = f32 ? S->U32 : S->U;
         g.Cx = f32 ? S->Cx32 : S->Cx; g.Cy = f32 ? S->Cy32 : S->Cy;
         g.nbx = Q->geo.nbx; g.blk0x = Q->geo.blk0x; g.nby = Q->geo.nby; g.blk0y = Q->geo.blk0y;

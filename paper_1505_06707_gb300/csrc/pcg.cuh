@@ -36,10 +36,10 @@ struct PcgGeo {
     const void* xfx; const void* xfy;      // forward band rows (complex)
     const void* xbx; const void* xby;      // backward band rows (complex)
     const void* lamx; const void* lamy;    // eigenvalues (complex)
-    // complex128 passes (pcg_fix.cuh): pass twiddles and kinetic factors (times
-    // 2^-pk) in fixed point; xf and xb are fixed-point factors times 2^-pf, 2^-pb
+    // complex128 passes (pcg_fix.cuh): pass twiddles in fixed point, k^2/2 as
+    // doubles; xf and xb are fixed-point factors times 2^-pf, 2^-pb
     const void* fWx; const void* fWy; const void* fKx; const void* fKy;
-    int pkx, pky, pfx, pfy, pbx, pby;
+    int pfx, pfy, pbx, pby;
     int64_t N;                              // nx * ny
 };
 

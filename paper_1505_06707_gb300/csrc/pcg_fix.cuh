@@ -10,14 +10,28 @@
 // products of ten complex terms (160).
 //
 // Scaling.  Forward and inverse FFTs are unitary (1/sqrt N each, so the band
-// rows come without it).  The kinetic factor enters as k^2/2 2^-pk <= 1, the
-// band rows as X 2^-pb, pb from a bound of their operator norm, so that no
-// line's norm grows.
+// rows come without it).  The band rows enter as X 2^-pb, pb from a bound of
+// their operator norm, so that no line's norm grows.  The kinetic factor is
+// applied in FP64 and the line given a new exponent after it (center_k): with
+// k^2/2 2^-pk <= 1 as a fixed-point factor the inverse FFT's rounding is
+// relative to max(k^2/2) |p| instead of |K p|, in the modes of small k too,
+// where P^-1 amplifies it (COCG with absorbing potentials took up to 9
+// iterations more, of 45, at low energies; A of a smooth vector, N = 1024: off
+// by 9.7e-15 of |p|, 2.7e-15 so, 3.5e-14 in FP64).  It costs 2 FP64
+// instructions per point (A and P^-1 at 1024^2: 335 -> 341 us).
 #pragma once
 #include "pcg.cuh"
 #include "soft2d_fix.cuh"
 
 namespace soft {
+
+// per-line scratch behind the buffers: sums and maxima of fx_line_exp
+struct PcgScr {
+    float* part;
+    unsigned* red;
+    __device__ __forceinline__ explicit PcgScr(void* p) : part(reinterpret_cast<float*>(p)),
+                                                         red(reinterpret_cast<unsigned*>(part + 16)) {}
+};
 
 template <int LOGN>
 struct PcgFx : LineFx<LOGN, 3, 3> {
@@ -32,8 +46,6 @@ struct PcgFx : LineFx<LOGN, 3, 3> {
         return sizeof(fx2) * ((size_t)bufs * TW * PITCH + L::TWN) + TW * L::SCR + 64;
     }
     static constexpr int MINB = L::MINB;
-    static constexpr int SH_K = -L::SH;         // exponent of what the last inverse pass leaves over
-
     // last forward pass (stride 1, no twiddles), unitary
     __device__ __forceinline__ static void fwd_last(fx2* S, int tid) {
         constexpr int RR = 1 << R;
@@ -47,6 +59,43 @@ struct PcgFx : LineFx<LOGN, 3, 3> {
 #pragma unroll
             for (int m = 0; m < RR; ++m) S[sb ^ swz<fx2>(m)] = fx_unit<R>(v[bitrev_c(m, R)]);
         }
+    }
+    // last forward pass, k^2/2 in FP64 (kt, the centre's transposed order), a
+    // new exponent, first inverse pass.  Returns the exponent relative to the
+    // line's before: of the normalisation, and of the scaling that the two
+    // passes and the last inverse pass (2^-1) leave over, which is a power of 2.
+    template <class B>
+    __device__ __forceinline__ static int center_k(fx2* S, const double* __restrict__ kt, PcgScr sc, int tid, B bar,
+                                                   bool& bad) {
+        constexpr int RR = 1 << R, cs = (3 - R) / 2;
+        double2 d[E];
+#pragma unroll
+        for (int u = 0; u < E / RR; ++u) {
+            const int sb = swz<fx2>((tid + u * T) * RR);
+            fx2 v[RR];
+#pragma unroll
+            for (int j = 0; j < RR; ++j) v[j] = S[sb ^ swz<fx2>(j)];
+            dft_reg<fx2, RR, -1>(v);
+#pragma unroll
+            for (int m = 0; m < RR; ++m)
+                d[u * RR + m] = cscale(fx_to_double(v[bitrev_c(m, R)]), __ldg(&kt[m * (N / RR) + tid + u * T]));
+        }
+        int ed;
+        const int e = fx_line_exp<E, T>(d, sc.part, sc.red, tid, bar, ed, bad);
+#pragma unroll
+        for (int u = 0; u < E / RR; ++u) {
+            const int sb = swz<fx2>((tid + u * T) * RR);
+            fx2 w[RR];
+#pragma unroll
+            for (int m = 0; m < RR; ++m) w[m] = fx_from_double(d[u * RR + m], ed);
+            dft_reg<fx2, RR, +1>(w);
+#pragma unroll
+            for (int m = 0; m < RR; ++m) {
+                const fx2 o = w[bitrev_c(m, R)];
+                S[sb ^ swz<fx2>(m)] = make_longlong2(o.x << cs, o.y << cs);
+            }
+        }
+        return e - R - cs;
     }
     // first inverse pass, left as large as a pass of 3 bits leaves it (the
     // tables before it carry the half bits)
@@ -66,14 +115,6 @@ struct PcgFx : LineFx<LOGN, 3, 3> {
             }
         }
     }
-};
-
-// per-line scratch behind the buffers: sums and maxima of fx_line_exp
-struct PcgScr {
-    float* part;
-    unsigned* red;
-    __device__ __forceinline__ explicit PcgScr(void* p) : part(reinterpret_cast<float*>(p)),
-                                                         red(reinterpret_cast<unsigned*>(part + 16)) {}
 };
 
 __device__ __forceinline__ double2 fx_nan2() {
@@ -140,10 +181,11 @@ a_row_fx_kernel(PcgGeo g, const void* __restrict__ p_v, void* __restrict__ w_v, 
     cp_async_wait<0>();
     __syncthreads();
     F::fwd_all(S, Ws, W, tid, bar);
-    F::template center<false>(S, reinterpret_cast<const int4*>(g.fKx), tid, nullptr, nullptr);
+    bool bad2;
+    el += Q::center_k(S, reinterpret_cast<const double*>(g.fKx), sc, tid, bar, bad2);
+    bad = bad || bad2;
     __syncthreads();
     F::inv_all(S, Ws, W, tid, bar);
-    el += Q::SH_K + g.pkx;
     const double2* __restrict__ U = reinterpret_cast<const double2*>(g.U) + (int64_t)y * N;
     const double2* __restrict__ Cx = reinterpret_cast<const double2*>(g.Cx);
     const double En = E[e];
@@ -228,11 +270,13 @@ a_col_fx_kernel(PcgGeo g, const void* __restrict__ p_v, void* __restrict__ w_v, 
     const int col = threadIdx.x / T, tid = threadIdx.x % T;
     const BarGroup bar{1 + col, T};
     fx2* Sc = S + col * PITCH;
-    bool bad;
-    const int el = col_exp<LOGN>(Sc, true, PcgScr(scr + col * Q::SCR), tid, bar, bad) + Q::SH_K + g.pky;
+    const PcgScr sc(scr + col * Q::SCR);
+    bool bad, bad2;
+    int el = col_exp<LOGN>(Sc, true, sc, tid, bar, bad);
     bar.sync();
     F::fwd_all(Sc, Ws, W, tid, bar);
-    F::template center<false>(Sc, reinterpret_cast<const int4*>(g.fKy), tid, nullptr, nullptr);
+    el += Q::center_k(Sc, reinterpret_cast<const double*>(g.fKy), sc, tid, bar, bad2);
+    bad = bad || bad2;
     bar.sync();
     F::inv_all(Sc, Ws, W, tid, bar);
     if (tid == 0) ecol[col] = bad ? BADE : el;

@@ -60,6 +60,10 @@ struct Geo2D;
 struct NNState;
 struct Sse1D;
 void sse1d_free(Sse1D* s);
+// tables of the fixed-point stationary solvers (pcg.cu)
+struct BandAxis;
+int upload_ksq(void** dst, const Axis1D& A, int logn, int logrm);
+int upload_band_fx(void** dst, const BandAxis& B, const std::vector<cd>& tab, int logn, int logrm, bool back, int* p);
 struct Surf1D;
 void surf1d_free(Surf1D* s);
 int sse1d_refill_potential(soft_plan* P);
