@@ -8,30 +8,38 @@
 // vectors x, r, p, z of that energy stay in shared memory (6 N complex128,
 // 192 KB at N = 2048), so an iteration touches global memory only for the
 // tables, which every CTA shares through L2.  The scalars of the iteration
-// are block sums broadcast through shared memory: every thread takes the
-// same branch, and the loop ends at convergence, breakdown or maxit.
+// are block sums, which every thread forms alike and so takes the same
+// branch; the loop ends at convergence, breakdown or maxit.
+//
+// FFTs and the band products run in 64-bit fixed point (pcg_fix.cuh); the
+// vectors, k^2/2, the potential and strip terms, 1/(lambda - E) and the sums
+// are FP64.  In FP64 throughout an iteration took about 170
+// clocks of an SM per point, most of it in the FP64 pipe (2 instructions per
+// clock and SM); 38 FP64 instructions per point are left: 30 energies at
+// N = 1024, tolerance 1e-12, take 2.17 ms instead of 4.83.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 
 #include "band.h"
-#include "pcg.cuh"
+#include "pcg_fix.cuh"
 #include "plan_internal.h"
 
 namespace soft {
 
 struct Sse1DGeo {
-    const double2* W;                  // pass twiddle bases (double2)
-    const double2* K;                  // k^2/(2N) in the forward FFT's output order
+    const int4* W;                     // pass twiddles
+    const double* K;                   // k^2/2 in the order of the fused centre
     const double2* U;                  // U(z(x_j)), natural order
     const double2* C;                  // C[j][j-1], C[j][j], C[j][j+1] (3N)
     int nb, blk0;                      // rows of the cyclic block where C is non-zero
     const int* pos;                    // FFT output position of natural index m
     const int* bs;                     // band start of row nu
     const int* bw;                     // band width of row nu
-    const double2* xf;                 // band rows of X (u-major, e^{i k x0}/sqrt N folded in)
-    const double2* xb;                 // band rows of X^T (u-major, e^{-i k x0}/sqrt N folded in)
+    const int4* xf;                    // band rows of X 2^-pf (u-major, e^{i k x0} folded in)
+    const int4* xb;                    // band rows of X^T 2^-pb (u-major, e^{-i k x0} folded in)
     const double2* lam;                // eigenvalues lambda_nu
+    int pf, pb;
 };
 
 namespace {
@@ -41,187 +49,223 @@ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
     return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
 }
 
-// sum of v over the CTA, returned to every thread (red: 33 entries)
-__device__ __forceinline__ double2 bsum(double2 v, double2* red) {
+// One energy's CTA: S (the FFT buffer, swizzled), T1, x, r, p, z of N complex
+// each, the twiddles, scratch and two sets of warp sums
+template <int LOGN>
+struct Sse1 {
+    using Q = PcgFx<LOGN>;
+    using F = typename Q::F;
+    static constexpr int N = Q::N, T = Q::T, E = Q::E, NW = T / 32;
+    static constexpr size_t SMEM = sizeof(fx2) * (6 * N + Q::TWN) + Q::SCR + sizeof(double2) * 2 * NW;
+    static_assert(SMEM <= 227 * 1024, "shared memory");
+    const Sse1DGeo& g;
+    fx2 *S, *T1;
+    double2 *x, *r, *p, *z;
+    int4* Ws;
+    PcgScr sc;
+    double2* red;
+    const int tid;
+    const BarCTA bar;
+    int par = 0;
+    double2 ri[E];                     // 1/(lambda_nu - E) on the thread's rows nu = tid + j T
+
+    __device__ __forceinline__ Sse1(const Sse1DGeo& g_, unsigned char* sm, double En, bool pc)
+        : g(g_), S(reinterpret_cast<fx2*>(sm)), T1(S + N), x(reinterpret_cast<double2*>(T1 + N)), r(x + N), p(r + N),
+          z(p + N), Ws(reinterpret_cast<int4*>(z + N)), sc(Ws + Q::TWN),
+          red(reinterpret_cast<double2*>(reinterpret_cast<unsigned char*>(Ws + Q::TWN) + Q::SCR)), tid(threadIdx.x), bar() {
+        for (int i = tid; i < Q::TWN; i += T) cp_async<16>(&Ws[i], &g.W[i]);
+        cp_async_commit();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-    }
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-    __syncthreads();                    // red may still be read by the previous sum
-    if (l == 0) red[w] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double2 t = make_double2(0.0, 0.0);
-        for (int i = 0; i < nw; ++i) { t.x += red[i].x; t.y += red[i].y; }
-        red[32] = t;
-    }
-    __syncthreads();
-    return red[32];
-}
-
-// w = A p for the CTA's energy (p, w natural order in shared memory; S is
-// the swizzled FFT buffer).  Ends with a barrier.
-template <int LOGN, int LOGE, int LOGRM>
-__device__ __forceinline__ void apply_A(const Sse1DGeo& g, const double2* p, double2* w, double2* S, double En,
-                                        int tid) {
-    using K = Cfg1D<double, LOGN, LOGE, LOGRM>;
-    constexpr int N = K::N, T = K::T, E_ = K::E;
-    for (int j = 0; j < E_; ++j) {
-        const int n = tid + j * T;
-        S[swz<double2>(n)] = p[n];
-    }
-    __syncthreads();
-    fwd_fft<double, LOGN, LOGE, LOGRM, 0>(S, g.W, tid);
-    kmul<double, LOGN, LOGE, LOGRM>(S, g.K, tid);
-    inv_fft<double, LOGN, LOGE, LOGRM, K::NPASS - 1>(S, g.W, tid);
-    for (int j = 0; j < E_; ++j) {
-        const int n = tid + j * T;
-        const double2 pv = p[n];
-        double2 u = __ldg(&g.U[n]);
-        u.x -= En;
-        double2 v = cfma(u, pv, S[swz<double2>(n)]);
-        if (((n - g.blk0) & (N - 1)) < g.nb) {
-            v = cfma(__ldg(&g.C[n]), p[(n + N - 1) & (N - 1)], v);
-            v = cfma(__ldg(&g.C[N + n]), pv, v);
-            v = cfma(__ldg(&g.C[2 * N + n]), p[(n + 1) & (N - 1)], v);
+        for (int j = 0; j < E; ++j) {
+            if (!pc) { ri[j] = make_double2(0.0, 0.0); continue; }
+            double2 den = __ldg(&g.lam[tid + j * T]);
+            den.x -= En;
+            ri[j] = cscale(cconj(den), 1.0 / (den.x * den.x + den.y * den.y));
         }
-        w[n] = v;
+        cp_async_wait<0>();
+        __syncthreads();
     }
-    __syncthreads();
-}
 
-// z = P^-1 r (r, z natural order; T1 natural-order scratch; S the FFT
-// buffer).  The paper's F has e^{+ikx}: conj(FFT(conj(.))).  Ends with a barrier.
-template <int LOGN, int LOGE, int LOGRM>
-__device__ __forceinline__ void apply_P(const Sse1DGeo& g, const double2* r, double2* z, double2* S, double2* T1,
-                                        double En, int tid) {
-    using K = Cfg1D<double, LOGN, LOGE, LOGRM>;
-    constexpr int N = K::N, T = K::T, E_ = K::E;
-    for (int j = 0; j < E_; ++j) {
-        const int n = tid + j * T;
-        S[swz<double2>(n)] = cconj(r[n]);
+    // sum of v over the CTA in every thread; consecutive sums use the two sets in turn
+    __device__ __forceinline__ double2 bsum(double2 v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+            v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+        }
+        if constexpr (NW == 1) return v;
+        double2* s = red + par * NW;
+        par ^= 1;
+        if ((tid & 31) == 0) s[tid >> 5] = v;
+        __syncthreads();
+        v = s[tid & (NW - 1)];
+#pragma unroll
+        for (int o = NW / 2; o > 0; o >>= 1) {
+            v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+            v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+        }
+        return v;
     }
-    __syncthreads();
-    fwd_fft<double, LOGN, LOGE, LOGRM, 0>(S, g.W, tid);
-    for (int j = 0; j < E_; ++j) {
-        const int m = tid + j * T;
-        T1[m] = cconj(S[swz<double2>(__ldg(&g.pos[m]))]);
-    }
-    __syncthreads();
-    for (int j = 0; j < E_; ++j) {               // X F r, then / (lambda - E)
-        const int nu = tid + j * T;
-        const int s0 = __ldg(&g.bs[nu]), wd = __ldg(&g.bw[nu]);
-        double2 o = make_double2(0.0, 0.0);
-        for (int u = 0; u < wd; ++u) o = cfma(__ldg(&g.xf[u * N + nu]), T1[s0 + u], o);
-        double2 den = __ldg(&g.lam[nu]);
-        den.x -= En;
-        z[nu] = cdiv(o, den);
-    }
-    __syncthreads();
-    for (int j = 0; j < E_; ++j) {               // X^T into the FFT positions (conjugated)
-        const int m = tid + j * T;
-        const int s0 = __ldg(&g.bs[m]), wd = __ldg(&g.bw[m]);
-        double2 o = make_double2(0.0, 0.0);
-        for (int u = 0; u < wd; ++u) o = cfma(__ldg(&g.xb[u * N + m]), z[s0 + u], o);
-        S[swz<double2>(__ldg(&g.pos[m]))] = cconj(o);
-    }
-    __syncthreads();
-    inv_fft<double, LOGN, LOGE, LOGRM, K::NPASS - 1>(S, g.W, tid);
-    for (int j = 0; j < E_; ++j) {
-        const int n = tid + j * T;
-        z[n] = cconj(S[swz<double2>(n)]);
-    }
-    __syncthreads();
-}
 
-template <int LOGN, int LOGE, int LOGRM>
-constexpr size_t sse1d_smem() {
-    return sizeof(double2) * (6 * (size_t(1) << LOGN) + 33);
-}
+    // z = A p on the thread's own rows; returns the thread's part of p^T z
+    __device__ __forceinline__ double2 apply_A(double En) {
+        double2 d[E];
+#pragma unroll
+        for (int j = 0; j < E; ++j) d[j] = p[tid + j * T];
+        int ed;
+        bool bad;
+        int el = fx_line_exp<E, T>(d, sc.part, sc.red, tid, bar, ed, bad);
+#pragma unroll
+        for (int j = 0; j < E; ++j) S[swz<fx2>(tid + j * T)] = fx_from_double(d[j], ed);
+        __syncthreads();
+        F::fwd_all(S, Ws, g.W, tid, bar);
+        bool bad2;
+        el += Q::center_k(S, g.K, sc, tid, bar, bad2);
+        bad = bad || bad2;
+        __syncthreads();
+        F::inv_all(S, Ws, g.W, tid, bar);
+        double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 2
+        for (int j = 0; j < E; ++j) {
+            const int n = tid + j * T;
+            const double2 pv = p[n];
+            double2 u = __ldg(&g.U[n]);
+            u.x -= En;
+            double2 v = bad ? fx_nan2() : fx_value(S[swz<fx2>(n)], el);
+            v = cfma(u, pv, v);
+            if (((n - g.blk0) & (N - 1)) < g.nb) {
+                v = cfma(__ldg(&g.C[n]), p[(n + N - 1) & (N - 1)], v);
+                v = cfma(__ldg(&g.C[N + n]), pv, v);
+                v = cfma(__ldg(&g.C[2 * N + n]), p[(n + 1) & (N - 1)], v);
+            }
+            z[n] = v;
+            acc = cfma(pv, v, acc);
+        }
+        return acc;
+    }
+
+    // z = P^-1 r on the thread's own rows; returns the thread's part of r^T z.
+    // The paper's F has e^{+ikx}: conj(FFT(conj(.))).
+    __device__ __forceinline__ double2 apply_P() {
+        double2 d[E];
+#pragma unroll
+        for (int j = 0; j < E; ++j) d[j] = cconj(r[tid + j * T]);
+        int ed;
+        bool bad, bad2;
+        int el = fx_line_exp<E, T>(d, sc.part, sc.red, tid, bar, ed, bad) + g.pf;
+#pragma unroll
+        for (int j = 0; j < E; ++j) S[swz<fx2>(tid + j * T)] = fx_from_double(d[j], ed);
+        __syncthreads();
+        F::fwd_all(S, Ws, g.W, tid, bar);
+        Q::fwd_last(S, tid);
+        __syncthreads();
+#pragma unroll 2
+        for (int j = 0; j < E; ++j) {                  // F r in natural index order
+            const int m = tid + j * T;
+            T1[m] = fx_conj(S[swz<fx2>(__ldg(&g.pos[m]))]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j0 = 0; j0 < E; j0 += BAND_NJ) {      // X F r, then / (lambda - E)
+            fx2 o[BAND_NJ];
+            band_rows_fx<BAND_NJ>(tid + j0 * T, T, N, g.bs, g.bw, g.xf, [&](int m) { return T1[m]; }, o);
+#pragma unroll
+            for (int j = 0; j < BAND_NJ; ++j) d[j0 + j] = cmul(fx_value(o[j], el), ri[j0 + j]);
+        }
+        el = fx_line_exp<E, T>(d, sc.part, sc.red, tid, bar, ed, bad2) + g.pb - 1;    // (-1: as pc_col_fx_kernel)
+        bad = bad || bad2;
+        fx2* zf = reinterpret_cast<fx2*>(z);
+#pragma unroll
+        for (int j = 0; j < E; ++j) zf[tid + j * T] = fx_from_double(d[j], ed);
+        __syncthreads();
+#pragma unroll 1
+        for (int j0 = 0; j0 < E; j0 += BAND_NJ) {      // X^T into the FFT positions (conjugated)
+            fx2 o[BAND_NJ];
+            band_rows_fx<BAND_NJ>(tid + j0 * T, T, N, g.bs, g.bw, g.xb, [&](int nu) { return zf[nu]; }, o);
+#pragma unroll
+            for (int j = 0; j < BAND_NJ; ++j) S[swz<fx2>(__ldg(&g.pos[tid + (j0 + j) * T]))] = fx_conj(o[j]);
+        }
+        __syncthreads();
+        Q::inv_first(S, tid);
+        __syncthreads();
+        F::inv_all(S, Ws, g.W, tid, bar);
+        double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 2
+        for (int j = 0; j < E; ++j) {
+            const int n = tid + j * T;
+            const double2 zv = bad ? fx_nan2() : cconj(fx_value(S[swz<fx2>(n)], el));
+            z[n] = zv;
+            acc = cfma(r[n], zv, acc);
+        }
+        return acc;
+    }
+};
 
 // COCG (Sec. III after Eq. linsys: the bilinear r^T z replaces the inner
 // product), x0 = 0, stop when ||r||_2/||f||_2 < tol; energy blockIdx.x
-template <int LOGN, int LOGE, int LOGRM>
-__global__ void __launch_bounds__(Cfg1D<double, LOGN, LOGE, LOGRM>::T, 1)
+template <int LOGN>
+__global__ void __launch_bounds__(Sse1<LOGN>::T, 1)
 sse1d_cocg_kernel(Sse1DGeo g, const double2* __restrict__ f, double2* __restrict__ xout,
                   const double* __restrict__ Es, double tol, int maxit, int* __restrict__ iters,
                   double* __restrict__ relres, int* __restrict__ status)
 {
-    using K = Cfg1D<double, LOGN, LOGE, LOGRM>;
-    constexpr int N = K::N, T = K::T, E_ = K::E;
+    using Q = Sse1<LOGN>;
+    constexpr int N = Q::N, T = Q::T, E_ = Q::E;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2* S = reinterpret_cast<double2*>(smem_raw);
-    double2* T1 = S + N;
-    double2* x = T1 + N;
-    double2* r = x + N;
-    double2* p = r + N;
-    double2* z = p + N;
-    double2* red = z + N;
     const int e = blockIdx.x, tid = threadIdx.x;
     const double En = Es[e];
+    Q q(g, smem_raw, En, true);
+    double2 *x = q.x, *r = q.r, *p = q.p, *z = q.z;
     double ff = 0.0;
     for (int j = 0; j < E_; ++j) {
         const int n = tid + j * T;
         const double2 fv = f[n];
         r[n] = fv;
         x[n] = make_double2(0.0, 0.0);
+        p[n] = make_double2(0.0, 0.0);
         ff += fv.x * fv.x + fv.y * fv.y;
     }
-    ff = bsum(make_double2(ff, 0.0), red).x;
+    ff = q.bsum(make_double2(ff, 0.0)).x;
     int st = SOFT_ERR_NOT_CONVERGED, it = 0;
     double rel = 1.0;
     if (!(ff > 0.0) || !isfinite(ff)) {
         st = ff == 0.0 ? SOFT_OK : SOFT_ERR_NONFINITE;
         rel = 0.0;
     } else {
-        apply_P<LOGN, LOGE, LOGRM>(g, r, z, S, T1, En, tid);
-        double2 acc = make_double2(0.0, 0.0);
-        for (int j = 0; j < E_; ++j) {
-            const int n = tid + j * T;
-            p[n] = z[n];
-            acc = cfma(r[n], z[n], acc);
-        }
-        double2 rho = bsum(acc, red);
-        while (it < maxit) {
-            apply_A<LOGN, LOGE, LOGRM>(g, p, T1, S, En, tid);          // w = A p in T1
-            acc = make_double2(0.0, 0.0);
-            for (int j = 0; j < E_; ++j) {
-                const int n = tid + j * T;
-                acc = cfma(p[n], T1[n], acc);
+        double2 rho = make_double2(0.0, 0.0);
+#pragma unroll 1
+        for (;;) {
+            const double2 rn = q.bsum(q.apply_P());                   // r^T z
+            double2 be = make_double2(0.0, 0.0);
+            if (it > 0) {
+                if (!(rho.x * rho.x + rho.y * rho.y > 0.0)) { st = SOFT_ERR_BREAKDOWN; break; }
+                be = cdiv(rn, rho);
             }
-            const double2 pw = bsum(acc, red);
-            if (!(pw.x * pw.x + pw.y * pw.y > 0.0)) { st = SOFT_ERR_BREAKDOWN; break; }
-            const double2 al = cdiv(rho, pw);
-            double rr = 0.0;
-            for (int j = 0; j < E_; ++j) {
-                const int n = tid + j * T;
-                x[n] = cfma(al, p[n], x[n]);
-                const double2 rv = csub(r[n], cmul(al, T1[n]));
-                r[n] = rv;
-                rr += rv.x * rv.x + rv.y * rv.y;
-            }
-            rr = bsum(make_double2(rr, 0.0), red).x;
-            ++it;
-            rel = sqrt(rr / ff);
-            if (!isfinite(rel)) { st = SOFT_ERR_NONFINITE; break; }
-            if (rel < tol) { st = SOFT_OK; break; }
-            apply_P<LOGN, LOGE, LOGRM>(g, r, z, S, T1, En, tid);
-            acc = make_double2(0.0, 0.0);
-            for (int j = 0; j < E_; ++j) {
-                const int n = tid + j * T;
-                acc = cfma(r[n], z[n], acc);
-            }
-            const double2 rn = bsum(acc, red);
-            if (!(rho.x * rho.x + rho.y * rho.y > 0.0)) { st = SOFT_ERR_BREAKDOWN; break; }
-            const double2 be = cdiv(rn, rho);
             rho = rn;
+            if (it >= maxit) break;
+#pragma unroll 2
             for (int j = 0; j < E_; ++j) {
                 const int n = tid + j * T;
                 p[n] = cfma(be, p[n], z[n]);
             }
             __syncthreads();
+            const double2 pw = q.bsum(q.apply_A(En));                 // z = w = A p
+            if (!(pw.x * pw.x + pw.y * pw.y > 0.0)) { st = SOFT_ERR_BREAKDOWN; break; }
+            const double2 al = cdiv(rho, pw), nal = make_double2(-al.x, -al.y);
+            double rr = 0.0;
+#pragma unroll 2
+            for (int j = 0; j < E_; ++j) {
+                const int n = tid + j * T;
+                x[n] = cfma(al, p[n], x[n]);
+                const double2 rv = cfma(nal, z[n], r[n]);
+                r[n] = rv;
+                rr += rv.x * rv.x + rv.y * rv.y;
+            }
+            rr = q.bsum(make_double2(rr, 0.0)).x;
+            ++it;
+            rel = sqrt(rr / ff);
+            if (!isfinite(rel)) { st = SOFT_ERR_NONFINITE; break; }
+            if (rel < tol) { st = SOFT_OK; break; }
         }
     }
     for (int j = 0; j < E_; ++j) {
@@ -236,60 +280,51 @@ sse1d_cocg_kernel(Sse1DGeo g, const double2* __restrict__ f, double2* __restrict
 }
 
 // one application: what = 0: y = A x; 1: y = P^-1 x
-template <int LOGN, int LOGE, int LOGRM>
-__global__ void __launch_bounds__(Cfg1D<double, LOGN, LOGE, LOGRM>::T, 1)
+template <int LOGN>
+__global__ void __launch_bounds__(Sse1<LOGN>::T, 1)
 sse1d_apply_kernel(Sse1DGeo g, const double2* __restrict__ in, double2* __restrict__ out, double En, int what)
 {
-    using K = Cfg1D<double, LOGN, LOGE, LOGRM>;
-    constexpr int N = K::N, T = K::T, E_ = K::E;
+    using Q = Sse1<LOGN>;
+    constexpr int T = Q::T, E_ = Q::E;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2* S = reinterpret_cast<double2*>(smem_raw);
-    double2* T1 = S + N;
-    double2* a = T1 + N;
-    double2* b = a + N;
     const int tid = threadIdx.x;
+    Q q(g, smem_raw, En, what != 0);
+    double2* a = what == 0 ? q.p : q.r;
     for (int j = 0; j < E_; ++j) a[tid + j * T] = in[tid + j * T];
     __syncthreads();
-    if (what == 0) apply_A<LOGN, LOGE, LOGRM>(g, a, b, S, En, tid);
-    else apply_P<LOGN, LOGE, LOGRM>(g, a, b, S, T1, En, tid);
-    for (int j = 0; j < E_; ++j) out[tid + j * T] = b[tid + j * T];
+    if (what == 0) q.apply_A(En);
+    else q.apply_P();
+    for (int j = 0; j < E_; ++j) out[tid + j * T] = q.z[tid + j * T];
 }
 
-template <int LOGN, int LOGE, int LOGRM>
+template <int LOGN>
 int launch_t(const Sse1DGeo& g, int mode, const double2* in, double2* out, const double* dE, double En, int nE,
              double tol, int maxit, int* iters, double* relres, int* status, cudaStream_t st) {
-    using K = Cfg1D<double, LOGN, LOGE, LOGRM>;
-    const size_t smem = sse1d_smem<LOGN, LOGE, LOGRM>();
-    static_assert(sse1d_smem<LOGN, LOGE, LOGRM>() <= 227 * 1024, "shared memory");
+    using Q = Sse1<LOGN>;
+    const int smem = (int)Q::SMEM;
     if (mode == 0) {
-        auto k = sse1d_cocg_kernel<LOGN, LOGE, LOGRM>;
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        auto k = sse1d_cocg_kernel<LOGN>;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
             return SOFT_ERR_CUDA;
-        if (nE > 0) k<<<nE, K::T, smem, st>>>(g, in, out, dE, tol, maxit, iters, relres, status);
+        if (nE > 0) k<<<nE, Q::T, smem, st>>>(g, in, out, dE, tol, maxit, iters, relres, status);
     } else {
-        auto k = sse1d_apply_kernel<LOGN, LOGE, LOGRM>;
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        auto k = sse1d_apply_kernel<LOGN>;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
             return SOFT_ERR_CUDA;
-        k<<<1, K::T, smem, st>>>(g, in, out, En, mode - 1);
+        k<<<1, Q::T, smem, st>>>(g, in, out, En, mode - 1);
     }
     return cudaGetLastError() == cudaSuccess ? SOFT_OK : SOFT_ERR_CUDA;
 }
 
-// the FFT configuration of each supported size (E a multiple of 4, radix 8)
-bool cfg_for(int logn, int* loge, int* logrm) {
-    if (logn < 8 || logn > 11) return false;
-    *loge = 3;
-    *logrm = 3;
-    return true;
-}
+constexpr int LOGRM1 = 3;              // radix 8, as PcgFx
 
 int launch(int logn, const Sse1DGeo& g, int mode, const double2* in, double2* out, const double* dE, double En,
            int nE, double tol, int maxit, int* iters, double* relres, int* status, cudaStream_t st) {
     switch (logn) {
-    case 8: return launch_t<8, 3, 3>(g, mode, in, out, dE, En, nE, tol, maxit, iters, relres, status, st);
-    case 9: return launch_t<9, 3, 3>(g, mode, in, out, dE, En, nE, tol, maxit, iters, relres, status, st);
-    case 10: return launch_t<10, 3, 3>(g, mode, in, out, dE, En, nE, tol, maxit, iters, relres, status, st);
-    case 11: return launch_t<11, 3, 3>(g, mode, in, out, dE, En, nE, tol, maxit, iters, relres, status, st);
+    case 8: return launch_t<8>(g, mode, in, out, dE, En, nE, tol, maxit, iters, relres, status, st);
+    case 9: return launch_t<9>(g, mode, in, out, dE, En, nE, tol, maxit, iters, relres, status, st);
+    case 10: return launch_t<10>(g, mode, in, out, dE, En, nE, tol, maxit, iters, relres, status, st);
+    case 11: return launch_t<11>(g, mode, in, out, dE, En, nE, tol, maxit, iters, relres, status, st);
     }
     return SOFT_ERR_UNSUPPORTED;
 }
@@ -298,7 +333,7 @@ int launch(int logn, const Sse1DGeo& g, int mode, const double2* in, double2* ou
 
 // Per-plan tables of the 1D solver, built on first use.
 struct Sse1D {
-    int logn = 0, loge = 0, logrm = 0, n = 0;
+    int logn = 0, n = 0;
     void *W = nullptr, *K = nullptr, *U = nullptr, *C = nullptr, *pos = nullptr;
     void* pc[2][5] = {};               // per preconditioner: bs, bw, xf, xb, lam
     double* dE = nullptr;
@@ -327,19 +362,15 @@ static int build(soft_plan* P) {
     std::unique_ptr<Sse1D> S(new Sse1D());
     S->n = TB.ax.n;
     S->logn = TB.logn;
-    if (!cfg_for(S->logn, &S->loge, &S->logrm)) return SOFT_ERR_UNSUPPORTED;
+    if (S->logn < 8 || S->logn > 11) return SOFT_ERR_UNSUPPORTED;
     const Axis1D& A = TB.ax;
     const int n = S->n;
     int rc;
-    if ((rc = upload_c(&S->W, pass_twiddles(S->logn, S->logrm), SOFT_C128))) return rc;
-    const std::vector<int> perm = dif_output_order(S->logn, S->logrm);
-    std::vector<cd> kt(n);
+    if ((rc = upload_i32(&S->W, pass_twiddles_fx(S->logn, LOGRM1, FXFULL_MAXS)))) return rc;
+    if ((rc = upload_ksq(&S->K, A, S->logn, LOGRM1))) return rc;
+    const std::vector<int> perm = dif_output_order(S->logn, LOGRM1);
     std::vector<int> pos(n);
-    for (int q = 0; q < n; ++q) {
-        kt[q] = 0.5 * A.k[perm[q]] * A.k[perm[q]] / n;
-        pos[perm[q]] = q;
-    }
-    if ((rc = upload_c(&S->K, kt, SOFT_C128))) return rc;
+    for (int q = 0; q < n; ++q) pos[perm[q]] = q;
     if ((rc = upload_int(&S->pos, pos))) return rc;
     if ((rc = upload_c(&S->U, TB.U0, SOFT_C128))) return rc;
     std::vector<cd> c = A.Cs;
@@ -350,25 +381,17 @@ static int build(soft_plan* P) {
         BandAxis B;
         double chk = 0;
         if ((rc = build_band_axis(A, P->opt.band_width, type == 0, B, &chk))) return rc;
-        int wmax = 1;
-        for (int wd : B.width) wmax = std::max(wmax, wd);
-        std::vector<cd> xf((size_t)wmax * n, 0.0), xb((size_t)wmax * n, 0.0);
-        for (int nu = 0; nu < n; ++nu)
-            for (int u = 0; u < B.width[nu]; ++u) {
-                xf[(size_t)u * n + nu] = B.xf[(size_t)B.off[nu] + u];
-                xb[(size_t)u * n + nu] = B.xb[(size_t)B.off[nu] + u];
-            }
         void** t = S->pc[type];
         if ((rc = upload_int(&t[0], B.start))) return rc;
         if ((rc = upload_int(&t[1], B.width))) return rc;
-        if ((rc = upload_c(&t[2], xf, SOFT_C128))) return rc;
-        if ((rc = upload_c(&t[3], xb, SOFT_C128))) return rc;
-        if ((rc = upload_c(&t[4], B.lam, SOFT_C128))) return rc;
         Sse1DGeo& g = S->geo[type];
-        g.W = (const double2*)S->W; g.K = (const double2*)S->K; g.U = (const double2*)S->U;
+        if ((rc = upload_band_fx(&t[2], B, B.xf, S->logn, LOGRM1, false, &g.pf))) return rc;
+        if ((rc = upload_band_fx(&t[3], B, B.xb, S->logn, LOGRM1, true, &g.pb))) return rc;
+        if ((rc = upload_c(&t[4], B.lam, SOFT_C128))) return rc;
+        g.W = (const int4*)S->W; g.K = (const double*)S->K; g.U = (const double2*)S->U;
         g.C = (const double2*)S->C; g.nb = TB.nb; g.blk0 = TB.blk0; g.pos = (const int*)S->pos;
-        g.bs = (const int*)t[0]; g.bw = (const int*)t[1]; g.xf = (const double2*)t[2];
-        g.xb = (const double2*)t[3]; g.lam = (const double2*)t[4];
+        g.bs = (const int*)t[0]; g.bw = (const int*)t[1]; g.xf = (const int4*)t[2];
+        g.xb = (const int4*)t[3]; g.lam = (const double2*)t[4];
     }
     P->s1 = S.release();
     return SOFT_OK;

@@ -46,3 +46,57 @@ def test_A_and_preconditioners(nx, ny, scale):
         assert torch.isnan(dy.real).all()
     finally:
         S.soft_destroy(plan)
+
+
+# tolerances of test_gpu_pcg1d: 1e-12 for A, 1e-11 for the preconditioners
+@pytest.mark.parametrize("n", [256, 512, 1024, 2048])
+@pytest.mark.parametrize("scale", [1.0, 1e-250, 1e200])
+def test_1d_A_and_preconditioners(n, scale):
+    hw, R0, th = 51.2 * n / 1024, 40.0 * n / 1024, 0.6
+    plan = S.soft_create(n, (-hw, hw), R0, th, 0.02, prec=S.SOFT_C128, contour=S.CONTOUR_SECS, soft_a2=2.0)
+    p = P.Problem1D(n, -hw, hw, R0, theta=th, kind=T.SECS, a2=2.0, dt=0.02)
+    st = ST.Stationary1D(p, nbw=10)
+    rng = np.random.default_rng(n)
+    x = rng.standard_normal(n) + 1j * rng.standard_normal(n)
+    x[n // 4:n // 2] *= 1e-9
+    try:
+        dx = torch.tensor(x * scale, dtype=torch.complex128, device="cuda")
+        dy = torch.zeros_like(dx)
+        get = lambda: dy.cpu().numpy() / scale    # noqa: E731
+        S.sse_apply_A(plan, 0.7, dx, dy)
+        assert _err(get(), st.apply_A(x, 0.7)) < 1e-12
+        for kind, ref in ((0, st.precond_simple), (1, st.precond_band)):
+            S.sse_apply_precond(plan, 0.7, kind, dx, dy)
+            assert _err(get(), ref(x, 0.7)) < 1e-11
+        dx[3] = float("nan")
+        S.sse_apply_precond(plan, 0.7, 1, dx, dy)
+        assert torch.isnan(dy.real).all()
+    finally:
+        S.soft_destroy(plan)
+
+
+@pytest.mark.parametrize("n,precond", [(256, 0), (256, 1), (2048, 1)])
+def test_1d_solve_of_a_scaled_source(n, precond):
+    """x is linear in f; a non-finite source is refused as before."""
+    hw, R0 = 51.2 * n / 1024, 40.0 * n / 1024
+    plan = S.soft_create(n, (-hw, hw), R0, 0.6, 0.02, prec=S.SOFT_C128, contour=S.CONTOUR_SECS, soft_a2=2.0)
+    p = P.Problem1D(n, -hw, hw, R0, theta=0.6, kind=T.SECS, a2=2.0, dt=0.02)
+    st = ST.Stationary1D(p, nbw=10)
+    f = np.exp(-(p.x - 1.0) ** 2 / 3.0 + 0.4j * p.x)
+    Es = [0.35, 1.2, 2.5]
+    try:
+        for scale in (1.0, 1e-60, 1e60):
+            out = torch.zeros((3, n), dtype=torch.complex128, device="cuda")
+            rc, its, rr = S.sse_pcg_solve(plan, Es, torch.tensor(f * scale, device="cuda"), out, tol=1e-10,
+                                          maxit=3000, precond=precond)
+            assert rc == 0
+            for e, E in enumerate(Es):
+                res = np.linalg.norm(f - st.apply_A(out[e].cpu().numpy() / scale, E)) / np.linalg.norm(f)
+                assert res < 2e-10
+        bad = torch.tensor(f, device="cuda")
+        bad[5] = float("inf")
+        with pytest.raises(S.SoftError) as err:
+            S.sse_pcg_solve(plan, Es, bad, out, tol=1e-10, maxit=30, precond=precond)
+        assert err.value.status == -8
+    finally:
+        S.soft_destroy(plan)
