@@ -33,12 +33,12 @@ struct PcgScr {
                                                          red(reinterpret_cast<unsigned*>(part + 16)) {}
 };
 
-template <int LOGN>
-struct PcgFx : LineFx<LOGN, 3, 3> {
-    using L = LineFx<LOGN, 3, 3>;
+template <int LOGN, int LR = 3>                  // radix 2^LR, a butterfly per thread
+struct PcgFx : LineFx<LOGN, LR, LR> {
+    using L = LineFx<LOGN, LR, LR>;
     using F = typename L::F;
     static constexpr int N = L::N, T = L::T, E = L::E;
-    static constexpr int NP = F::NPASS, R = PassGeom<LOGN, 3, NP - 1>::LOGR;    // bits of the last pass
+    static constexpr int NP = F::NPASS, R = PassGeom<LOGN, LR, NP - 1>::LOGR;    // bits of the last pass
     static constexpr int PITCH = N + 4;
     static constexpr size_t SMEM_A = sizeof(fx2) * (N + L::TWN) + L::SCR;
     static constexpr size_t SMEM_P = sizeof(fx2) * (2 * N + L::TWN) + L::SCR;
@@ -67,7 +67,7 @@ struct PcgFx : LineFx<LOGN, 3, 3> {
     template <class B>
     __device__ __forceinline__ static int center_k(fx2* S, const double* __restrict__ kt, PcgScr sc, int tid, B bar,
                                                    bool& bad) {
-        constexpr int RR = 1 << R, cs = (3 - R) / 2;
+        constexpr int RR = 1 << R, cs = (LR - R) / 2;
         double2 d[E];
 #pragma unroll
         for (int u = 0; u < E / RR; ++u) {
@@ -97,10 +97,10 @@ struct PcgFx : LineFx<LOGN, 3, 3> {
         }
         return e - R - cs;
     }
-    // first inverse pass, left as large as a pass of 3 bits leaves it (the
+    // first inverse pass, left as large as a pass of LR bits leaves it (the
     // tables before it carry the half bits)
     __device__ __forceinline__ static void inv_first(fx2* S, int tid) {
-        constexpr int RR = 1 << R, cs = (3 - R) / 2;
+        constexpr int RR = 1 << R, cs = (LR - R) / 2;
 #pragma unroll 1
         for (int u = 0; u < E / RR; ++u) {
             const int sb = swz<fx2>((tid + u * T) * RR);

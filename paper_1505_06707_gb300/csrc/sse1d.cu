@@ -13,10 +13,10 @@
 //
 // FFTs and the band products run in 64-bit fixed point (pcg_fix.cuh); the
 // vectors, k^2/2, the potential and strip terms, 1/(lambda - E) and the sums
-// are FP64.  In FP64 throughout an iteration took about 170
-// clocks of an SM per point, most of it in the FP64 pipe (2 instructions per
-// clock and SM); 38 FP64 instructions per point are left: 30 energies at
-// N = 1024, tolerance 1e-12, take 2.17 ms instead of 4.83.
+// are FP64.  In FP64 throughout, an iteration took about 170 clocks of an SM
+// per point, most of it in the FP64 pipe (2 instructions per clock and SM); 38
+// FP64 instructions per point are left.  30 energies at N = 1024, tolerance
+// 1e-12: 4.83 -> 2.17 ms, and 1.76 ms with radix 4 instead of radix 8.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -49,11 +49,15 @@ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
     return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
 }
 
+// an energy has an SM to itself and mostly waits for its own barriers, so more
+// threads (N/4) of smaller butterflies are faster
+constexpr int SSE1_LOGRM = 2;
+
 // One energy's CTA: S (the FFT buffer, swizzled), T1, x, r, p, z of N complex
 // each, the twiddles, scratch and two sets of warp sums
 template <int LOGN>
 struct Sse1 {
-    using Q = PcgFx<LOGN>;
+    using Q = PcgFx<LOGN, SSE1_LOGRM>;
     using F = typename Q::F;
     static constexpr int N = Q::N, T = Q::T, E = Q::E, NW = T / 32;
     static constexpr size_t SMEM = sizeof(fx2) * (6 * N + Q::TWN) + Q::SCR + sizeof(double2) * 2 * NW;
@@ -316,8 +320,6 @@ int launch_t(const Sse1DGeo& g, int mode, const double2* in, double2* out, const
     return cudaGetLastError() == cudaSuccess ? SOFT_OK : SOFT_ERR_CUDA;
 }
 
-constexpr int LOGRM1 = 3;              // radix 8, as PcgFx
-
 int launch(int logn, const Sse1DGeo& g, int mode, const double2* in, double2* out, const double* dE, double En,
            int nE, double tol, int maxit, int* iters, double* relres, int* status, cudaStream_t st) {
     switch (logn) {
@@ -366,9 +368,9 @@ static int build(soft_plan* P) {
     const Axis1D& A = TB.ax;
     const int n = S->n;
     int rc;
-    if ((rc = upload_i32(&S->W, pass_twiddles_fx(S->logn, LOGRM1, FXFULL_MAXS)))) return rc;
-    if ((rc = upload_ksq(&S->K, A, S->logn, LOGRM1))) return rc;
-    const std::vector<int> perm = dif_output_order(S->logn, LOGRM1);
+    if ((rc = upload_i32(&S->W, pass_twiddles_fx(S->logn, SSE1_LOGRM, FXFULL_MAXS)))) return rc;
+    if ((rc = upload_ksq(&S->K, A, S->logn, SSE1_LOGRM))) return rc;
+    const std::vector<int> perm = dif_output_order(S->logn, SSE1_LOGRM);
     std::vector<int> pos(n);
     for (int q = 0; q < n; ++q) pos[perm[q]] = q;
     if ((rc = upload_int(&S->pos, pos))) return rc;
@@ -385,8 +387,8 @@ static int build(soft_plan* P) {
         if ((rc = upload_int(&t[0], B.start))) return rc;
         if ((rc = upload_int(&t[1], B.width))) return rc;
         Sse1DGeo& g = S->geo[type];
-        if ((rc = upload_band_fx(&t[2], B, B.xf, S->logn, LOGRM1, false, &g.pf))) return rc;
-        if ((rc = upload_band_fx(&t[3], B, B.xb, S->logn, LOGRM1, true, &g.pb))) return rc;
+        if ((rc = upload_band_fx(&t[2], B, B.xf, S->logn, SSE1_LOGRM, false, &g.pf))) return rc;
+        if ((rc = upload_band_fx(&t[3], B, B.xb, S->logn, SSE1_LOGRM, true, &g.pb))) return rc;
         if ((rc = upload_c(&t[4], B.lam, SOFT_C128))) return rc;
         g.W = (const int4*)S->W; g.K = (const double*)S->K; g.U = (const double2*)S->U;
         g.C = (const double2*)S->C; g.nb = TB.nb; g.blk0 = TB.blk0; g.pos = (const int*)S->pos;
