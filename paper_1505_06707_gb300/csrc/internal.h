@@ -23,7 +23,7 @@ struct Inst1D {
     const void* TV;       // e^{-iU0 tau} off the strip block, e^{-iU0 tau/2} on it (minus 1 for complex64;
                           // complex128: FxV in soft1d_fix.cuh)
     const void* W;        // per-pass twiddles (complex64: bases, soft1d.cuh; complex128: FxGeom, soft1d_fix.cuh)
-    const void* cn;       // strip CN coefficients, chunk-transposed (soft1d.cuh, strip_cn_1d; complex128:
+    const void* cn;       // strip CN tables, chunk-transposed (soft1d.cuh, strip_cn; complex128:
                           // FxCn in soft1d_fix.cuh)
     const void* TVs;      // TV on the strip rows, same transposed order
     int nb;               // strip block length (0: no absorbing term)
@@ -34,13 +34,13 @@ struct Inst1D {
     int fcls;             // index of the pulse-shape class in that table
     int iL, iR;           // x_n <= -R0 for n < iL, x_n >= R0 for n >= iR
     int n;                // grid points
-    int pad_;
+    int cnr;              // complex64: scan extents of cn (strip_tables_c)
 };
 
 // Table set of one distinct 1D problem (shared by identical instances).
 struct Tables1D {
     int prec = 0, logn = 0, loge = 0, logrm = 0;
-    int nb = 0, blk0 = 0, iL = 0, iR = 0;
+    int nb = 0, blk0 = 0, iL = 0, iR = 0, cnr = 0;
     bool cn_gen = false;          // complex128: the strip solve is not fit for fixed point
     double R0 = 0, theta = 0;
     Axis1D ax;                    // host FP64 grid, contour, C

@@ -165,46 +165,37 @@ static bool fxv_gen(const std::vector<cd>& lv) {
     return false;
 }
 
-// Strip tables of the fixed-point step (soft1d_fix.cuh, FxCn) from the LU of
-// the block: thr threads of ch rows each.  gen: a multiplier above 1, a g
-// above 1.9 (its halves still fit, and the rows it scales are below 2^59.5)
-// or a growth of the sweeps above 2^10; the kernel then solves in FP64.
-std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vector<cd>& mb,
-                                            const std::vector<cd>& g, int nb, int thr, bool* gen) {
+// Chunked strip solve for thr threads of ch = ceil(nb/thr) rows (thread t: rows
+// t ch + c): multipliers mf and g in chunk order (c thr + t), and for the
+// forward and backward scans over the chunks the products of the chunk totals
+// (soft1d_fix.cuh, FxCn) with the numbers of warp-scan rounds and of warps
+// that still reach, where products below tiny count as zero.
+struct StripScan {
+    std::vector<cd> m, g, scan[2];
+    int rounds[2], span[2];
+};
+static StripScan strip_scan(const std::vector<cd>& mf, const std::vector<cd>& g, int nb, int thr, double tiny) {
     const int ch = (nb + thr - 1) / thr, nw = thr / 32;
-    const double tiny = 0x1p-70;
-    double grow = 1.0, gy = 0.0;
-    std::vector<double> y(nb);
-    *gen = false;
-    for (int i = 0; i < nb; ++i) {
-        gy = std::abs(mf[i]) * gy + 1.0;
-        y[i] = gy;
-        grow = std::max(grow, gy);
-        if (!(std::abs(mf[i]) <= 1.0 + 1e-12 && std::abs(g[i]) <= 1.9)) *gen = true;
-    }
-    double gx = 0.0;
-    for (int i = nb - 1; i >= 0; --i) {
-        gx = std::abs(mb[i]) * gx + std::abs(g[i]) * y[i];
-        grow = std::max(grow, gx);
-    }
-    const int lg = (int)std::ceil(std::log2(grow));
-    if (!(lg >= 0 && lg <= 10)) *gen = true;
-    std::vector<cd> m((size_t)(ch + 1) * thr, 0.0), gg((size_t)ch * thr, 0.0), scan[2];
+    StripScan Q;
+    Q.m.assign((size_t)(ch + 1) * thr, 0.0);
+    Q.g.assign((size_t)ch * thr, 0.0);
+    std::vector<cd> &m = Q.m, &gg = Q.g;
     for (int t = 0; t < thr; ++t)
         for (int c = 0; c <= ch; ++c) {
             const int i = t * ch + c;
             if (i < nb) m[(size_t)c * thr + t] = mf[i];
             if (c < ch && i < nb) gg[(size_t)c * thr + t] = g[i];
         }
-    int rounds[2], span[2];
     for (int d = 0; d < 2; ++d) {
-        std::vector<cd> tot(thr, 1.0);
-        for (int t = 0; t < thr; ++t)
+        std::vector<cd> tot(thr, 0.0);           // (0: chunks without rows, which carry nothing)
+        for (int t = 0; t < thr; ++t) {
+            if (t * ch < nb) tot[t] = 1.0;
             for (int c = 0; c < ch && t * ch + c < nb; ++c) tot[t] *= m[(size_t)(c + d) * thr + t];
-        std::vector<cd>& s = scan[d];
+        }
+        std::vector<cd>& s = Q.scan[d];
         s.assign((size_t)6 * thr + nw, 1.0);
         std::vector<cd> prod = tot;              // of the 2^r totals ending (starting) at t
-        rounds[d] = 0;
+        Q.rounds[d] = 0;
         for (int r = 0; r < 5; ++r) {
             const int D = 1 << r;
             double big = 0.0;
@@ -213,7 +204,7 @@ std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vecto
                 const int l = t & 31;
                 if (d ? l + D < 32 : l >= D) big = std::max(big, std::abs(prod[t]));
             }
-            if (big > tiny) rounds[d] = r + 1;
+            if (!(big <= tiny)) Q.rounds[d] = r + 1;
             std::vector<cd> nx = prod;
             for (int t = 0; t < thr; ++t) {
                 const int o = d ? t + D : t - D;
@@ -230,7 +221,7 @@ std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vecto
             }
             s[(size_t)6 * thr + w] = p;
         }
-        span[d] = nw;                            // warps whose totals still reach
+        Q.span[d] = nw;                            // warps whose totals still reach
         for (int k = 1; k < nw; ++k) {
             double big = 0.0;
             for (int w = 0; w + k <= nw; ++w) {
@@ -238,18 +229,55 @@ std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vecto
                 for (int q = 0; q < k; ++q) p *= s[(size_t)6 * thr + w + q];
                 big = std::max(big, std::abs(p));
             }
-            if (big <= tiny) { span[d] = k; break; }
+            if (big <= tiny) { Q.span[d] = k; break; }
         }
     }
+    return Q;
+}
+// the tables of a complex64 strip solve (soft1d.cuh, strip_cn); cnr: rounds of
+// the forward and backward scans (4 bits each), their spans (8 bits each), also
+// the first two entries
+std::vector<cd> strip_tables_c(const std::vector<cd>& mf, const std::vector<cd>& g, int nb, int thr, int* cnr) {
+    const StripScan Q = strip_scan(mf, g, nb, thr, 0x1p-40);
+    *cnr = Q.rounds[0] | Q.rounds[1] << 4 | Q.span[0] << 8 | Q.span[1] << 16;
+    std::vector<cd> t = {cd(Q.rounds[0], Q.rounds[1]), cd(Q.span[0], Q.span[1])};
+    for (const std::vector<cd>* v : {&Q.m, &Q.g, &Q.scan[0], &Q.scan[1]}) t.insert(t.end(), v->begin(), v->end());
+    return t;
+}
+
+// Strip tables of the fixed-point step (soft1d_fix.cuh, FxCn) from the LU of
+// the block: thr threads of ch rows each.  gen: a multiplier above 1, a g
+// above 1.9 (its halves still fit, and the rows it scales are below 2^59.5)
+// or a growth of the sweeps above 2^10; the kernel then solves in FP64.
+std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vector<cd>& mb,
+                                            const std::vector<cd>& g, int nb, int thr, bool* gen) {
+    double grow = 1.0, gy = 0.0;
+    std::vector<double> y(nb);
+    *gen = false;
+    for (int i = 0; i < nb; ++i) {
+        gy = std::abs(mf[i]) * gy + 1.0;
+        y[i] = gy;
+        grow = std::max(grow, gy);
+        if (!(std::abs(mf[i]) <= 1.0 + 1e-12 && std::abs(g[i]) <= 1.9)) *gen = true;
+    }
+    double gx = 0.0;
+    for (int i = nb - 1; i >= 0; --i) {
+        gx = std::abs(mb[i]) * gx + std::abs(g[i]) * y[i];
+        grow = std::max(grow, gx);
+    }
+    const int lg = (int)std::ceil(std::log2(grow));
+    if (!(lg >= 0 && lg <= 10)) *gen = true;
+    const StripScan Q = strip_scan(mf, g, nb, thr, 0x1p-70);
+    const std::vector<cd> &m = Q.m, &gg = Q.g;
     std::vector<cd> all = m;
     all.insert(all.end(), gg.begin(), gg.end());
-    all.insert(all.end(), scan[0].begin(), scan[0].end());
-    all.insert(all.end(), scan[1].begin(), scan[1].end());
+    all.insert(all.end(), Q.scan[0].begin(), Q.scan[0].end());
+    all.insert(all.end(), Q.scan[1].begin(), Q.scan[1].end());
     std::vector<int32_t> buf(4 + 4 * (all.size() + m.size() + gg.size()), 0);
     buf[0] = *gen ? 0 : lg;
-    buf[1] = rounds[0];
-    buf[2] = rounds[1];
-    buf[3] = span[0] | span[1] << 16;
+    buf[1] = Q.rounds[0];
+    buf[2] = Q.rounds[1];
+    buf[3] = Q.span[0] | Q.span[1] << 16;
     if (!*gen) {
         std::vector<int32_t> f(4 * all.size());
         fx_fill(f.data(), all, 1.0);
@@ -416,11 +444,8 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
         tkh[q] = std::polar(1.0 / n, phh[q]);
     }
     potential_logs_1d(*T, n, tau, tv, tvs);
-    // Strip CN coefficients for the kernel's chunked solve: thread t of the
-    // T = n >> loge threads owns rows t*ch .. t*ch + ch - 1 (ch = ceil(nb/T)).
-    // M is complex symmetric, so mb_i = mf_{i+1}: the kernel reads mf of rows
-    // t*ch + c, c <= ch, at c*T + t (0 past the block), then g of row t*ch + c
-    // at (ch+1)*T + c*T + t (tvs holds the rows' potential factors).
+    // Strip CN tables of the T = n >> loge threads; M is complex symmetric, so
+    // mb_i = mf_{i+1} (tvs holds the rows' potential factors in chunk order)
     std::vector<cd> mf, mb, g, cnv;
     std::vector<int32_t> cnfx;
     if (T->nb > 0) {
@@ -431,14 +456,7 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
         for (int i = 0; i + 1 < nb; ++i)
             if (std::abs(mb[i] - mf[i + 1]) > 1e-12 * (std::abs(mb[i]) + 1e-300)) return SOFT_ERR_SETUP;
         if (o.prec == SOFT_C128) cnfx = strip_tables_fx(mf, mb, g, nb, thr, &T->cn_gen);
-        const int ch = (nb + thr - 1) / thr, P1 = (ch + 1) * thr;
-        cnv.assign((size_t)P1 + (size_t)ch * thr, 0.0);
-        for (int t = 0; t < thr; ++t)
-            for (int c = 0; c <= ch; ++c) {
-                const int i = t * ch + c;
-                if (i < nb) cnv[(size_t)c * thr + t] = mf[i];
-                if (c < ch && i < nb) cnv[P1 + (size_t)c * thr + t] = g[i];
-            }
+        else cnv = strip_tables_c(mf, g, nb, thr, &T->cnr);
     }
     if (o.prec == SOFT_C128) {
         const bool gen = T->cn_gen || fxv_gen(tv);
@@ -549,7 +567,7 @@ static int autotune_size(const soft_options& o, int n, double a, double b, doubl
                 for (int i = 0; i < ns; ++i) {
                     std::memset(&d[i], 0, sizeof(Inst1D));
                     d[i].off = (int64_t)i * n;
-                    d[i].TK = T.TK; d[i].TKh = T.TKh; d[i].TV = T.TV; d[i].W = T.W; d[i].cn = T.cn;
+                    d[i].TK = T.TK; d[i].TKh = T.TKh; d[i].TV = T.TV; d[i].W = T.W; d[i].cn = T.cn; d[i].cnr = T.cnr;
                     d[i].TVs = T.TVs;
                     d[i].nb = T.nb; d[i].blk0 = T.blk0; d[i].x0 = T.ax.x[0]; d[i].h = T.ax.h;
                     d[i].R0 = R0; d[i].tau = dt; d[i].iL = T.iL; d[i].iR = T.iR; d[i].n = n;
@@ -843,7 +861,7 @@ Inst1D soft_plan::descriptor(int i) const {
     Inst1D d;
     std::memset(&d, 0, sizeof(d));
     d.off = ih.off;
-    d.TK = T.TK; d.TKh = T.TKh; d.TV = T.TV; d.W = T.W; d.cn = T.cn; d.TVs = T.TVs;
+    d.TK = T.TK; d.TKh = T.TKh; d.TV = T.TV; d.W = T.W; d.cn = T.cn; d.cnr = T.cnr; d.TVs = T.TVs;
     d.nb = T.nb; d.blk0 = T.blk0;
     d.x0 = T.ax.x[0]; d.h = T.ax.h; d.R0 = T.R0; d.tau = dt;
     d.E0 = ih.E0; d.has_field = ih.has_field; d.fcls = ih.fcls;

@@ -47,7 +47,7 @@ int Plan2D::row(int mode, void* psi, const void* tkx, cudaStream_t st) {
 }
 int Plan2D::col(int mode, void* psi, const void* tky, cudaStream_t st) {
     ++launches;
-    const LineGeo lg{geo.Wy, geo.nx, 0, geo.cny, geo.TVh, geo.nby, geo.blk0y, 0, 1, 0, 0, geo.vmeta};
+    const LineGeo lg{geo.Wy, geo.nx, 0, geo.cny, geo.TVh, geo.nby, geo.blk0y, 0, 1, 0, 0, geo.vmeta, geo.cnry};
     if (prec == SOFT_C64) return soft2d_col_c64(ly, ley, lry, mode, lg, 1, psi, tky, st);
     return soft2d_col_c128(ly, ley, lry, mode, lg, 1, psi, tky, st);
 }
@@ -134,16 +134,10 @@ int create_2d(const soft_grid* grid, const double* box, double R0, double theta,
         for (int q = 0; q < A.n; ++q) t[q] = std::polar(1.0 / A.n, ph[q]);
         return upload_tab(dst, t, pr);
     };
-    std::vector<cd> mfx, mbx, gx, mfy, mby, gy, cnx, cny;
+    std::vector<cd> mfx, mbx, gx, mfy, mby, gy;
     double err;
-    if (nbx > 0) {
-        if ((rc = strip_factor(Q->ax, bx0, nbx, mfx, mbx, gx, &err))) return rc;
-        cnx = mfx; cnx.insert(cnx.end(), mbx.begin(), mbx.end()); cnx.insert(cnx.end(), gx.begin(), gx.end());
-    }
-    if (nby > 0) {
-        if ((rc = strip_factor(Q->ay, by0, nby, mfy, mby, gy, &err))) return rc;
-        cny = mfy; cny.insert(cny.end(), mby.begin(), mby.end()); cny.insert(cny.end(), gy.begin(), gy.end());
-    }
+    if (nbx > 0 && (rc = strip_factor(Q->ax, bx0, nbx, mfx, mbx, gx, &err))) return rc;
+    if (nby > 0 && (rc = strip_factor(Q->ay, by0, nby, mfy, mby, gy, &err))) return rc;
     // pass twiddles: the four bases per pass (complex64), fixed-point factors (complex128)
     auto twid = [&](void** d, int logn, int logrm) {
         return pr == SOFT_C128 ? upload_i32(d, pass_twiddles_fx(logn, logrm, FXFULL_MAXS))
@@ -163,8 +157,8 @@ int create_2d(const soft_grid* grid, const double* box, double R0, double theta,
         if ((rc = Q->fxv.build(tvh))) return rc;
     } else {
         if ((rc = upload_vtab(&Q->TVh, tvh, pr))) return rc;
-        if ((rc = upload_c(&Q->cnx, cnx, pr))) return rc;
-        if ((rc = upload_c(&Q->cny, cny, pr))) return rc;
+        if (nbx > 0 && (rc = upload_c(&Q->cnx, strip_tables_c(mfx, gx, nbx, thr, &Q->geo.cnrx), pr))) return rc;
+        if (nby > 0 && (rc = upload_c(&Q->cny, strip_tables_c(mfy, gy, nby, (int)(ny >> Q->ley), &Q->geo.cnry), pr))) return rc;
     }
     Geo2D& g = Q->geo;
     g.Wx = Q->Wx; g.Wy = Q->Wy; g.TVh = pr == SOFT_C128 ? Q->fxv.tab : Q->TVh; g.cnx = Q->cnx; g.cny = Q->cny;

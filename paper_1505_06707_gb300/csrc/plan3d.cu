@@ -100,7 +100,7 @@ int Plan3D::line(int d, int mode, void* psi, const void* tk, cudaStream_t st) {
     // z lines (c = y nx + x): V/2 off the z-strip block only on lines with y
     // in the y-strip block (the row pass applied it on the others)
     const LineGeo lg{W[d], d == 1 ? nx : nx * ny, d == 1 ? nx * ny : 0, cn[d], geo.TVh, nb[d], blk0[d],
-                     d == 2 ? nx : 0, n[1], nb[1], blk0[1], geo.vmeta};
+                     d == 2 ? nx : 0, n[1], nb[1], blk0[1], geo.vmeta, cnr[d]};
     const int planes = d == 1 ? n[2] : 1;
     if (prec == SOFT_C64) return soft2d_col_c64(l[d], le[d], lr[d], mode, lg, planes, psi, tk, st);
     return soft2d_col_c128(l[d], le[d], lr[d], mode, lg, planes, psi, tk, st);
@@ -215,6 +215,10 @@ int create_3d(const soft_grid* grid, const double* box, double R0, double theta,
                 Q->fxv.cn_gen = Q->fxv.cn_gen || gen;
                 continue;
             }
+            if (d != 1) {
+                if ((rc = upload_c(&Q->cn[d], strip_tables_c(mf, g, Q->nb[d], Q->n[d] >> Q->le[d], &Q->cnr[d]), pr))) return rc;
+                continue;
+            }
             mf.insert(mf.end(), mb.begin(), mb.end());
             mf.insert(mf.end(), g.begin(), g.end());
             if ((rc = upload_c(&Q->cn[d], mf, pr))) return rc;
@@ -226,7 +230,7 @@ int create_3d(const soft_grid* grid, const double* box, double R0, double theta,
     }
     Geo2D& g = Q->geo;
     std::memset(&g, 0, sizeof(g));
-    g.Wx = Q->W[0]; g.TVh = pr == SOFT_C128 ? Q->fxv.tab : Q->TVh; g.cnx = Q->cn[0];
+    g.Wx = Q->W[0]; g.TVh = pr == SOFT_C128 ? Q->fxv.tab : Q->TVh; g.cnx = Q->cn[0]; g.cnrx = Q->cnr[0];
     g.vmeta = Q->fxv.meta;
     g.nx = Q->n[0]; g.ny = Q->n[1] * Q->n[2];
     g.nbx = Q->nb[0]; g.blk0x = Q->blk0[0];

@@ -37,6 +37,7 @@ int upload_fx_phases(void** dst, const std::vector<double>& ph, int half);
 int upload_i32(void** dst, const std::vector<int32_t>& v);
 std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vector<cd>& mb, const std::vector<cd>& g,
                                      int nb, int thr, bool* gen);
+std::vector<cd> strip_tables_c(const std::vector<cd>& mf, const std::vector<cd>& g, int nb, int thr, int* cnr);
 // fn(begin, end) over 0 .. n - 1 on host threads (the calling one if none can start)
 void host_parallel(int64_t n, const std::function<void(int64_t, int64_t)>& fn);
 // Potential factors of a complex128 2D or 3D plan: factors e^{lv} 2^-p
@@ -124,6 +125,7 @@ struct Plan3D {
     Axis1D ax[3];
     std::vector<cd> ua[3];         // comparison-absorber potential of each axis
     void *W[3] = {}, *TK[3] = {}, *TKh[3] = {}, *TVh = nullptr, *cn[3] = {};
+    int cnr[3] = {};
     FxPotential fxv;               // complex128 (instead of TVh)
     Geo2D geo{};
     int64_t launches = 0, graph_launches = 0;

@@ -290,135 +290,160 @@ __device__ __forceinline__ void kmul(typename CT<R>::C* S, const typename TabT<R
     __syncthreads();
 }
 
-// Crank-Nicolson factor on the strip block (Sec. II, CN form of e^{-iC tau}):
-// with M = 1 + i tau C/2 factored on the host (no pivoting) into the
-// recurrences y_i = mf_i y_{i-1} + r_i and x_i = mb_i x_{i+1} + g_i y_i, the
-// block rows r_i = S[(blk0 + i) mod N] become post(n, 2 x_i - r_i), which is
-// (1 + i tau C/2)^{-1} (1 - i tau C/2) r.  Each thread runs a contiguous chunk
-// of rows; the chunks are joined by block-wide scans of the affine maps.
-// cn holds mf[nb], mb[nb], g[nb].  All T threads must call.
-template <typename C, int T, int CMAX, int N, class Post>
-__device__ __forceinline__ void strip_cn(C* S, const C* __restrict__ cn, int nb, int blk0, int tid,
-                                         C* scan, Post post) {
-    const int chunk = (nb + T - 1) / T;          // host guarantees chunk <= CMAX
-    const int i0 = tid * chunk;
-    C y[CMAX];
-    C Mp; Mp.x = 1; Mp.y = 0;
-    C yl; yl.x = 0; yl.y = 0;
-#pragma unroll
-    for (int c = 0; c < CMAX; ++c) {
-        const int i = i0 + c;
-        if (c < chunk && i < nb) {
-            const C rc = S[swz<C>((blk0 + i) & (N - 1))];
-            const C m = __ldg(&cn[i]);
-            yl = cfma(m, yl, rc);
-            Mp = cmul(m, Mp);
-            y[c] = yl;
-        }
-    }
-    C carry = affine_carry<C, T, false>(Mp, yl, scan, tid);
-    {
-        C pr; pr.x = 1; pr.y = 0;
-#pragma unroll
-        for (int c = 0; c < CMAX; ++c) {
-            const int i = i0 + c;
-            if (c < chunk && i < nb) {
-                pr = cmul(__ldg(&cn[i]), pr);
-                y[c] = cfma(pr, carry, y[c]);
-            }
-        }
-    }
-    Mp.x = 1; Mp.y = 0;
-    C xl; xl.x = 0; xl.y = 0;
-#pragma unroll
-    for (int c = CMAX - 1; c >= 0; --c) {
-        const int i = i0 + c;
-        if (c < chunk && i < nb) {
-            const C m = __ldg(&cn[nb + i]);
-            const C g = __ldg(&cn[2 * nb + i]);
-            xl = cfma(m, xl, cmul(g, y[c]));
-            Mp = cmul(m, Mp);
-            y[c] = xl;
-        }
-    }
-    carry = affine_carry<C, T, true>(Mp, xl, scan, tid);
-    C pr; pr.x = 1; pr.y = 0;
-#pragma unroll
-    for (int c = CMAX - 1; c >= 0; --c) {
-        const int i = i0 + c;
-        if (c < chunk && i < nb) {
-            pr = cmul(__ldg(&cn[nb + i]), pr);
-            const C xv = cfma(pr, carry, y[c]);
-            const int n = (blk0 + i) & (N - 1);
-            const C rc = S[swz<C>(n)];
-            S[swz<C>(n)] = post(n, cmk<C>(2 * xv.x - rc.x, 2 * xv.y - rc.y));
-        }
-    }
-}
+// Crank-Nicolson factor on the strip block (Sec. II, CN form of e^{-iC tau}),
+// complex64.  With M = 1 + i tau C/2 factored on the host (no pivoting) into
+// the recurrences y_i = mf_i y_{i-1} + r_i and x_i = mb_i x_{i+1} + g_i y_i,
+// the block rows r_i = S[(blk0 + i) mod N] become post(v, c, n),
+// v = 2 x_i - r_i, which is (1 + i tau C/2)^{-1} (1 - i tau C/2) r (c: the row's
+// place in its thread's chunk, n: its grid index).  M is complex symmetric (C
+// is, Sec. II), so mb_i = mf_{i+1}.  Each thread runs a contiguous chunk of ch
+// rows, each sweep twice: with carry 0, for the chunk's constant part, and with
+// the carry that a scan over the chunks gives.
+//
+// Tables (host: strip_tables_c, chunk order, coalesced): (rounds, span) of the
+// two scans, mf of rows t ch + c, c <= ch, at c T + t, g, then
+// per scan the products [5][T] of the 2^r chunk totals that end (start) at t,
+// the exclusive product of t's warp [T] and the warp totals [T/32].  The
+// multipliers decay (|mf| = 0.1 to 0.9 on the workloads' strips), so rounds of
+// the warp scan and warps whose products are below 2^-40 are left out: FP32
+// results round 2^16 times coarser.
+//
+// Against scans that formed the products in the kernel, with uncoalesced
+// coefficients in the line passes: 12.06 -> 11.74 ms for the 4096-instance laser
+// batch, 85.2 -> 82.7 us per step at 2048^2, 491 -> 476 at 256^3.
 
-// The same solve for the 1D step kernel.  M is complex symmetric (C is,
-// Sec. II), so mb_i = mf_{i+1} and one multiplier array serves both sweeps.
-// The host lays the coefficients out for coalesced reads: thread t owns rows
-// i0 = t*ch .. i0 + ch - 1 (ch = ceil(nb/T)); cn[c*T + t] = mf_{i0+c} for
-// c <= ch (0 past the block), cn[(ch+1)*T + c*T + t] = g_{i0+c}, and
-// tvs[c*T + t] = TV at row i0 + c.  Every coefficient is read once, before
-// the sweep that uses it; the in-chunk products of the carry corrections are
-// formed from registers.  post(n, tv, v) gets the row's grid index and potential.
-template <typename C, typename VT, int T, int CMAX, int N, class Post, class B = BarCTA>
-__device__ __forceinline__ void strip_cn_1d(C* S, const C* __restrict__ cn, const VT* __restrict__ tvs,
-                                            int nb, int blk0, int tid, C* scan, Post post, B bar = B()) {
+// the thread's products of a scan
+template <int T>
+struct StripScanTab {
+    float2 p[5], ex;
+    __device__ __forceinline__ void load(const float2* __restrict__ tab, int rounds, int tid) {
+#pragma unroll
+        for (int r = 0; r < 5; ++r)
+            if (r < rounds) p[r] = __ldg(&tab[r * T + tid]);
+        if constexpr (T > 32) ex = __ldg(&tab[5 * T + tid]);
+    }
+};
+// carry that enters this thread's chunk.  scratch: T/32 values; AHEAD: s is loaded
+template <int T, bool REV, bool AHEAD, class B>
+__device__ __forceinline__ float2 strip_carry(float2 Y, StripScanTab<T>& s, const float2* __restrict__ tab,
+                                              int rounds, int span, float2* scratch, int tid, B bar) {
+    constexpr int NW = T / 32;
+    const int lane = tid & 31, warp = tid >> 5;
+    auto shift = [&](float2 v, int d) {
+        return REV ? make_float2(__shfl_down_sync(0xffffffffu, v.x, d), __shfl_down_sync(0xffffffffu, v.y, d))
+                   : make_float2(__shfl_up_sync(0xffffffffu, v.x, d), __shfl_up_sync(0xffffffffu, v.y, d));
+    };
+    if constexpr (!AHEAD && NW > 1) s.ex = __ldg(&tab[5 * T + tid]);
+#pragma unroll
+    for (int r = 0; r < 5; ++r) {
+        if (r < rounds) {
+            const float2 p = AHEAD ? s.p[r] : __ldg(&tab[r * T + tid]);
+            const float2 o = shift(Y, 1 << r);
+            if (REV ? lane + (1 << r) < 32 : lane >= (1 << r)) Y = cfma(p, o, Y);
+        }
+    }
+    float2 ex = shift(Y, 1);
+    if (lane == (REV ? 31 : 0)) ex = make_float2(0.0f, 0.0f);
+    if constexpr (NW > 1) {
+        if (lane == (REV ? 0 : 31)) scratch[warp] = Y;
+        bar.sync();
+        if (REV ? warp + 1 < NW : warp > 0) {
+            // the warps before this one, farthest first
+            const int k = min(span, REV ? NW - 1 - warp : warp);
+            const int w0 = REV ? warp + k : warp - k;
+            float2 c = scratch[w0];
+#pragma unroll 1
+            for (int q = 1; q < k; ++q) {
+                const int w = REV ? w0 - q : w0 + q;
+                c = cfma(__ldg(&tab[6 * T + w]), c, scratch[w]);
+            }
+            ex = cfma(s.ex, c, ex);
+        }
+    }
+    return ex;
+}
+// all of a thread's coefficients, for kernels that keep them over many steps
+// (resident: 4 elements per thread)
+template <int T, int CMAX>
+struct StripRegs {
+    float2 m[CMAX + 1], g[CMAX];
+    StripScanTab<T> f, b;
+    __device__ __forceinline__ void load(const float2* __restrict__ cn, int cnr, int nb, int tid) {
+        const int ch = (nb + T - 1) / T;
+        const float2* __restrict__ gt = cn + 2 + (ch + 1) * T;
+#pragma unroll
+        for (int c = 0; c <= CMAX; ++c)
+            if (c <= ch) m[c] = __ldg(&cn[2 + c * T + tid]);
+#pragma unroll
+        for (int c = 0; c < CMAX; ++c)
+            if (c < ch) g[c] = __ldg(&gt[c * T + tid]);
+        f.load(gt + ch * T, cnr & 15, tid);
+        b.load(gt + (ch + 6) * T + T / 32, (cnr >> 4) & 15, tid);
+    }
+};
+// scan: 32 complex of scratch.  AHEAD: cnr gives rounds and spans, and the
+// scans' products are requested before the sweeps that lead to them (line
+// passes, which solve once per CTA, and 1D steps of up to 8 elements per thread;
+// at 16 and 32 that costs more in spills than the waits: 11.7 -> 12.2 ms for the
+// laser batch)
+template <int T, int CMAX, int N, bool AHEAD, class Post, class B = BarCTA, bool RES = false>
+__device__ __forceinline__ void strip_cn(float2* S, const float2* __restrict__ cn, int cnr, int nb, int blk0, int tid,
+                                         float2* scan, Post post, B bar = B(), const StripRegs<T, CMAX>* res = nullptr) {
+    using C = float2;
+    static_assert(T / 32 <= 16, "scratch");
     const int ch = (nb + T - 1) / T;             // host guarantees ch <= CMAX
-    const int P1 = (ch + 1) * T;
     const int i0 = tid * ch;
     const int nv = min(ch, nb - i0);             // rows of this thread (may be <= 0)
+    int rf = cnr & 15, rb = (cnr >> 4) & 15, kf = (cnr >> 8) & 255, kb = cnr >> 16;
+    if constexpr (!AHEAD) {                      // (not held in registers across the steps)
+        const float2 r = __ldg(&cn[0]), k = __ldg(&cn[1]);
+        rf = (int)r.x; rb = (int)r.y; kf = (int)k.x; kb = (int)k.y;
+    }
+    cn += 2;
+    const float2* __restrict__ g = cn + (ch + 1) * T;
+    const float2* __restrict__ sf = g + ch * T;
+    const float2* __restrict__ sb = sf + 6 * T + T / 32;
     C y[CMAX], m[CMAX + 1];
+    StripScanTab<T> tf, tb;
+    if constexpr (RES) {
 #pragma unroll
-    for (int c = 0; c <= CMAX; ++c)
-        if (c <= ch) m[c] = __ldg(&cn[c * T + tid]);
-    C Mp; Mp.x = 1; Mp.y = 0;
-    C yl; yl.x = 0; yl.y = 0;
+        for (int c = 0; c <= CMAX; ++c) m[c] = res->m[c];
+        tf = res->f;
+        tb = res->b;
+    } else {
 #pragma unroll
-    for (int c = 0; c < CMAX; ++c) {
-        if (c < nv) {
-            const C rc = S[swz<C>((blk0 + i0 + c) & (N - 1))];
-            yl = cfma(m[c], yl, rc);
-            Mp = cmul(m[c], Mp);
-            y[c] = yl;
-        }
+        for (int c = 0; c <= CMAX; ++c)
+            if (c <= ch) m[c] = __ldg(&cn[c * T + tid]);
+        if constexpr (AHEAD) tf.load(sf, rf, tid);
     }
-    C carry = affine_carry<C, T, false>(Mp, yl, scan, tid, bar);
-    {
-        C pr; pr.x = 1; pr.y = 0;
+    C l = cmk<C>(0, 0);
 #pragma unroll
-        for (int c = 0; c < CMAX; ++c) {
-            if (c < nv) {
-                pr = cmul(m[c], pr);
-                y[c] = cfma(pr, carry, y[c]);
-            }
-        }
-    }
-    Mp.x = 1; Mp.y = 0;
-    C xl; xl.x = 0; xl.y = 0;
-#pragma unroll
-    for (int c = CMAX - 1; c >= 0; --c) {
+    for (int c = 0; c < CMAX; ++c)
         if (c < nv) {
-            xl = cfma(m[c + 1], xl, cmul(__ldg(&cn[P1 + c * T + tid]), y[c]));
-            Mp = cmul(m[c + 1], Mp);
-            y[c] = xl;
+            y[c] = S[swz<C>((blk0 + i0 + c) & (N - 1))];
+            l = cfma(m[c], l, y[c]);
         }
-    }
-    carry = affine_carry<C, T, true>(Mp, xl, scan, tid, bar);
-    C pr; pr.x = 1; pr.y = 0;
+    if constexpr (AHEAD && !RES) tb.load(sb, rb, tid);
+    l = strip_carry<T, false, AHEAD>(l, tf, sf, rf, kf, scan, tid, bar);
 #pragma unroll
-    for (int c = CMAX - 1; c >= 0; --c) {
+    for (int c = 0; c < CMAX; ++c)
         if (c < nv) {
-            pr = cmul(m[c + 1], pr);
-            const C xv = cfma(pr, carry, y[c]);
+            l = cfma(m[c], l, y[c]);
+            y[c] = cmul(RES ? res->g[c] : __ldg(&g[c * T + tid]), l);
+        }
+    l = cmk<C>(0, 0);
+#pragma unroll
+    for (int c = CMAX - 1; c >= 0; --c)
+        if (c < nv) l = cfma(m[c + 1], l, y[c]);
+    l = strip_carry<T, true, AHEAD>(l, tb, sb, rb, kb, scan + 16, tid, bar);
+#pragma unroll
+    for (int c = CMAX - 1; c >= 0; --c)
+        if (c < nv) {
+            l = cfma(m[c + 1], l, y[c]);
             const int n = (blk0 + i0 + c) & (N - 1);
-            const C rc = S[swz<C>(n)];
-            S[swz<C>(n)] = post(n, __ldg(&tvs[c * T + tid]), cmk<C>(2 * xv.x - rc.x, 2 * xv.y - rc.y));
+            C& r = S[swz<C>(n)];
+            r = post(cmk<C>(2 * l.x - r.x, 2 * l.y - r.y), c, n);
         }
-    }
 }
 
 __device__ __forceinline__ void sincos_r(float a, float* s, float* c) { sincosf(a, s, c); }
@@ -710,14 +735,20 @@ __device__ __forceinline__ void soft1d_run(const Inst1D& I, void* __restrict__ p
     // ends with the potential factor of the next step, applied as the last
     // inverse FFT pass stores (none after the final half-kinetic factor).
     R al = 0;
+    StripRegs<T, K::CMAX> sr;                    // (E <= 4)
+    if constexpr (E <= 4) {
+        if (nb > 0) sr.load(cn, I.cnr, nb, tid);
+    }
     for (int64_t step = -1; step < nsteps; ++step) {
         // ---- Crank-Nicolson on the strip block, then the second e^{-iU tau/2}
         if (step >= 0 && nb > 0) {
-            strip_cn_1d<C, VT, T, K::CMAX, N>(S, cn, TVs, nb, blk0, tid, scan, [&](int n, const VT& tv, C v) {
-                v = vmul(v, tv);
+            auto post = [&](C v, int c, int n) {
+                v = vmul(v, __ldg(&TVs[c * T + tid]));
                 if (I.has_field) v = cmul(v, strip_field<R, C, E>(fr, al, I, n));
                 return v;
-            }, bar);
+            };
+            strip_cn<T, K::CMAX, N, E <= 8, decltype(post), B, E <= 4>(S, cn, I.cnr, nb, blk0, tid, scan, post, bar,
+                                                                       &sr);
             bar.sync();
         }
         // ---- kinetic: forward FFT, e^{-iK tau} (e^{-iK tau/2} in the first

@@ -122,8 +122,8 @@ row_pass_kernel(Geo2D g, void* __restrict__ psi_v, const void* __restrict__ tkx_
         inv_pass0_post<R, LOGN, LOGE, LOGRM, true>(S, Ws, tid, [&](int n, C v) { return vmul(v, Tv[n]); });
         __syncthreads();
         if (g.nbx > 0) {
-            strip_cn<C, T, K::CMAX, N>(S, reinterpret_cast<const C*>(g.cnx), g.nbx, g.blk0x, tid, scan,
-                                       [](int, C v) { return v; });
+            strip_cn<T, K::CMAX, N, true>(S, reinterpret_cast<const C*>(g.cnx), g.cnrx, g.nbx, g.blk0x, tid, scan,
+                                    [](C v, int, int) { return v; });
             __syncthreads();
         }
     }
@@ -244,8 +244,8 @@ col_pass_kernel(LineGeo lg, void* __restrict__ psi_v, const void* __restrict__ t
         if (lg.nb > 0) {
             const VT* tvc = Tvs + col * CC::VCAP;
             C* scan = reinterpret_cast<C*>(smem_raw + CC::OFF_SCAN) + 32 * col;
-            strip_cn<C, T, K::CMAX, N>(Sc, reinterpret_cast<const C*>(lg.cn), lg.nb, lg.blk0, tid, scan,
-                                       [&](int n, C v) { return vmul(v, tvc[(n - lg.blk0) & (N - 1)]); });
+            strip_cn<T, K::CMAX, N, true>(Sc, reinterpret_cast<const C*>(lg.cn), lg.cnr, lg.nb, lg.blk0, tid, scan,
+                                    [&](C v, int, int n) { return vmul(v, tvc[(n - lg.blk0) & (N - 1)]); });
         }
     }
     __syncthreads();

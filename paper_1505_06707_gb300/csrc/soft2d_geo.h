@@ -9,8 +9,8 @@ struct Geo2D {              // passed by value to every 2D kernel
     const void* Wx;         // pass twiddles of the row FFT (length nx)
     const void* Wy;         // pass twiddles of the column FFT (length ny)
     const void* TVh;        // e^{-iU tau/2}, [ny][nx] (minus 1, float2, for complex64; complex128: factors)
-    const void* cnx;        // x-strip LU (mf, mb, g) for the row pass (complex128: FxCn)
-    const void* cny;        // y-strip LU (mf, mb, g) for the column pass
+    const void* cnx;        // x-strip CN tables of the row pass (soft1d.cuh, strip_cn; complex128: FxCn)
+    const void* cny;        // y-strip CN tables of the column pass
     int nx, ny;             // row length; number of rows (3D: ny nz)
     int nbx, blk0x;         // x-strip block (same for every row)
     int nby, blk0y;         // y-strip block (same for every column)
@@ -19,6 +19,7 @@ struct Geo2D {              // passed by value to every 2D kernel
     // z = r / ny1 (2D: ny1 = ny, no z block)
     int v2, ny1, nz1, nbz1, blk0z1;
     const void* vmeta;      // complex128: FxMeta of TVh
+    int cnrx, cnry;         // complex64: scan extents of cnx, cny (strip_tables_c)
 };
 
 // Lines along a strided axis: element i of line c of plane p sits at
@@ -27,7 +28,7 @@ struct Geo2D {              // passed by value to every 2D kernel
 struct LineGeo {
     const void* W;          // pass twiddles of the line FFT
     int64_t ld, plane;
-    const void* cn;         // strip CN LU (mf, mb, g) along the lines (COL_CVK; complex128: FxCn)
+    const void* cn;         // strip CN tables along the lines (COL_CVK; soft1d.cuh, strip_cn; complex128: FxCn)
     const void* tv;         // e^{-iU tau/2}, laid out as the state (COL_CVK)
     int nb, blk0;           // strip block along the lines (COL_CVK)
     // COL_CVK: with sel_div > 0 only lines whose (c / sel_div) mod sel_n lies
@@ -36,6 +37,7 @@ struct LineGeo {
     int64_t sel_div;
     int sel_n, sel_nb, sel_blk0;
     const void* vmeta;      // complex128: FxMeta of tv
+    int cnr;                // complex64: scan extents of cn (strip_tables_c)
 };
 
 // The strip CN along a strided axis: the cyclic block blk0 .. blk0 + nb - 1
