@@ -109,6 +109,7 @@ int persist_config(int prec, int logn, int* loge, int* logrm, int* groups);
 int launch_advance_time(double* d_t, double dt, cudaStream_t st);
 bool soft1d_supported(int prec, int logn, int loge, int logrm);
 void soft1d_default_cfg(int prec, int logn, int* loge, int* logrm);
+void soft1d_single_cfg(int prec, int logn, int* loge, int* logrm);
 
 int launch_observe1d(int prec, const Inst1D* d_inst, int count, const void* psi,
                      double* norm_in, double* flux, cudaStream_t st);

@@ -38,6 +38,19 @@ void soft1d_default_cfg(int prec, int logn, int* loge, int* logrm) {
     *logrm = e > 4 ? 4 : e;
 }
 
+// the same for one instance on its own, which has an SM to itself: latency
+// counts, and more threads of smaller butterflies shorten it.  us per step
+// with this / with the batch's (GB300, laser-batch contour, 100 steps):
+//   complex64   256: 1.53/1.94   1024: 2.76/5.31   2048: 3.94/5.39   4096: 7.29/8.03   8192: 14.3/19.1
+//   complex128  256: 6.20/8.11    512: 7.36/8.75   1024: 9.21/10.4   4096: 23.6/29.3
+// (radix 4 at N = 2048: 4.40 and 17.4 against radix 8's 3.94 and 16.2)
+void soft1d_single_cfg(int prec, int logn, int* loge, int* logrm) {
+    soft1d_default_cfg(prec, logn, loge, logrm);
+    if (logn >= 8 && logn <= 10) *loge = *logrm = 2;
+    else if (logn == 11 || logn == 12) *loge = *logrm = 3;
+    else if (logn == 13) *loge = *logrm = 4;
+}
+
 // every built (elements per thread, radix) variant of a size
 int soft1d_variants(int prec, int logn, int* loge, int* logrm, int maxv) {
     int k = 0;

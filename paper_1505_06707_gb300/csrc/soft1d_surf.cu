@@ -28,13 +28,14 @@ namespace {
 using SurfLaunch = int (*)(const Inst1D*, void*, int64_t, const double*, int64_t, int*, const void*, void*,
                            cudaStream_t);
 
-// the sampled step kernel is built for the default complex128 configuration
-// of N = 256 .. 8192
+// the sampled step kernel is built for a single complex128 instance's
+// configuration (soft1d_single_cfg) of N = 256 .. 8192
 SurfLaunch find_surf(int logn, int loge, int logrm) {
 #define SURF_CASE(LN, LE, LRM) \
     if (logn == LN && loge == LE && logrm == LRM) return &launch_soft1d_surf_t<double, LN, LE, LRM>;
-    SURF_CASE(8, 3, 3) SURF_CASE(9, 3, 3) SURF_CASE(10, 3, 3) SURF_CASE(11, 3, 3)
-    SURF_CASE(12, 4, 4) SURF_CASE(13, 4, 4)
+    SURF_CASE(8, 2, 2) SURF_CASE(9, 2, 2) SURF_CASE(10, 2, 2) SURF_CASE(11, 3, 3)
+    SURF_CASE(12, 3, 3) SURF_CASE(13, 4, 4)
+    SURF_CASE(8, 3, 3) SURF_CASE(9, 3, 3) SURF_CASE(10, 3, 3) SURF_CASE(12, 4, 4)      // (tuned plans)
 #undef SURF_CASE
     return nullptr;
 }
