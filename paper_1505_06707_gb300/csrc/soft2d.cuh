@@ -45,6 +45,11 @@ struct Cfg2DRow : Cfg1D<R, LOGN, LOGE, LOGRM> {
     static constexpr size_t OFF_B = sizeof(C) * (N + 64);
     static constexpr size_t OFF_W = OFF_B + sizeof(VT) * N;
     static constexpr size_t SMEM2 = OFF_W + sizeof(TWT) * TWN;
+    // N = 2048: five CTAs of 128 threads per SM (96 registers, no spills); with
+    // four, a row's loads and barriers leave half of the issue slots idle (82.7 ->
+    // 78.4 us per step at 2048^2).  Shorter rows are often a single wave, which
+    // runs faster with the registers.
+    static constexpr int MINB_ROW = LOGN >= 11 ? 640 / Cfg1D<R, LOGN, LOGE, LOGRM>::T : Cfg1D<R, LOGN, LOGE, LOGRM>::MINB;
     static_assert(OFF_B % 16 == 0 && OFF_W % 16 == 0, "16-byte aligned parts");
 };
 
@@ -80,7 +85,7 @@ __device__ __forceinline__ void inv_pass0_post(typename CT<R>::C* S, const TW* _
 // as the last inverse pass stores, then CN_x on the x-strip block.  ROW_K:
 // the kinetic factor alone.
 template <typename R, int LOGN, int LOGE, int LOGRM, int MODE>
-__global__ void __launch_bounds__(Cfg1D<R, LOGN, LOGE, LOGRM>::T, Cfg1D<R, LOGN, LOGE, LOGRM>::MINB)
+__global__ void __launch_bounds__(Cfg1D<R, LOGN, LOGE, LOGRM>::T, Cfg2DRow<R, LOGN, LOGE, LOGRM>::MINB_ROW)
 row_pass_kernel(Geo2D g, void* __restrict__ psi_v, const void* __restrict__ tkx_v)
 {
     using K = Cfg1D<R, LOGN, LOGE, LOGRM>;
@@ -110,6 +115,10 @@ row_pass_kernel(Geo2D g, void* __restrict__ psi_v, const void* __restrict__ tkx_
     }
     for (int i = tid; i < RC::TWN; i += T) cp_async<sizeof(TWT)>(&Ws[i], &W[i]);
     cp_async_commit();
+    StripRegs<T, K::CMAX> sr;                       // (E <= 4: requested with the row)
+    if constexpr (MODE == ROW_KVC && E <= 4) {
+        if (g.nbx > 0) sr.load(reinterpret_cast<const C*>(g.cnx), g.cnrx, g.nbx, tid);
+    }
     cp_async_wait<0>();
     __syncthreads();
     fwd_passes<R, LOGN, LOGE, LOGRM, 0, K::NPASS - 1>(S, Ws, tid);
@@ -122,8 +131,9 @@ row_pass_kernel(Geo2D g, void* __restrict__ psi_v, const void* __restrict__ tkx_
         inv_pass0_post<R, LOGN, LOGE, LOGRM, true>(S, Ws, tid, [&](int n, C v) { return vmul(v, Tv[n]); });
         __syncthreads();
         if (g.nbx > 0) {
-            strip_cn<T, K::CMAX, N, true>(S, reinterpret_cast<const C*>(g.cnx), g.cnrx, g.nbx, g.blk0x, tid, scan,
-                                    [](C v, int, int) { return v; });
+            auto post = [](C v, int, int) { return v; };
+            strip_cn<T, K::CMAX, N, true, decltype(post), BarCTA, E <= 4>(
+                S, reinterpret_cast<const C*>(g.cnx), g.cnrx, g.nbx, g.blk0x, tid, scan, post, BarCTA(), &sr);
             __syncthreads();
         }
     }
@@ -162,7 +172,9 @@ struct ColCfg {
     using K = Cfg1D<R, LOGN, LOGE, LOGRM>;
     using C = typename K::C;
     static constexpr int THREADS = TW * K::T;
-    static constexpr int MINB = THREADS >= 512 ? 1 : 512 / THREADS;   // <= 128 registers
+    // <= 128 registers; 80 for lines of 256 points and less, whose CTAs mostly wait
+    // for their tile (256^3 step: 479 -> 461 us; longer lines spill and lose)
+    static constexpr int MINB = THREADS >= 512 ? 1 : THREADS <= 128 && K::E <= 8 ? 768 / THREADS : 512 / THREADS;
     // column pitch: N + 64 bytes, so that the TW columns of one row fall in
     // different banks when the tile is filled and drained row by row
     static constexpr int PITCH = K::N + 64 / (int)sizeof(C);
@@ -218,8 +230,12 @@ col_pass_kernel(LineGeo lg, void* __restrict__ psi_v, const void* __restrict__ t
     }
     for (int i = threadIdx.x; i < CC::TWN; i += TW * T) cp_async<sizeof(TWT)>(&Ws[i], &W[i]);
     cp_async_commit();
-    cp_async_wait<0>();
     const int col = threadIdx.x / T, tid = threadIdx.x % T;
+    StripRegs<T, K::CMAX> sr;                       // (E <= 4: requested with the tile)
+    if constexpr (MODE != COL_K && K::E <= 4) {
+        if (lg.nb > 0) sr.load(reinterpret_cast<const C*>(lg.cn), lg.cnr, lg.nb, tid);
+    }
+    cp_async_wait<0>();
     C* Sc = S + col * PITCH;
     bool off_v = MODE == COL_CVK;                    // V/2 off the strip block here
     if (MODE == COL_CVK && lg.sel_div > 0) {
@@ -244,8 +260,9 @@ col_pass_kernel(LineGeo lg, void* __restrict__ psi_v, const void* __restrict__ t
         if (lg.nb > 0) {
             const VT* tvc = Tvs + col * CC::VCAP;
             C* scan = reinterpret_cast<C*>(smem_raw + CC::OFF_SCAN) + 32 * col;
-            strip_cn<T, K::CMAX, N, true>(Sc, reinterpret_cast<const C*>(lg.cn), lg.cnr, lg.nb, lg.blk0, tid, scan,
-                                    [&](C v, int, int n) { return vmul(v, tvc[(n - lg.blk0) & (N - 1)]); });
+            auto post = [&](C v, int, int n) { return vmul(v, tvc[(n - lg.blk0) & (N - 1)]); };
+            strip_cn<T, K::CMAX, N, true, decltype(post), BarCTA, K::E <= 4>(
+                Sc, reinterpret_cast<const C*>(lg.cn), lg.cnr, lg.nb, lg.blk0, tid, scan, post, BarCTA(), &sr);
         }
     }
     __syncthreads();
