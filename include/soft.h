@@ -101,8 +101,8 @@ typedef struct {
     int persistent;      /* batch plans: 1 advances the instances with
                             N = 2048 .. 16384 by one persistent kernel that
                             takes packs of same-size instances from a queue,
-                            largest N first, if there is at most one pack per
-                            SM, and else, as 0 always does, by one kernel per
+                            largest N first, if there is at most one instance
+                            per SM, and else, as 0 always does, by one kernel per
                             size group (faster for larger batches; the results
                             are the same).  With autotune the plan times both
                             on one 16-step chunk and keeps the faster [1]    */

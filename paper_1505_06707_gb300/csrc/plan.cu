@@ -891,6 +891,23 @@ int soft_plan::build_1d_device() {
     // the persistent kernel's sizes leave the group list: their instances
     // form packs of up to G same-size instances, largest N first
     if (!single && opt.persistent) {
+        int dev = 0, nsm = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return SOFT_ERR_CUDA;
+        // the fewest instances per pack that still give at most one pack per SM:
+        // SMs left idle cost more than part-filled CTAs (24 steps of 8 complex64
+        // instances, full packs / one each: N = 2048 474 / 371 us, N = 8192 880 / 670)
+        auto packs_for = [&](size_t cap) {
+            size_t k = 0;
+            int le, lr, G;
+            for (const auto& g : groups)
+                if (persist_config(prec, g.logn, &le, &lr, &G) >= 0 && le == g.loge && lr == g.logrm)
+                    k += (g.members.size() + std::min<size_t>(G, cap) - 1) / std::min<size_t>(G, cap);
+            return k;
+        };
+        size_t cap = 1;
+        while (cap < 8 && packs_for(cap) > (size_t)nsm) cap *= 2;
         std::vector<Pack1D> packs;
         std::vector<Inst1D> pd;
         for (auto& g : groups) {
@@ -898,6 +915,7 @@ int soft_plan::build_1d_device() {
             const int v = persist_config(prec, g.logn, &le, &lr, &G);
             if (v < 0 || le != g.loge || lr != g.logrm) continue;
             g.in_persist = true;
+            G = (int)std::min<size_t>(G, cap);
             for (size_t k = 0; k < g.members.size(); k += G) {
                 Pack1D pk;
                 pk.var = v;
@@ -910,17 +928,14 @@ int soft_plan::build_1d_device() {
         }
         std::stable_sort(packs.begin(), packs.end(), [](const Pack1D& a, const Pack1D& b) { return a.var < b.var; });
         npacks = (int)packs.size();
-        // The persistent kernel keeps one 512-thread CTA per SM for every size;
-        // per-size kernels keep two or more CTAs of the smaller sizes, whose
-        // phases fill each other's waits.  With more packs than SMs the latter
-        // are faster (16 steps of the mixed laser batch, persistent / per size:
-        // complex64, 4096 instances 7.71 / 6.24 ms, complex128, 1216 instances
-        // 9.5 / 7.9 ms), so the queue runs batches of at most one pack per SM.
-        int dev = 0, nsm = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return SOFT_ERR_CUDA;
-        use_persist = npacks > 0 && npacks <= nsm;
+        // The persistent kernel keeps one 512-thread CTA per SM for every size and
+        // spills registers (four sizes in one kernel); per-size kernels keep two
+        // or more CTAs of the smaller sizes, whose phases fill each other's waits.
+        // With more instances than SMs the latter are faster (16 steps of the mixed
+        // laser batch, persistent / per size: complex64, 4096 instances 7.71 / 6.24
+        // ms, complex128, 1216 instances 9.5 / 7.9 ms), so the queue runs batches of
+        // at most one instance per SM, in one launch.
+        use_persist = npacks > 0 && npacks <= nsm && cap == 1;
         if (npacks > 0) {
             if ((rc = upload((void**)&d_pinst, pd.data(), pd.size() * sizeof(Inst1D)))) return rc;
             if ((rc = upload(&d_packs, packs.data(), packs.size() * sizeof(Pack1D)))) return rc;

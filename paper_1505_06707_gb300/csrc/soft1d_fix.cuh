@@ -403,7 +403,7 @@ __device__ __noinline__ float fx_normalise(fx2* S, int& e, unsigned* red, int ti
 // Strip Crank-Nicolson tables of complex128 plans (host: plan.cu,
 // strip_tables_fx), T threads of ch rows: entry 0 is the header (lg, rounds of
 // the forward and backward scans, spans), then factors in chunk order as in
-// strip_cn_1d: mf of rows t ch + c, c <= ch, at c T + t, and g; then for the
+// strip_cn: mf of rows t ch + c, c <= ch, at c T + t, and g; then for the
 // forward and for the backward scan the products [5][T] of the 2^r chunk
 // totals that end (start) at t, the exclusive product of t's warp [T] and the
 // warp totals [T/32]; last (gen) mf and g as double2.
@@ -470,7 +470,7 @@ __device__ __forceinline__ fx2 fx_carry(fx2 Y, const int4* __restrict__ tab, int
     return ex;
 }
 
-// Strip Crank-Nicolson (strip_cn_1d in soft1d.cuh) in fixed point, followed by
+// Strip Crank-Nicolson (strip_cn in soft1d.cuh) in fixed point, followed by
 // post(v, c, n) on row c of the thread, grid index n (|v| < 2^60.5): the second
 // half potential and field factor.  Every multiplier and chunk product
 // has modulus <= 1 and the sweeps grow the rows by at most 2^lg (host check;
@@ -541,7 +541,7 @@ __device__ __forceinline__ float strip_cn_fx(fx2* S, const FxCn<Fx1D<LOGN, LOGE,
     return t2;
 }
 
-// The same on rows held as doubles, in FP64 (strip_cn_1d): plans with the
+// The same on rows held as doubles, in FP64 (the chunk products formed in the kernel): plans with the
 // `gen` flag.  cn: mf and g in chunk order.
 template <int LOGN, int LOGE, int LOGRM, class B, class Post>
 __device__ __forceinline__ void strip_cn_gen(fx2* S, const double2* __restrict__ cn, int nb, int blk0, int tid,

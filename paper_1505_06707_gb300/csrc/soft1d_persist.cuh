@@ -47,7 +47,7 @@ struct PVar {
 // one pack: the twiddles of its size into shared memory (the same for every
 // instance of that size), then each group advances its instance
 template <typename R, class V>
-__device__ __forceinline__ void run_pack(const Pack1D& pk, const Inst1D* __restrict__ insts, void* psi,
+__device__ __noinline__ void run_pack(const Pack1D& pk, const Inst1D* __restrict__ insts, void* psi,
                                          int64_t nsteps, const double* ftab, int64_t fstride, int* status,
                                          unsigned char* smem) {
     using C = typename CT<R>::C;
