@@ -5,9 +5,9 @@ Workload: 4096 independent 1D instances, N drawn from {2048, 4096, 8192,
 the half-width to theta = 0.5 at the edge, soft-Coulomb a^2 = 2, laser pulse
 E0 sin^2 sin with omega = 0.057, 4 cycles, E0 ~ U[0.01, 0.1]; dt = 0.02.
 One benchmark step advances every instance by STEPS_PER_CALL time steps in
-one library call (one persistent kernel over all instances).
+one library call (one kernel per size group).
 
-The headline line is complex128 (FP64 arithmetic, the oracle's precision);
+The headline line is complex128 (64-bit arithmetic, the oracle's precision);
 complex64 is reported beside it with its error after the whole pulse.
 
 Metric: grid-point-steps per second = sum_j N_j * time steps / seconds.
@@ -90,6 +90,12 @@ def _traffic(prec, n, instances, steps):
 # 2.07 GHz, which the FMA probe of this package reproduces within a few %)
 FP32_FMA_PER_SM_CLK = 128
 FP64_FMA_PER_SM_CLK = 2
+# The complex128 kernels compute in 64-bit fixed point on the integer pipes:
+# 59 32 x 32 -> 64 bit multiply-adds or 64-bit additions per clock and SM
+# (measured 58 and 60).  A radix-2 butterfly, 10 flops, is a complex product of
+# 12 multiply-adds and 4 additions: 1.6 slots per flop.
+FX_SLOTS_PER_SM_CLK = 59
+FX_SLOTS_PER_FLOP = 1.6
 
 
 def alu_peaks(torch=None, dev=0):
@@ -104,6 +110,7 @@ def alu_peaks(torch=None, dev=0):
     return {"fp32_tflops": nsm * FP32_FMA_PER_SM_CLK * 2 * mhz * 1e6 / 1e12,
             "fp64_tflops": nsm * FP64_FMA_PER_SM_CLK * 2 * mhz * 1e6 / 1e12,
             "sms": nsm, "sm_max_mhz": mhz,
+            "fixed64_tflops": nsm * FX_SLOTS_PER_SM_CLK / FX_SLOTS_PER_FLOP * mhz * 1e6 / 1e12,
             "how": "SMs x FMA lanes per SM (FP32 128, FP64 2) x 2 flop x max SM clock"}
 
 
@@ -847,7 +854,7 @@ def roofline_w2(torch, dev, m, prec_name):
     persistent kernel, the whole call (one launch)."""
     ap_ = alu_peaks(torch, dev.index or 0)
     c64 = prec_name == "c64"
-    peak = ap_["fp32_tflops"] if c64 else ap_["fp64_tflops"]
+    peak = ap_["fp32_tflops"] if c64 else ap_["fixed64_tflops"]
     dom = m.get("dominant")
     if dom:
         achieved = dom["flops"] / (dom["ms"] / 1e3) / 1e12
@@ -868,9 +875,11 @@ def roofline_w2(torch, dev, m, prec_name):
             "kernel": kern,
             "whole_call": {"achieved": whole, "frac": whole / peak,
                            "schedule": m["schedule"], "ms_per_call": m["call_ms"]},
-            "peak_source": "derived: %d SMs x %d %s FMA per clock x 2 x %.0f MHz" % (
-                ap_["sms"], FP32_FMA_PER_SM_CLK if c64 else FP64_FMA_PER_SM_CLK, "FP32" if c64 else "FP64",
-                ap_["sm_max_mhz"]),
+            "peak_source": "derived: %d SMs x %d FP32 FMA per clock x 2 x %.0f MHz" % (
+                ap_["sms"], FP32_FMA_PER_SM_CLK, ap_["sm_max_mhz"]) if c64 else
+            "derived: %d SMs x %d 64-bit fixed-point slots per clock / %.1f slots per flop x %.0f MHz (FP64 pipe: "
+            "%.2f TFLOP/s)" % (ap_["sms"], FX_SLOTS_PER_SM_CLK, FX_SLOTS_PER_FLOP, ap_["sm_max_mhz"],
+                               ap_["fp64_tflops"]),
             "flop_count": "per time step and instance 10 N log2 N (two FFTs) + 12 N (phase products) + "
                           "6 N (field) + 32 per strip row"}
 
