@@ -61,8 +61,11 @@ __device__ __forceinline__ void fx_halves(long long v, int& h, int& l) {
     h = fx_hi(v) + (int)((unsigned)l >> 31);
 }
 
-// v w 2^(K-2) (CONJ: v conj(w)); |v| 2^K < 2^62.9 per component.  The product
-// of the low halves (below 1/4 unit) is dropped.  The high word of the middle
+// v w 2^(K-2) (CONJ: v conj(w)).  Range: the middle sum is at most
+// (|v| 2^K + |w| 2^62)/sqrt(2) in size (|v|, |w|: moduli of the complex values),
+// and must stay below 2^63: |v| 2^K <= 2^62.8 for |w| <= 1.01 (lines with norms
+// of FX_NORM in units of 1/4), 2^62.3 for |w| <= 1.43, 2^61.5 for |w| <= 1.9.
+// The product of the low halves (below 1/4 unit) is dropped.  The high word of the middle
 // sum is added by a multiplication by 1, which needs no sign extension into a
 // register pair: 27 instructions, 0.51 clocks of an SM (0.57 with the
 // extension and the halves' carry as 64-bit additions), bound by the wide

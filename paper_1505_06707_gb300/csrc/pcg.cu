@@ -96,7 +96,9 @@ static std::vector<cd> umajor(const BandAxis& B, const std::vector<cd>& tab) {
 }
 // the same as fixed-point factors (pcg_fix.cuh): without the 1/sqrt n, times
 // 2^-p with 2^p a bound of the operator norm (row sums times column sums);
-// back: the half bits of the inverse FFT that follows
+// back: the half bits of the inverse FFT that follows, as sqrt(1/2) and, where
+// they are +1, one more in p: the lines have norms up to FX_NORM, which leaves
+// no room for entries above 1 (fx_mul)
 int upload_band_fx(void** dst, const BandAxis& B, const std::vector<cd>& tab, int logn, int logrm, bool back, int* p) {
     std::vector<cd> t = umajor(B, tab);
     const double sn = std::sqrt((double)B.n);
@@ -109,10 +111,11 @@ int upload_band_fx(void** dst, const BandAxis& B, const std::vector<cd>& tab, in
         }
     const double nrm = std::sqrt(*std::max_element(rows.begin(), rows.end()) *
                                  *std::max_element(cols.begin(), cols.end()));
-    *p = std::max(0, (int)std::ceil(std::log2(nrm) - 1e-6));       // (a norm of 1 keeps p = 0)
     const int lrl = (logn % logrm) ? logn % logrm : logrm;
     const int half = back ? ((logrm - lrl) & 1) - (logrm & 1) : 0;
-    const double sc = sn * std::ldexp(half == 0 ? 1.0 : half > 0 ? std::sqrt(2.0) : std::sqrt(0.5), -*p);
+    const int pn = std::max(0, (int)std::ceil(std::log2(nrm) - 1e-6));       // (a norm of 1 keeps pn = 0)
+    const double sc = sn * std::ldexp(half == 0 ? 1.0 : std::sqrt(0.5), -pn);
+    *p = pn + (half > 0 ? 1 : 0);
     for (cd& v : t) v *= sc;
     return upload_fx(dst, t);
 }
