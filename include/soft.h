@@ -164,7 +164,8 @@ int soft_batch_layout(const soft_plan* plan, int64_t* offsets, int64_t* total);
  * lines (rows, then columns), with C = C_x + C_y (+ C_z) as Kronecker sums
  * so that e^{-iC tau} factors into one CN per axis; the middle steps are
  * replayed from a CUDA graph captured on the first call with a given state
- * pointer and stream. */
+ * pointer and stream.  1D calls are not recorded into a caller's stream
+ * capture (SOFT_ERR_CUDA; soft_step_noalloc is). */
 int soft_step(soft_plan* plan, void* psi, int64_t nsteps, const soft_field* field,
               double* t_inout, void* stream);
 

@@ -728,6 +728,16 @@ int soft_batch_layout(const soft_plan* P, int64_t* offsets, int64_t* total) {
     return SOFT_OK;
 }
 
+// 1D steps are not recorded into a caller's stream capture: a replay would use
+// the start time, and the host copies of a new field, of the call that
+// recorded it (soft_step_noalloc takes both by value)
+static int not_capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(st, &cs);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && cs == cudaStreamCaptureStatusNone ? SOFT_OK : SOFT_ERR_CUDA;
+}
+
 static int soft_step_impl(soft_plan* P, void* psi, int64_t nsteps, const soft_field* field, double* t_inout,
                           void* stream) {
     if (!P || !psi || !t_inout || nsteps < 0) return SOFT_ERR_INVALID_ARG;
@@ -735,7 +745,8 @@ static int soft_step_impl(soft_plan* P, void* psi, int64_t nsteps, const soft_fi
     if (P->kind == 3) return P->step_3d(psi, nsteps, t_inout, (cudaStream_t)stream);
     if (P->kind != 1) return SOFT_ERR_INVALID_ARG;
     if (P->single) {
-        int rc = P->set_single_field(field, (cudaStream_t)stream);
+        int rc = nsteps > 0 ? not_capturing((cudaStream_t)stream) : SOFT_OK;
+        if (rc == SOFT_OK) rc = P->set_single_field(field, (cudaStream_t)stream);
         if (rc) return rc;
     }
     return P->step_1d(psi, nsteps, t_inout, (cudaStream_t)stream);
@@ -747,6 +758,8 @@ int soft_step(soft_plan* P, void* psi, int64_t nsteps, const soft_field* field, 
 
 static int soft_step_batch_impl(soft_plan* P, void* psi, int64_t nsteps, double* t_inout, void* stream) {
     if (!P || !psi || !t_inout || nsteps < 0 || P->kind != 1) return SOFT_ERR_INVALID_ARG;
+    const int rc = P->single && nsteps > 0 ? not_capturing((cudaStream_t)stream) : SOFT_OK;
+    if (rc) return rc;
     return P->step_1d(psi, nsteps, t_inout, (cudaStream_t)stream);
 }
 int soft_step_batch(soft_plan* P, void* psi, int64_t nsteps, double* t_inout, void* stream) {
