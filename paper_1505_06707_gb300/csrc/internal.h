@@ -109,6 +109,8 @@ int persist_config(int prec, int logn, int* loge, int* logrm, int* groups);
 int launch_advance_time(double* d_t, double dt, cudaStream_t st);
 bool soft1d_supported(int prec, int logn, int loge, int logrm);
 void soft1d_default_cfg(int prec, int logn, int* loge, int* logrm);
+// the surface-sampled step is built for the variant
+bool soft1d_surf_supported(int logn, int loge, int logrm);
 void soft1d_single_cfg(int prec, int logn, int* loge, int* logrm);
 
 int launch_observe1d(int prec, const Inst1D* d_inst, int count, const void* psi,

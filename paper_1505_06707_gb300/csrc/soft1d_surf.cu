@@ -20,6 +20,7 @@
 
 #include "plan_internal.h"
 #include "soft1d.cuh"
+#include "soft1d_c128_list.h"
 
 namespace soft {
 
@@ -28,14 +29,12 @@ namespace {
 using SurfLaunch = int (*)(const Inst1D*, void*, int64_t, const double*, int64_t, int*, const void*, void*,
                            cudaStream_t);
 
-// the sampled step kernel is built for a single complex128 instance's
-// configuration (soft1d_single_cfg) of N = 256 .. 8192
+// the sampled step kernel of a complex128 variant, N = 256 .. 8192
 SurfLaunch find_surf(int logn, int loge, int logrm) {
 #define SURF_CASE(LN, LE, LRM) \
     if (logn == LN && loge == LE && logrm == LRM) return &launch_soft1d_surf_t<double, LN, LE, LRM>;
-    SURF_CASE(8, 2, 2) SURF_CASE(9, 2, 2) SURF_CASE(10, 2, 2) SURF_CASE(11, 3, 3)
-    SURF_CASE(12, 3, 3) SURF_CASE(13, 4, 4)
-    SURF_CASE(8, 3, 3) SURF_CASE(9, 3, 3) SURF_CASE(10, 3, 3) SURF_CASE(12, 4, 4)      // (tuned plans)
+    SOFT1D_C128_256_TO_2048(SURF_CASE)
+    SOFT1D_C128_4096_TO_8192(SURF_CASE)
 #undef SURF_CASE
     return nullptr;
 }
@@ -224,6 +223,8 @@ surff_kernel(const double2* __restrict__ xw, int n, const double2* __restrict__ 
 }
 
 }  // namespace
+
+bool soft1d_surf_supported(int logn, int loge, int logrm) { return find_surf(logn, loge, logrm) != nullptr; }
 
 struct Surf1D {
     SurfTabs t;
