@@ -362,8 +362,8 @@ __device__ __forceinline__ unsigned fx_group_max(unsigned v, unsigned* red, int 
 }
 
 // The state as doubles in units 2^e -> fixed point: the largest component
-// between 2^59 and 2^60, e changed to match.  Returns the thread's sum of
-// fx_abs2; bad: a non-finite sample.
+// between 2^59 and 2^60, e changed to match (not for zeros).  Returns the
+// thread's sum of fx_abs2; bad: a non-finite sample.
 template <int LOGN, int LOGE, int LOGRM, class B>
 __device__ __noinline__ float fx_normalise(fx2* S, int& e, unsigned* red, int tid, B bar, bool& bad) {
     using F = Fx1D<LOGN, LOGE, LOGRM>;
@@ -372,6 +372,8 @@ __device__ __noinline__ float fx_normalise(fx2* S, int& e, unsigned* red, int ti
 #pragma unroll 1
     for (int j = 0; j < E; ++j) m = max(m, fx_mag(fx_asd(S[swz<fx2>(tid + j * T)])));
     m = fx_group_max<T>(m, red, tid, bar);
+    bool zero = false;
+    int off = 0;
     if (m < (128u << 20)) {                       // tiny (or zero): scale up first
         unsigned q = 0;
 #pragma unroll 1
@@ -381,10 +383,11 @@ __device__ __noinline__ float fx_normalise(fx2* S, int& e, unsigned* red, int ti
             r = fx_bits(d);
             q = max(q, fx_mag(d));
         }
-        e -= 800;
+        off = -800;
         bar.sync();
         m = fx_group_max<T>(q, red, tid, bar);
-        if (m < (128u << 20)) m = 1023u << 20;    // zero
+        zero = m < (128u << 20);
+        if (zero) m = 1023u << 20;
     }
     bad = (m >> 20) == 0x7ff;
     const int ed = (int)(m >> 20) - 1022 - 60;
@@ -396,7 +399,7 @@ __device__ __noinline__ float fx_normalise(fx2* S, int& e, unsigned* red, int ti
         r = v;
         t2 += fx_abs2(v);
     }
-    e += ed;
+    if (!zero) e += ed + off;
     return t2;
 }
 
@@ -706,7 +709,7 @@ __device__ __forceinline__ void soft1d_run_fx(const Inst1D& I, void* __restrict_
 #pragma unroll
         for (int w = 1; w < NW; ++w) t2 += part[w];
         const int k = fx_norm_shift(t2, N);
-        e -= k;
+        e = max(e - k, -(1 << 24));     // (a zero state is shifted in every step; below 2^-1074 all is zero)
         if (k != 0 || kx != 0) rescale_fx<LOGN, LOGE, LOGRM>(S, k, kx, nb, blk0, tid);
         // ---- kinetic: forward FFT, e^{-iK tau} (e^{-iK tau/2} in the first
         //      and last pass of the call), inverse FFT, potential of the next step
