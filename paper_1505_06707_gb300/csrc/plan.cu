@@ -1071,8 +1071,8 @@ int soft_plan::ensure_side() {
     return groups.size() > MAX_SIDE ? SOFT_ERR_UNSUPPORTED : SOFT_OK;
 }
 
-// The schedule autotuner of a batch plan: one chunk of 16 steps on a zero
-// state with the persistent kernel and with one kernel per size group
+// The schedule autotuner of a batch plan: one chunk of 16 steps on a constant,
+// non-zero state (as autotune_size: a zero one is not a step's usual work) with the persistent kernel and with one kernel per size group
 // (each timed after a warm-up run); the faster is kept.
 int soft_plan::time_schedules() {
     int rc = ensure_side();
@@ -1083,7 +1083,7 @@ int soft_plan::time_schedules() {
     cudaStream_t st = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     float ms[2] = {0, 0};
-    rc = cuda_status(cudaMemset(tmp, 0, eb * (size_t)total));
+    rc = cuda_status(cudaMemset(tmp, 0x3c, eb * (size_t)total));
     if (!rc) rc = cuda_status(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
     if (!rc) rc = cuda_status(cudaEventCreate(&e0));
     if (!rc) rc = cuda_status(cudaEventCreate(&e1));
