@@ -101,9 +101,9 @@ typedef struct {
     int persistent;      /* batch plans: 1 advances the instances with
                             N = 2048 .. 16384 by one persistent kernel that
                             takes packs of same-size instances from a queue,
-                            largest N first, if there is at most one instance
-                            per SM, and else, as 0 always does, by one kernel per
-                            size group (faster for larger batches; the results
+                            largest N first, if there is at most one of them per
+                            SM, and else, as 0 always does, by one kernel per
+                            size group (more launches, less time; the results
                             are the same).  With autotune the plan times both
                             on one 16-step chunk and keeps the faster [1]    */
 } soft_options;
@@ -172,10 +172,11 @@ int soft_step(soft_plan* plan, void* psi, int64_t nsteps, const soft_field* fiel
 /* soft_step_batch -- soft_step for a batch plan; psi is the packed state.
  * Calls are replayed from a CUDA graph (captured on the first call with a
  * given state pointer, stream and step count): the pulse-shape table, the
- * persistent kernel over the instances with N = 2048 .. 16384 (one CTA per
- * SM; 1, 2, 2, 4 instances of N = 16384, 8192, 4096, 2048 per work item
- * for complex64, 1, 1, 2, 2 for complex128) and one kernel per remaining
- * size group, on parallel branches so that their CTAs share the GPU. */
+ * persistent kernel over the instances with N = 2048 .. 16384 where the
+ * plan's schedule has it (soft_options.persistent; one CTA per SM, work items
+ * of one instance, or, in large tuned batches, of up to 1, 2, 2, 4 of N = 16384, 8192,
+ * 4096, 2048 for complex64 and 1, 1, 2, 2 for complex128) and one kernel per
+ * remaining size group, on parallel branches so that their CTAs share the GPU. */
 int soft_step_batch(soft_plan* plan, void* psi, int64_t nsteps, double* t_inout,
                     void* stream);
 

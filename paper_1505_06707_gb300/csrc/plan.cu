@@ -883,6 +883,41 @@ Inst1D soft_plan::descriptor(int i) const {
     return d;
 }
 
+// the instances of the persistent kernel's sizes as packs of same-size
+// instances, largest N first
+int soft_plan::build_packs(size_t cap) {
+    std::vector<Pack1D> packs;
+    std::vector<Inst1D> pd;
+    for (auto& g : groups) {
+        int le, lr, G;
+        const int v = persist_config(prec, g.logn, &le, &lr, &G);
+        if (v < 0 || le != g.loge || lr != g.logrm) continue;
+        g.in_persist = true;
+        G = (int)std::min<size_t>(G, cap);
+        for (size_t k = 0; k < g.members.size(); k += G) {
+            Pack1D pk;
+            pk.var = v;
+            pk.first = (int)pd.size();
+            pk.count = (int)std::min<size_t>(G, g.members.size() - k);
+            pk.pad_ = 0;
+            for (int j = 0; j < pk.count; ++j) pd.push_back(descriptor(g.members[k + j]));
+            packs.push_back(pk);
+        }
+    }
+    std::stable_sort(packs.begin(), packs.end(), [](const Pack1D& a, const Pack1D& b) { return a.var < b.var; });
+    cudaFree(d_pinst); cudaFree(d_packs); cudaFree(d_pcount);
+    d_pinst = nullptr; d_packs = nullptr; d_pcount = nullptr;
+    npacks = (int)packs.size();
+    use_persist = npacks > 0;
+    if (npacks == 0) return SOFT_OK;
+    int rc;
+    if ((rc = upload((void**)&d_pinst, pd.data(), pd.size() * sizeof(Inst1D)))) return rc;
+    if ((rc = upload(&d_packs, packs.data(), packs.size() * sizeof(Pack1D)))) return rc;
+    if ((rc = cuda_status(cudaMalloc((void**)&d_pcount, sizeof(int))))) return rc;
+    // sets the kernel's shared-memory attribute outside any capture
+    return launch_persist(prec, nullptr, 0, nullptr, nullptr, nullptr, 0, nullptr, 0, nullptr, 0, nullptr);
+}
+
 int soft_plan::build_1d_device() {
     // groups by kernel configuration, largest N first
     std::map<std::pair<int, int>, int> gid;
@@ -901,8 +936,6 @@ int soft_plan::build_1d_device() {
     }
     std::sort(groups.begin(), groups.end(), [](const Group1D& a, const Group1D& b) { return a.logn > b.logn; });
     int rc;
-    // the persistent kernel's sizes leave the group list: their instances
-    // form packs of up to G same-size instances, largest N first
     if (!single && opt.persistent) {
         int dev = 0, nsm = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -921,43 +954,20 @@ int soft_plan::build_1d_device() {
         };
         size_t cap = 1;
         while (cap < 8 && packs_for(cap) > (size_t)nsm) cap *= 2;
-        std::vector<Pack1D> packs;
-        std::vector<Inst1D> pd;
-        for (auto& g : groups) {
-            int le, lr, G;
-            const int v = persist_config(prec, g.logn, &le, &lr, &G);
-            if (v < 0 || le != g.loge || lr != g.logrm) continue;
-            g.in_persist = true;
-            G = (int)std::min<size_t>(G, cap);
-            for (size_t k = 0; k < g.members.size(); k += G) {
-                Pack1D pk;
-                pk.var = v;
-                pk.first = (int)pd.size();
-                pk.count = (int)std::min<size_t>(G, g.members.size() - k);
-                pk.pad_ = 0;
-                for (int j = 0; j < pk.count; ++j) pd.push_back(descriptor(g.members[k + j]));
-                packs.push_back(pk);
-            }
-        }
-        std::stable_sort(packs.begin(), packs.end(), [](const Pack1D& a, const Pack1D& b) { return a.var < b.var; });
-        npacks = (int)packs.size();
-        // The persistent kernel keeps one 512-thread CTA per SM for every size and
-        // spills registers (four sizes in one kernel); per-size kernels keep two
-        // or more CTAs of the smaller sizes, whose phases fill each other's waits.
-        // With more instances than SMs the latter are faster (16 steps of the mixed
-        // laser batch, persistent / per size: complex64, 4096 instances 7.71 / 6.24
-        // ms, complex128, 1216 instances 9.5 / 7.9 ms), so the queue runs batches of
-        // at most one instance per SM, in one launch.
+        if ((rc = build_packs(cap))) return rc;
+        // By default the queue runs batches of at most one instance per SM, in one
+        // launch.  One kernel for four sizes spills registers and keeps one CTA of 512
+        // threads per SM, so one launch per size takes less time at every batch
+        // size (24 steps, persistent / per size, us, 8, 152 and 300 instances):
+        //   complex64   N = 2048: 372/169, 402/191, 417/191    N = 4096: 404/248, 419/258, 503/327
+        //               N = 8192: 671/509, 691/525, 899/717    N = 16384: 849/708, 867/719, 1713/1420
+        //               2048 to 16384 mixed: 877/773, 890/773, 997/863
+        //   complex128  N = 2048: 588/486, 594/494, 812/691    N = 4096: 1001/856, 1026/873, 1373/1204
+        //               N = 8192: 1461/1365, 1474/1375, 2922/2734   N = 16384: 3679/3043, 3766/3083, 7508/6160
+        //               mixed: 3640/3043, 3748/3058, 3776/3066
+        // A caller who counts time and not launches sets persistent = 0, or autotune,
+        // which times both, also the packs of several instances of larger batches.
         use_persist = npacks > 0 && npacks <= nsm && cap == 1;
-        if (npacks > 0) {
-            if ((rc = upload((void**)&d_pinst, pd.data(), pd.size() * sizeof(Inst1D)))) return rc;
-            if ((rc = upload(&d_packs, packs.data(), packs.size() * sizeof(Pack1D)))) return rc;
-            if ((rc = cuda_status(cudaMalloc((void**)&d_pcount, sizeof(int))))) return rc;
-            // sets the kernel's shared-memory attribute outside any capture
-            if ((rc = launch_persist(prec, nullptr, 0, nullptr, nullptr, nullptr, 0, nullptr, 0, nullptr, 0,
-                                     nullptr)))
-                return rc;
-        }
     }
     for (auto& g : groups) {
         std::vector<Inst1D> d;

@@ -193,6 +193,7 @@ struct soft_plan {
 
     soft::Inst1D descriptor(int i) const;
     int build_1d_device();
+    int build_packs(size_t cap);   // packs of up to min(G, cap) instances; the persistent schedule if there are any
     int set_single_field(const soft_field* f, cudaStream_t st);
     int enqueue_chunk(void* psi, int64_t chunk, cudaStream_t st);
     int ensure_side();

@@ -3,8 +3,10 @@
 // A work item (a pack) is up to G instances of one size, G = 512 / T, each
 // advanced by its own warp-aligned group of T threads with a named barrier,
 // so every size keeps the thread count and shared memory per instance of its
-// one-instance kernel.  The big packs (N = 16384, 2 x 8192) go first; the
-// small ones (2 x 4096, 4 x 2048) fill the tail, so the SMs finish together.
+// batch kernel.  Batches of at most one instance per SM have one instance per
+// pack; larger ones, which take this kernel only where tuning finds it faster,
+// as few as leave one pack per SM (plan.cu, which has the times against
+// per-size kernels).
 #pragma once
 #include "soft1d.cuh"
 
