@@ -11,10 +11,13 @@
 // FP32 operands (the network's input, the loss gradient) enter as three BF16
 // terms that add up to them exactly (8 + 8 + 8 bits), so the products are
 // those of the FP32 value.  The tensor cores' FP32 accumulation truncates, a
-// bias that grows with the chain (54 products deep it left 1.6e-6 of the
-// gradient, against 1.1e-6 of the scalar sums), so a chain is at most FLUSH
-// rows, 8 products, and is then added, rounded to nearest, to the thread's own
-// sums in shared memory; the CTAs' sums are added in FP64.
+// bias that grows with the chain: 8 products deep it left 5.5e-8 of the gradient
+// of exact operands (32 fields of 128^2), the scalar sums 2.3e-8.  So each product starts from zero, where the sum of 16
+// terms of 16 bits loses little, and is added, rounded to nearest, to the
+// thread's sums in registers; the CTAs' sums are added in FP64.  2.3e-8, as the
+// scalar sums, and less on small fields (3 x 128: 3.5e-8 against 9.1e-8); the
+// additions cost less than the shared-memory sums that 8-product chains were
+// added to (a gradient of 32 fields of 128^2: 425 -> 411 us).
 //
 // The scalar form took 7.4 of the 7.7 ms of a gradient on 32 fields of 128^2:
 // two shared-memory loads per multiply-add.  These kernels read each row
@@ -51,6 +54,15 @@ __device__ __forceinline__ void split3(float2 v, uint32_t* s) {
     }
 }
 
+// d = a b, rounded toward zero by the tensor core, into fresh accumulators
+__device__ __forceinline__ void mma_bf16_zero(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};\n"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
+}
+
 template <int AK, int BK>
 struct WgCfg {
     static constexpr int MT = AK == WG_BF16_32 ? 2 : 1;      // m16 tiles: 32 outputs, or 2 x 3 terms
@@ -66,10 +78,8 @@ struct WgCfg {
     static constexpr int RED = MT * 16 * COLS * 4;
     static constexpr int TILES = 2 * AROW + 4 * BROW;
     static_assert(RED <= TILES, "the final sums reuse the tiles' memory");
-    static constexpr int NACC = MT * (3 * NB + 1) * 4;       // accumulators of a thread
-    static constexpr int SMEM = TILES + NACC * THREADS * 4;
+    static constexpr int SMEM = TILES;
     static constexpr int MAXROWS = 64;                       // rows of 128 pixels per CTA
-    static constexpr int FLUSH = 4;                          // rows of one accumulator chain
 };
 
 // Rows r0 .. r0 + rows - 1 of the list (field, 128-pixel segment, y), y
@@ -131,30 +141,18 @@ wgrad_tc_kernel(const void* __restrict__ in, const void* __restrict__ gout, int 
     // acc[m][d][n]: tap column d, input tile n; acc[m][3 NB ...]: the bias
     constexpr int TL = 3 * NB + 1;
     float acc[MT][TL][4];
-    float* mine = reinterpret_cast<float*>(sm + Q::TILES) + tid;     // this thread's sums, stride THREADS
-    auto zero = [&] {
 #pragma unroll
-        for (int m = 0; m < MT; ++m)
+    for (int m = 0; m < MT; ++m)
 #pragma unroll
-            for (int n = 0; n < TL; ++n)
+        for (int n = 0; n < TL; ++n)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[m][n][k] = 0.0f;
+            for (int k = 0; k < 4; ++k) acc[m][n][k] = 0.0f;
+    auto product = [&](float (&s)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+        float t[4];
+        mma_bf16_zero(t, a, b0, b1);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s[k] += t[k];
     };
-    auto flush = [&](bool first) {
-#pragma unroll
-        for (int m = 0; m < MT; ++m)
-#pragma unroll
-            for (int n = 0; n < TL; ++n)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    float* p = &mine[((m * TL + n) * 4 + k) * Q::THREADS];
-                    *p = first ? acc[m][n][k] : *p + acc[m][n][k];
-                }
-        zero();
-    };
-    zero();
-    bool first = true;
-    int chain = 0;
     const int mi = lane >> 3, mr = lane & 7;      // matrix and row of this lane's ldmatrix address
     int sb = 0, sa = 0;                           // ring slots of input row y - 1 and of g
     bool primed = false;
@@ -192,28 +190,21 @@ wgrad_tc_kernel(const void* __restrict__ in, const void* __restrict__ gout, int 
                         ldsm_x4_t(b, B + (16 * q + d + (mi & 1) * 8 + mr) * Q::BP + h * 32 + (mi >> 1) * 16);
 #pragma unroll
                         for (int m = 0; m < MT; ++m) {
-                            mma_bf16(acc[m][4 * d + 2 * h], a[m][0], a[m][1], a[m][2], a[m][3], b[0], b[1]);
-                            mma_bf16(acc[m][4 * d + 2 * h + 1], a[m][0], a[m][1], a[m][2], a[m][3], b[2], b[3]);
+                            product(acc[m][4 * d + 2 * h], a[m], b[0], b[1]);
+                            product(acc[m][4 * d + 2 * h + 1], a[m], b[2], b[3]);
                         }
                     }
                 } else {
                     uint32_t b[2];
                     ldsm_x2_t(b, B + (16 * q + d + (mi & 1) * 8 + mr) * Q::BP);
 #pragma unroll
-                    for (int m = 0; m < MT; ++m)
-                        mma_bf16(acc[m][d], a[m][0], a[m][1], a[m][2], a[m][3], b[0], b[1]);
+                    for (int m = 0; m < MT; ++m) product(acc[m][d], a[m], b[0], b[1]);
                 }
             }
             if (dy == 1) {                        // bias: times ones
 #pragma unroll
-                for (int m = 0; m < MT; ++m)
-                    mma_bf16(acc[m][TL - 1], a[m][0], a[m][1], a[m][2], a[m][3], 0x3f803f80u, 0x3f803f80u);
+                for (int m = 0; m < MT; ++m) product(acc[m][TL - 1], a[m], 0x3f803f80u, 0x3f803f80u);
             }
-        }
-        if (++chain == Q::FLUSH || r + 1 == r1) {
-            flush(first);
-            first = false;
-            chain = 0;
         }
         cp_async_wait<0>();
         __syncthreads();
@@ -235,7 +226,7 @@ wgrad_tc_kernel(const void* __restrict__ in, const void* __restrict__ gout, int 
                         if (bias && (dy != 1 || t != 0 || (e & 1))) continue;
                         const int col = bias ? 9 * NB * 8 : (dy * 3 * NB + n) * 8 + 2 * t + (e & 1);
                         float* p = &red[(m * 16 + g + (e >> 1) * 8) * Q::COLS + col];
-                        const float v = mine[((m * TL + n) * 4 + e) * Q::THREADS];
+                        const float v = acc[m][n][e];
                         *p = k == 0 ? v : *p + v;
                     }
         }
