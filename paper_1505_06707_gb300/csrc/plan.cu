@@ -158,11 +158,24 @@ static std::vector<int32_t> fxv_table(const std::vector<cd>& lv, bool gen, bool 
     }
     return buf;
 }
-// a gain above 2 or a non-finite factor
-static bool fxv_gen(const std::vector<cd>& lv) {
-    for (const cd& x : lv)
-        if (!(std::exp(x.real()) <= 2.0) || !std::isfinite(x.imag())) return true;
-    return false;
+// Factors e^{lv} that are applied in FP64: a gain above 2, a non-finite one, or
+// a loss to less than 1/8 at every point (the nb rows from blk0 on enter twice
+// per step).  Products round to 2^-62 of the line's norm before them, 2^-55 in
+// all at 16384 samples, so a loss that spares no point would take its bits from
+// the result (a uniform e^-14 per step: 1.2e-10 off after 3 steps, now below
+// 2e-15 per step; e^-60: nothing left).  Where some points keep a
+// factor near 1, the FFTs' rounding (2e-16 of the norm, at every point) passes
+// there, in FP64 too.
+static bool fx_gen_factors(const std::vector<cd>& lv, int blk0 = 0, int nb = 0) {
+    const int64_t n = (int64_t)lv.size();
+    double gain = -HUGE_VAL, keep = -HUGE_VAL;
+    for (int64_t i = 0; i < n; ++i) {
+        const cd& x = lv[i];
+        if (!std::isfinite(x.real()) || !std::isfinite(x.imag())) return true;
+        gain = std::max(gain, x.real());
+        keep = std::max(keep, (nb > 0 && (i - blk0 + n) % n < nb ? 2.0 : 1.0) * x.real());
+    }
+    return std::exp(gain) > 2.0 || std::exp(keep) < 0.125;
 }
 
 // Chunked strip solve for thr threads of ch = ceil(nb/thr) rows (thread t: rows
@@ -311,12 +324,8 @@ struct FxMetaHost { int p, gen; const void* d; };
 static int fx_potential_fill(FxPotential& P, const std::vector<cd>& lv) {
     const int64_t n = (int64_t)lv.size();
     double m = 0;
-    bool fin = true;
-    for (const cd& x : lv) {
-        m = std::max(m, x.real());
-        fin = fin && std::isfinite(x.real()) && std::isfinite(x.imag());
-    }
-    FxMetaHost h{0, P.cn_gen || !fin || std::exp(m) > 2.0, nullptr};
+    for (const cd& x : lv) m = std::max(m, x.real());
+    FxMetaHost h{0, P.cn_gen || fx_gen_factors(lv), nullptr};
     h.p = !h.gen && std::exp(m) > 1.01;
     std::vector<int32_t> buf(4 * n);
     host_parallel(n, [&](int64_t b, int64_t e) {
@@ -459,7 +468,7 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
         else cnv = strip_tables_c(mf, g, nb, thr, &T->cnr);
     }
     if (o.prec == SOFT_C128) {
-        const bool gen = T->cn_gen || fxv_gen(tv);
+        const bool gen = T->cn_gen || fx_gen_factors(tv, T->blk0, T->nb);
         if ((rc = upload_i32(&T->cn, cnfx))) return rc;
         const bool s2 = fx_center(lrl, logrm).s2;
         if ((rc = upload_fx_phases(&T->TK, ph, s2))) return rc;
@@ -808,7 +817,7 @@ static int soft_set_potential_impl(soft_plan* P, const double* U, int64_t n) {
     std::vector<cd> tv, tvs;
     potential_logs_1d(*T, nn, P->dt, tv, tvs);
     if (T->prec == SOFT_C128) {
-        const bool gen = T->cn_gen || fxv_gen(tv);
+        const bool gen = T->cn_gen || fx_gen_factors(tv, T->blk0, T->nb);
         for (int i = 0; i < 2; ++i) {
             const std::vector<cd>& v = i ? tvs : tv;
             if (v.empty()) continue;

@@ -1,20 +1,28 @@
 // The complex128 resident 1D step: the scheme of soft1d.cuh with the FFTs,
-// the phase factors and the state in 64-bit fixed point (fix64.cuh), and the
-// strip Crank-Nicolson in FP64.
+// the phase factors, the strip Crank-Nicolson and the state in 64-bit fixed
+// point (fix64.cuh).
 //
 // A step in FP64 (N = 16384) spent 64 clocks of its SM per point, 87 % of
-// them in the FP64 pipe, most of it FFT butterflies.  In fixed point the FFTs
-// and phase factors run on the integer pipes; what stays in FP64 is the strip
-// solve, whose long recurrences want relative precision.
+// them in the FP64 pipe, most of it FFT butterflies.  In fixed point all of it
+// runs on the integer pipes, but for plans with the flag `gen` below.
 //
 // Exponent.  The state is X 2^e.  Each step sums |X|^2 (FP32, of the high
 // words) as the rows are written and shifts the state as the next forward
 // pass loads it, so that its norm stays in (2^59.6, 2^60.8]; the shift is 0
 // in almost every step.  Potential factors enter scaled by 2^-p, p = 0
-// (|e^{-iU tau}| <= 1.01, which the products' range allows) or 1 (<= 2).  A plan with a larger or non-finite factor (a user
-// potential with a large gain) has the flag `gen` in its table: its factors
-// are applied in FP64 and the state is converted anew in every step, so that
-// a sample keeps its relative precision however the factors spread.
+// (|e^{-iU tau}| <= 1.01, which the products' range allows) or 1 (<= 2).  A
+// plan with a larger or non-finite factor, or none above 1/8 (a user potential
+// with a large gain or a loss at every point; fx_gen_factors in plan.cu), or
+// with strip multipliers above 1 (backward steps) has the flag `gen` in its
+// tables: its factors and strip solve are applied in FP64 and the state is
+// converted anew in every step, so that a sample keeps its relative precision
+// however the factors spread.
+//
+// Strip solve (strip_cn_fx): every product rounds to half a unit and the
+// multipliers are at most 1, so the two sweeps leave at most 2^lg units where
+// they grow the rows by 2^lg; a block shifted by lg + 2 bits first (`coarse`,
+// a packet inside the strip) loses those bits of its samples' 59.
+//
 // Code size.  A step runs once through straight-line code, and with 4 to 16
 // warps per SM the instruction fetch bounds it when that code leaves the
 // instruction cache: fully unrolled and templated per pass (225 to 340 KB), the
