@@ -43,8 +43,11 @@ inline void fx_cis_host(uint64_t t, int64_t* c, int64_t* s) {
     *s = (int64_t)((C * ws + (__int128)sn * wc + (1LL << 62)) >> 63);
 }
 
-// the phase ph (radians) in turns 2^-64: ph/(2 pi) to 106 bits, mod 1
+// the phase ph (radians) in turns 2^-64: ph/(2 pi) to 106 bits, mod 1.  Beyond
+// 2^50 (a wall of 10^17, say) the second part of the product would leave the
+// range of its integer; such a phase is reduced by the library.
 inline uint64_t fx_turns_host(double ph) {
+    if (std::fabs(ph) > 0x1p50) ph = std::atan2(std::sin(ph), std::cos(ph));
     const double chi = 0.15915494309189535, clo = -9.839338337591243e-18;
     const double th = ph * chi, tl = std::fma(ph, chi, -th) + ph * clo;
     const double f = th - std::rint(th);

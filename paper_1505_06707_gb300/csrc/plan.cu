@@ -162,10 +162,9 @@ static std::vector<int32_t> fxv_table(const std::vector<cd>& lv, bool gen, bool 
 // a loss to less than 1/8 at every point (the nb rows from blk0 on enter twice
 // per step).  Products round to 2^-62 of the line's norm before them, 2^-55 in
 // all at 16384 samples, so a loss that spares no point would take its bits from
-// the result (a uniform e^-14 per step: 1.2e-10 off after 3 steps, now below
-// 2e-15 per step; e^-60: nothing left).  Where some points keep a
-// factor near 1, the FFTs' rounding (2e-16 of the norm, at every point) passes
-// there, in FP64 too.
+// the result (a uniform e^-14 per step: 1.2e-10 off after 3 steps at 16384
+// samples; e^-60: nothing left).  Where some points keep a factor near 1, the
+// FFTs' rounding (2e-16 of the norm, at every point) passes there, in FP64 too.
 static bool fx_gen_factors(const std::vector<cd>& lv, int blk0 = 0, int nb = 0) {
     const int64_t n = (int64_t)lv.size();
     double gain = -HUGE_VAL, keep = -HUGE_VAL;
