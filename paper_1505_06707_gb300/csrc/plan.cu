@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <thread>
 #include <tuple>
 
@@ -107,6 +108,7 @@ int upload_tw_comp(void** dst, const std::vector<cd>& v, int prec) {
     return upload_tab(dst, v, prec);
 }
 
+static double modulus(cd v) { return std::sqrt(std::norm(v)); }      // (std::abs guards against overflow, slowly)
 static void fx_fill(int32_t* out, const std::vector<cd>& v, double scale) {
     for (size_t i = 0; i < v.size(); ++i) {
         fx_halves_host(std::llrint(v[i].real() * scale * 0x1p62), out + 4 * i);
@@ -122,59 +124,81 @@ int upload_fx(void** dst, const std::vector<cd>& v) {
 int upload_fx_phases(void** dst, const std::vector<double>& ph, int half) {
     std::vector<int32_t> buf(4 * ph.size());
     auto sc = [&](int64_t w) { return half == 0 ? w : half > 0 ? fx_sqrt2_host(w) : (fx_sqrt2_host(w) + 1) >> 1; };
-    for (size_t i = 0; i < ph.size(); ++i) {
-        int64_t c, s;
-        fx_cis_host(fx_turns_host(ph[i]), &c, &s);
-        fx_halves_host(sc(c), &buf[4 * i]);
-        fx_halves_host(sc(s), &buf[4 * i + 2]);
-    }
+    host_parallel((int64_t)ph.size(), [&](int64_t b, int64_t e) {
+        for (int64_t i = b; i < e; ++i) {
+            int64_t c, s;
+            fx_cis_host(fx_turns_host(ph[i]), &c, &s);
+            fx_halves_host(sc(c), &buf[4 * i]);
+            fx_halves_host(sc(s), &buf[4 * i + 2]);
+        }
+    });
     return upload(dst, buf.data(), buf.size() * sizeof(int32_t));
 }
 
+// the factor e^{lv} 2^-p, times sqrt(2) if s2
+static void fx_put_factor(int32_t* out, cd lv, int p, bool s2) {
+    int64_t c, s;
+    fx_cis_host(fx_turns_host(lv.imag()), &c, &s);
+    const int64_t mod = std::llrint(std::exp(lv.real()) * (p ? 0x1p60 : 0x1p61));
+    c = (int64_t)(((__int128)c * mod + (1LL << 60)) >> 61);
+    s = (int64_t)(((__int128)s * mod + (1LL << 60)) >> 61);
+    fx_halves_host(s2 ? fx_sqrt2_host(c) : c, out);
+    fx_halves_host(s2 ? fx_sqrt2_host(s) : s, out + 2);
+}
+// largest real part of the logarithms, the same with those of the nb rows from
+// blk0 on doubled (factors that enter twice per step), and whether all are finite
+struct LogRange { double gain, keep; bool finite; };
+static LogRange log_range(const std::vector<cd>& lv, int64_t blk0 = 0, int64_t nb = 0) {
+    const int64_t n = (int64_t)lv.size();
+    LogRange R{-HUGE_VAL, -HUGE_VAL, true};
+    std::mutex mx;
+    host_parallel(n, [&](int64_t b, int64_t e) {
+        LogRange r{-HUGE_VAL, -HUGE_VAL, true};
+        for (int64_t i = b; i < e; ++i) {
+            const double x = lv[i].real();
+            const int64_t j = i < blk0 ? i - blk0 + n : i - blk0;
+            r.finite = r.finite && std::isfinite(x) && std::isfinite(lv[i].imag());
+            r.gain = std::max(r.gain, x);
+            r.keep = std::max(r.keep, j < nb ? 2.0 * x : x);
+        }
+        std::lock_guard<std::mutex> l(mx);
+        R.finite = R.finite && r.finite;
+        R.gain = std::max(R.gain, r.gain);
+        R.keep = std::max(R.keep, r.keep);
+    });
+    return R;
+}
+// Factors e^{lv} that are applied in FP64: a gain above 2, a non-finite one, or
+// a loss to less than 1/8 at every point.  Products round to 2^-62 of the line's
+// norm before them, 2^-55 in all at 16384 samples, so a loss that spares no
+// point would take its bits from the result (a uniform e^-14 per step: 1.2e-10
+// off after 3 steps at 16384 samples; e^-60: nothing left).  Where some points
+// keep a factor near 1, the FFTs' rounding (2e-16 of the norm, at every point)
+// passes there, in FP64 too.
+static bool fx_gen_factors(const LogRange& r) {
+    return !r.finite || std::exp(r.gain) > 2.0 || std::exp(r.keep) < 0.125;
+}
 // potential table of the fixed-point step (soft1d_fix.cuh, FxV) from the
 // factors' logarithms: the factors times 2^-p, p = 0 (|v| <= 1.01) or 1 (<= 2),
 // and sqrt(2) if s2 (the last inverse pass's share), then the entry
-// (p, gen, 0, 0) and the factors as double2, which plans with gen use
+// (p, gen, 0, 0) and, for plans with gen, the factors as double2 instead
 static std::vector<int32_t> fxv_table(const std::vector<cd>& lv, bool gen, bool s2) {
     const size_t n = lv.size();
     std::vector<int32_t> buf(8 * n + 4, 0);
-    double m = 0;
-    for (const cd& x : lv) m = std::max(m, std::exp(x.real()));
-    const int p = !gen && m > 1.01 ? 1 : 0;
-    for (size_t i = 0; i < n && !gen; ++i) {
-        int64_t c, s;
-        fx_cis_host(fx_turns_host(lv[i].imag()), &c, &s);
-        const int64_t mod = std::llrint(std::exp(lv[i].real()) * (p ? 0x1p60 : 0x1p61));
-        c = (int64_t)(((__int128)c * mod + (1LL << 60)) >> 61);
-        s = (int64_t)(((__int128)s * mod + (1LL << 60)) >> 61);
-        fx_halves_host(s2 ? fx_sqrt2_host(c) : c, &buf[4 * i]);
-        fx_halves_host(s2 ? fx_sqrt2_host(s) : s, &buf[4 * i + 2]);
-    }
+    const int p = !gen && std::exp(log_range(lv).gain) > 1.01 ? 1 : 0;
+    host_parallel((int64_t)n, [&](int64_t b, int64_t e) {
+        for (int64_t i = b; i < e; ++i) {
+            if (gen) {
+                const cd v = std::exp(lv[i]);
+                std::memcpy(buf.data() + 4 * n + 4 + 4 * i, &v, 16);
+            } else {
+                fx_put_factor(&buf[4 * i], lv[i], p, s2);
+            }
+        }
+    });
     buf[4 * n] = p;
     buf[4 * n + 1] = gen;
-    for (size_t i = 0; i < n; ++i) {
-        const cd v = std::exp(lv[i]);
-        std::memcpy(buf.data() + 4 * n + 4 + 4 * i, &v, 16);
-    }
     return buf;
-}
-// Factors e^{lv} that are applied in FP64: a gain above 2, a non-finite one, or
-// a loss to less than 1/8 at every point (the nb rows from blk0 on enter twice
-// per step).  Products round to 2^-62 of the line's norm before them, 2^-55 in
-// all at 16384 samples, so a loss that spares no point would take its bits from
-// the result (a uniform e^-14 per step: 1.2e-10 off after 3 steps at 16384
-// samples; e^-60: nothing left).  Where some points keep a factor near 1, the
-// FFTs' rounding (2e-16 of the norm, at every point) passes there, in FP64 too.
-static bool fx_gen_factors(const std::vector<cd>& lv, int blk0 = 0, int nb = 0) {
-    const int64_t n = (int64_t)lv.size();
-    double gain = -HUGE_VAL, keep = -HUGE_VAL;
-    for (int64_t i = 0; i < n; ++i) {
-        const cd& x = lv[i];
-        if (!std::isfinite(x.real()) || !std::isfinite(x.imag())) return true;
-        gain = std::max(gain, x.real());
-        keep = std::max(keep, (nb > 0 && (i - blk0 + n) % n < nb ? 2.0 : 1.0) * x.real());
-    }
-    return std::exp(gain) > 2.0 || std::exp(keep) < 0.125;
 }
 
 // Chunked strip solve for thr threads of ch = ceil(nb/thr) rows (thread t: rows
@@ -214,7 +238,7 @@ static StripScan strip_scan(const std::vector<cd>& mf, const std::vector<cd>& g,
             for (int t = 0; t < thr; ++t) {
                 s[(size_t)r * thr + t] = prod[t];
                 const int l = t & 31;
-                if (d ? l + D < 32 : l >= D) big = std::max(big, std::abs(prod[t]));
+                if (d ? l + D < 32 : l >= D) big = std::max(big, modulus(prod[t]));
             }
             if (!(big <= tiny)) Q.rounds[d] = r + 1;
             std::vector<cd> nx = prod;
@@ -239,7 +263,7 @@ static StripScan strip_scan(const std::vector<cd>& mf, const std::vector<cd>& g,
             for (int w = 0; w + k <= nw; ++w) {
                 cd p = 1.0;
                 for (int q = 0; q < k; ++q) p *= s[(size_t)6 * thr + w + q];
-                big = std::max(big, std::abs(p));
+                big = std::max(big, modulus(p));
             }
             if (big <= tiny) { Q.span[d] = k; break; }
         }
@@ -267,43 +291,44 @@ std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vecto
     std::vector<double> y(nb);
     *gen = false;
     for (int i = 0; i < nb; ++i) {
-        gy = std::abs(mf[i]) * gy + 1.0;
+        gy = modulus(mf[i]) * gy + 1.0;
         y[i] = gy;
         grow = std::max(grow, gy);
-        if (!(std::abs(mf[i]) <= 1.0 + 1e-12 && std::abs(g[i]) <= 1.9)) *gen = true;
+        if (!(modulus(mf[i]) <= 1.0 + 1e-12 && modulus(g[i]) <= 1.9)) *gen = true;
     }
     double gx = 0.0;
     for (int i = nb - 1; i >= 0; --i) {
-        gx = std::abs(mb[i]) * gx + std::abs(g[i]) * y[i];
+        gx = modulus(mb[i]) * gx + modulus(g[i]) * y[i];
         grow = std::max(grow, gx);
     }
     const int lg = (int)std::ceil(std::log2(grow));
     if (!(lg >= 0 && lg <= 10)) *gen = true;
     const StripScan Q = strip_scan(mf, g, nb, thr, 0x1p-70);
     const std::vector<cd> &m = Q.m, &gg = Q.g;
-    std::vector<cd> all = m;
-    all.insert(all.end(), gg.begin(), gg.end());
-    all.insert(all.end(), Q.scan[0].begin(), Q.scan[0].end());
-    all.insert(all.end(), Q.scan[1].begin(), Q.scan[1].end());
-    std::vector<int32_t> buf(4 + 4 * (all.size() + m.size() + gg.size()), 0);
+    const size_t nf = m.size() + gg.size() + Q.scan[0].size() + Q.scan[1].size();
+    std::vector<int32_t> buf(4 + 4 * (nf + m.size() + gg.size()), 0);
     buf[0] = *gen ? 0 : lg;
     buf[1] = Q.rounds[0];
     buf[2] = Q.rounds[1];
     buf[3] = Q.span[0] | Q.span[1] << 16;
     if (!*gen) {
-        std::vector<int32_t> f(4 * all.size());
-        fx_fill(f.data(), all, 1.0);
-        std::memcpy(buf.data() + 4, f.data(), 16 * all.size());
+        int32_t* f = buf.data() + 4;
+        for (const std::vector<cd>* v : {&m, &gg, &Q.scan[0], &Q.scan[1]}) {
+            fx_fill(f, *v, 1.0);
+            f += 4 * v->size();
+        }
     }
-    std::memcpy(buf.data() + 4 + 4 * all.size(), m.data(), 16 * m.size());
-    std::memcpy(buf.data() + 4 + 4 * (all.size() + m.size()), gg.data(), 16 * gg.size());
+    std::memcpy(buf.data() + 4 + 4 * nf, m.data(), 16 * m.size());
+    std::memcpy(buf.data() + 4 + 4 * (nf + m.size()), gg.data(), 16 * gg.size());
     return buf;
 }
 
 int upload_i32(void** dst, const std::vector<int32_t>& v) { return upload(dst, v.data(), v.size() * 4); }
 
 void host_parallel(int64_t n, const std::function<void(int64_t, int64_t)>& fn) {
-    const int64_t nt = std::max<int64_t>(1, std::min<int64_t>({(int64_t)std::thread::hardware_concurrency(), 32, n / 4096}));
+    if (n < 8192) return fn(0, n);      // (a thread costs as much as about 2000 factors)
+    static const int64_t cores = std::thread::hardware_concurrency();      // (the query reads a file)
+    const int64_t nt = std::max<int64_t>(1, std::min<int64_t>({cores, 32, n / 4096}));
     std::vector<std::thread> pool;
     int64_t done = 0;              // handed to threads; the rest runs here
     try {
@@ -322,11 +347,10 @@ void host_parallel(int64_t n, const std::function<void(int64_t, int64_t)>& fn) {
 struct FxMetaHost { int p, gen; const void* d; };
 static int fx_potential_fill(FxPotential& P, const std::vector<cd>& lv) {
     const int64_t n = (int64_t)lv.size();
-    double m = 0;
-    for (const cd& x : lv) m = std::max(m, x.real());
-    FxMetaHost h{0, P.cn_gen || fx_gen_factors(lv), nullptr};
-    h.p = !h.gen && std::exp(m) > 1.01;
-    std::vector<int32_t> buf(4 * n);
+    const LogRange r = log_range(lv);
+    FxMetaHost h{0, P.cn_gen || fx_gen_factors(r), nullptr};
+    h.p = !h.gen && std::exp(r.gain) > 1.01;
+    const std::unique_ptr<int32_t[]> buf(new int32_t[4 * (size_t)n]);      // (pages first touched by the threads)
     host_parallel(n, [&](int64_t b, int64_t e) {
         for (int64_t i = b; i < e; ++i) {
             if (h.gen) {
@@ -334,16 +358,12 @@ static int fx_potential_fill(FxPotential& P, const std::vector<cd>& lv) {
                 std::memcpy(&buf[4 * i], &v, 16);
                 continue;
             }
-            int64_t c, s;
-            fx_cis_host(fx_turns_host(lv[i].imag()), &c, &s);
-            const int64_t mod = std::llrint(std::exp(lv[i].real()) * (h.p ? 0x1p60 : 0x1p61));
-            fx_halves_host((int64_t)(((__int128)c * mod + (1LL << 60)) >> 61), &buf[4 * i]);
-            fx_halves_host((int64_t)(((__int128)s * mod + (1LL << 60)) >> 61), &buf[4 * i + 2]);
+            fx_put_factor(&buf[4 * i], lv[i], h.p, false);
         }
     });
     // gen plans read the same buffer as double2
     if (h.gen) h.d = P.tab;
-    int rc = cuda_status(cudaMemcpy(P.tab, buf.data(), 16 * (size_t)n, cudaMemcpyHostToDevice));
+    int rc = cuda_status(cudaMemcpy(P.tab, buf.get(), 16 * (size_t)n, cudaMemcpyHostToDevice));
     return rc ? rc : cuda_status(cudaMemcpy(P.meta, &h, sizeof(h), cudaMemcpyHostToDevice));
 }
 int FxPotential::build(const std::vector<cd>& lv) {
@@ -435,8 +455,8 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
     // kinetic tables in the forward FFT's output order, 1/N folded in
     // (complex128: the fixed-point passes carry the 1/N)
     const std::vector<int> perm = dif_output_order(logn, logrm);
-    std::vector<cd> tk(n), tkh(n), tv, tvs;
-    std::vector<double> ph(n), phh(n);        // complex128: their phases
+    std::vector<cd> tv, tvs;
+    std::vector<double> ph(n), phh(n);        // their phases
     const std::vector<cd> w = o.prec == SOFT_C64 ? pass_twiddles(logn, logrm) : std::vector<cd>();
     // The step kernel reads them in its last forward pass, whose butterflies
     // hold R consecutive positions b*R + m (R its radix): entry (b, m) is
@@ -448,8 +468,6 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
         const int q = (p % Rl) * nbf + p / Rl;
         ph[q] = -0.5 * k * k * tau;
         phh[q] = -0.25 * k * k * tau;
-        tk[q] = std::polar(1.0 / n, ph[q]);
-        tkh[q] = std::polar(1.0 / n, phh[q]);
     }
     potential_logs_1d(*T, n, tau, tv, tvs);
     // Strip CN tables of the T = n >> loge threads; M is complex symmetric, so
@@ -467,7 +485,7 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
         else cnv = strip_tables_c(mf, g, nb, thr, &T->cnr);
     }
     if (o.prec == SOFT_C128) {
-        const bool gen = T->cn_gen || fx_gen_factors(tv, T->blk0, T->nb);
+        const bool gen = T->cn_gen || fx_gen_factors(log_range(tv, T->blk0, T->nb));
         if ((rc = upload_i32(&T->cn, cnfx))) return rc;
         const bool s2 = fx_center(lrl, logrm).s2;
         if ((rc = upload_fx_phases(&T->TK, ph, s2))) return rc;
@@ -477,6 +495,11 @@ int make_tables_1d(Tables1D* T, int n, double a, double b, double R0, double the
         return tvs.empty() ? SOFT_OK : upload_i32(&T->TVs, fxv_table(tvs, gen, false));
     }
     if ((rc = upload_c(&T->cn, cnv, o.prec))) return rc;
+    std::vector<cd> tk(n), tkh(n);
+    for (int q = 0; q < n; ++q) {
+        tk[q] = std::polar(1.0 / n, ph[q]);
+        tkh[q] = std::polar(1.0 / n, phh[q]);
+    }
     if ((rc = upload_tab(&T->TK, tk, o.prec))) return rc;
     if ((rc = upload_tab(&T->TKh, tkh, o.prec))) return rc;
     if ((rc = upload_vtab(&T->TV, vexp(tv), o.prec))) return rc;
@@ -816,7 +839,7 @@ static int soft_set_potential_impl(soft_plan* P, const double* U, int64_t n) {
     std::vector<cd> tv, tvs;
     potential_logs_1d(*T, nn, P->dt, tv, tvs);
     if (T->prec == SOFT_C128) {
-        const bool gen = T->cn_gen || fx_gen_factors(tv, T->blk0, T->nb);
+        const bool gen = T->cn_gen || fx_gen_factors(log_range(tv, T->blk0, T->nb));
         for (int i = 0; i < 2; ++i) {
             const std::vector<cd>& v = i ? tvs : tv;
             if (v.empty()) continue;
