@@ -244,7 +244,11 @@ static int wgrad(NNState& S, const void* in, const void* g, int F, int H, int W,
                  cudaStream_t st) {
     using Q = WgCfg<AK, BK>;
     const int64_t nrows = (int64_t)F * H * (W / 128);
-    const int rows = (int)std::max<int64_t>(1, std::min<int64_t>(Q::MAXROWS, (nrows + 151) / 152));
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
+        return SOFT_ERR_CUDA;
+    const int rows = (int)std::max<int64_t>(1, std::min<int64_t>(Q::MAXROWS, (nrows + nsm - 1) / nsm));
     const int64_t ncta = (nrows + rows - 1) / rows;
     if (ncta > 0x7fffffff) return SOFT_ERR_TOO_LARGE;
     if (ncta * Q::NP > S.part_cap) {
