@@ -165,7 +165,7 @@ static LogRange log_range(const std::vector<cd>& lv, int64_t blk0 = 0, int64_t n
         R.finite = R.finite && r.finite;
         R.gain = std::max(R.gain, r.gain);
         R.keep = std::max(R.keep, r.keep);
-    });
+    }, 1 << 17);
     return R;
 }
 // Factors e^{lv} that are applied in FP64: a gain above 2, a non-finite one, or
@@ -325,10 +325,10 @@ std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vecto
 
 int upload_i32(void** dst, const std::vector<int32_t>& v) { return upload(dst, v.data(), v.size() * 4); }
 
-void host_parallel(int64_t n, const std::function<void(int64_t, int64_t)>& fn) {
-    if (n < 8192) return fn(0, n);      // (a thread costs as much as about 2000 factors)
+void host_parallel(int64_t n, const std::function<void(int64_t, int64_t)>& fn, int64_t grain) {
+    if (n < 2 * grain) return fn(0, n);
     static const int64_t cores = std::thread::hardware_concurrency();      // (the query reads a file)
-    const int64_t nt = std::max<int64_t>(1, std::min<int64_t>({cores, 32, n / 4096}));
+    const int64_t nt = std::max<int64_t>(1, std::min<int64_t>({cores, 32, n / grain}));
     std::vector<std::thread> pool;
     int64_t done = 0;              // handed to threads; the rest runs here
     try {

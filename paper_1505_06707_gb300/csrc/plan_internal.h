@@ -29,8 +29,6 @@ int upload_tab(void** dst, const std::vector<cd>& v, int prec);
 int upload_vtab(void** dst, const std::vector<cd>& v, int prec);
 int upload_tw(void** dst, const std::vector<cd>& v, int prec);
 int upload_tw_comp(void** dst, const std::vector<cd>& v, int prec);
-// rewrite an existing device buffer in place (same size and format as the
-// matching upload_*), so that pointers held by kernels and graphs stay valid
 // fixed-point factors (fix64.cuh): values, and phases e^{i ph} times 2^(half/2)
 int upload_fx(void** dst, const std::vector<cd>& v);
 int upload_fx_phases(void** dst, const std::vector<double>& ph, int half);
@@ -38,8 +36,9 @@ int upload_i32(void** dst, const std::vector<int32_t>& v);
 std::vector<int32_t> strip_tables_fx(const std::vector<cd>& mf, const std::vector<cd>& mb, const std::vector<cd>& g,
                                      int nb, int thr, bool* gen);
 std::vector<cd> strip_tables_c(const std::vector<cd>& mf, const std::vector<cd>& g, int nb, int thr, int* cnr);
-// fn(begin, end) over 0 .. n - 1 on host threads (the calling one if none can start)
-void host_parallel(int64_t n, const std::function<void(int64_t, int64_t)>& fn);
+// fn(begin, end) over 0 .. n - 1 on host threads, each at least grain (a thread
+// costs as much as about 2000 factors); on the calling one if none can start
+void host_parallel(int64_t n, const std::function<void(int64_t, int64_t)>& fn, int64_t grain = 4096);
 // Potential factors of a complex128 2D or 3D plan: factors e^{lv} 2^-p
 // (fix64.cuh) or, for gen plans, double2 in the same buffer, and the device
 // FxMeta record (soft2d_fix.cuh).  build allocates; refill rewrites in place.
@@ -50,6 +49,8 @@ struct FxPotential {
     int refill(const std::vector<cd>& lv);
     ~FxPotential();
 };
+// rewrite an existing device buffer in place (same size and format as the
+// matching upload_*), so that pointers held by kernels and graphs stay valid
 int refill_c(void* dst, const std::vector<cd>& v, int prec);
 int refill_vtab(void* dst, const std::vector<cd>& v, int prec);
 struct Plan2D;
