@@ -1,20 +1,20 @@
 // Complex128 FFTs in 64-bit fixed point.
 //
 // GB300 runs 2 FP64 instructions per clock and SM, but 64 32 x 32 -> 64 bit
-// multiply-adds (mad.wide) and 64 64-bit additions (measured: DFMA 1.9,
-// mad.wide 58, add.s64 60 per clock and SM, the two integer pipes
-// together).  A complex product of 64-bit fixed-point numbers takes 12
-// mad.wide, 0.19 clocks of an SM against 2 clocks for the 4 FP64
-// instructions, and a complex sum and difference 0.06 against 2.  So the
-// complex128 FFTs run on integers: a line's samples are X 2^e with one
-// exponent e per line and X a 64-bit integer.
+// multiply-adds (mad.wide) or 64-bit additions (probe/alu_peak.cu: DFMA 1.98,
+// mad.wide 62.7, add.s64 63.7 per clock and SM, the two in turn 63.6).  A
+// complex product of 64-bit fixed-point numbers takes 12 mad.wide, 0.19 clocks
+// of an SM against 2 clocks for the 4 FP64 instructions (0.51 with the halves'
+// splitting and carries, fx_mul), and a complex sum and difference 0.06 against
+// 2.  So the complex128 FFTs run on integers: a line's samples are X 2^e with
+// one exponent e per line and X a 64-bit integer.
 //
 // Range.  Every operator between two conversions is unitary (FFT passes with
 // their power-of-2 shares of 1/N, phase factors), so the Euclidean norm of a
 // line is kept, and it bounds every component.  Lines enter with
 // norm < FX_NORM = 2^60.8; a radix-16 butterfly, unscaled, grows that to
-// 2^62.8 < 2^63 at most, and each pass shifts back what the unitary scaling
-// allows (FxSched).
+// 2^62.8 < 2^63 at most, and the products after it, or before the next one,
+// take the unitary scaling back (FxPass, fx_center).
 //
 // Accuracy.  Products round to 1/2 unit in the last place.  With the norm
 // between 2^59.6 and 2^60.8 units, k roundings of n complex samples leave
@@ -22,8 +22,9 @@
 // FFT of n = 16384 (k = 14), less for shorter lines; the FP64 passes, whose
 // roundings are relative to each sample, leave 2e-16 to 4e-16.
 //
-// A factor w with |w| <= 1 (up to 1.9 where the comments say so) is stored as W = w 2^62 split into signed 32-bit
-// halves, W = h 2^32 + l: int4 (re.h, re.l, im.h, im.l), l > -2^31.
+// A factor w with |w| <= 1 (up to 1.9 where the comments say so) is stored as
+// W = w 2^62 split into signed 32-bit halves, W = h 2^32 + l: int4 (re.h, re.l,
+// im.h, im.l), l > -2^31.
 #pragma once
 #include "device_common.cuh"
 

@@ -2,12 +2,14 @@
 // instantiations of the A-apply and preconditioner passes and the vector /
 // scalar kernels of the iteration.
 //
-// Pass precisions (compute R, vector I/O IO):
-//   FP64 path (precond 0, 1)          A and P^-1: R double, IO complex128
-//   FP32 preconditioner (precond 4)   P^-1: R float, IO complex128
-//   mixed iteration (precond 5)       A and P^-1: R float, IO complex64; the
-//                                     energies that fall back: A with R double,
-//                                     IO complex64
+// Pass arithmetic and vector I/O:
+//   precond 0, 1                      A and P^-1: FFTs and band products in 64-bit
+//                                     fixed point, the rest in FP64 (pcg_fix.cuh),
+//                                     I/O complex128
+//   FP32 preconditioner (precond 4)   P^-1: FP32, I/O complex128 (A as above)
+//   mixed iteration (precond 5)       A and P^-1: FP32, I/O complex64; the
+//                                     energies that fall back: A as above with
+//                                     I/O complex64
 #include "pcg.cuh"
 #include "pcg_fix.cuh"
 #include "pcg_launch.h"
@@ -16,7 +18,7 @@ namespace soft {
 
 namespace {
 
-constexpr int TWP = 2;    // columns per CTA of the FP64 column passes
+constexpr int TWP = 2;    // columns per CTA of the fixed-point column passes
 // columns per CTA of the FP32 column passes: 8 (64-byte row runs of
 // complex64), fewer where that would exceed 1024 threads
 template <int LN>

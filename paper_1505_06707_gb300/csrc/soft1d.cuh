@@ -66,7 +66,7 @@ __device__ __forceinline__ float2 tmulc(float2 x, float4 t) {
 // exact to ~2^-48 and only the data's own roundings remain.
 // Complex128 plans of the 1D step store fixed-point factors (TwFix,
 // soft1d_fix.cuh), and so do the complex128 line passes of the 2D and 3D steps
-// (soft2d_fix.cuh); the stationary solvers' FP64 passes use the bases.
+// (soft2d_fix.cuh) and the stationary solvers' complex128 passes (pcg_fix.cuh).
 struct TwFix { int4 v; };
 constexpr int FX_FR = 68;       // field factors of the fixed-point step behind its 2 E per-row ones
 

@@ -12,12 +12,13 @@
 // terms that add up to them exactly (8 + 8 + 8 bits), so the products are
 // those of the FP32 value.  The tensor cores' FP32 accumulation truncates, a
 // bias that grows with the chain: 8 products deep it left 5.5e-8 of the gradient
-// of exact operands (32 fields of 128^2), the scalar sums 2.3e-8.  So each product starts from zero, where the sum of 16
-// terms of 16 bits loses little, and is added, rounded to nearest, to the
-// thread's sums in registers; the CTAs' sums are added in FP64.  2.3e-8, as the
-// scalar sums, and less on small fields (3 x 128: 3.5e-8 against 9.1e-8); the
-// additions cost less than the shared-memory sums that 8-product chains were
-// added to (a gradient of 32 fields of 128^2: 425 -> 411 us).
+// of exact operands (32 fields of 128^2), the scalar sums 2.3e-8.  So each
+// product starts from zero, where the sum of 16 terms of 16 bits loses little,
+// and is added, rounded to nearest, to the thread's sums in registers; the CTAs'
+// sums are added in FP64.  2.3e-8, as the scalar sums, and less on small fields
+// (3 x 128: 3.5e-8 against 9.1e-8); the additions cost less than the
+// shared-memory sums that 8-product chains were added to (a gradient of 32
+// fields of 128^2: 425 -> 411 us).
 //
 // The scalar form took 7.4 of the 7.7 ms of a gradient on 32 fields of 128^2:
 // two shared-memory loads per multiply-add.  These kernels read each row
