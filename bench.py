@@ -57,32 +57,13 @@ def _hbm_peak(d):
     return 6800.0
 
 
-# DRAM bytes (read + write) of one launch of the dominant kernel, from an
-# ncu capture of that launch (dram__bytes_read.sum + dram__bytes_write.sum),
-# valid only while the kernel sources hash to the same value and the launch
-# has the same instances and steps.
-TRAFFIC_MEASURED = {
-    "c64": {"src_sha1": "017cc908ca484d84bee6e1e40864622eadd99c5a", "n": 16384, "instances": 988,
-            "steps": 256, "bytes": 133621504 + 78311936},
-}
-
-
 def _kernel_src_sha1():
     import hashlib
     h = hashlib.sha1()
-    for f in ("soft1d.cuh", "device_common.cuh"):
+    for f in ("soft1d.cuh", "soft1d_fix.cuh", "fix64.cuh", "device_common.cuh"):
         with open(os.path.join(ROOT, "paper_1505_06707_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
-
-
-def _traffic(prec, n, instances, steps):
-    t = TRAFFIC_MEASURED.get(prec)
-    if not t or t["src_sha1"] != _kernel_src_sha1():
-        return None
-    if (t["n"], t["instances"], t["steps"]) != (n, instances, steps):
-        return None
-    return float(t["bytes"])
 
 
 # FMA lanes per SM and clock: 128 FP32 lanes; FP64 2 DFMA per clock per SM
@@ -91,10 +72,10 @@ def _traffic(prec, n, instances, steps):
 FP32_FMA_PER_SM_CLK = 128
 FP64_FMA_PER_SM_CLK = 2
 # The complex128 kernels compute in 64-bit fixed point on the integer pipes:
-# 59 32 x 32 -> 64 bit multiply-adds or 64-bit additions per clock and SM
-# (measured 58 and 60).  A radix-2 butterfly, 10 flops, is a complex product of
-# 12 multiply-adds and 4 additions: 1.6 slots per flop.
-FX_SLOTS_PER_SM_CLK = 59
+# 63 32 x 32 -> 64 bit multiply-adds or 64-bit additions per clock and SM (the
+# probe: 62.7, 63.7, and 63.6 of both in turn).  A radix-2 butterfly, 10 flops,
+# is a complex product of 12 multiply-adds and 4 additions: 1.6 slots per flop.
+FX_SLOTS_PER_SM_CLK = 63
 FX_SLOTS_PER_FLOP = 1.6
 
 
@@ -115,8 +96,9 @@ def alu_peaks(torch=None, dev=0):
 
 
 def alu_probe(iters=4096):
-    """The FMA throughput probe (paper_1505_06707_gb300/probe/alu_peak.cu):
-    measured FP32 and FP64 rates, TFLOP/s."""
+    """The throughput probe (paper_1505_06707_gb300/probe/alu_peak.cu): measured
+    FP32 and FP64 rates, TFLOP/s, and the two operations of the fixed-point
+    kernels, 10^12 per second."""
     import ctypes as C
     lib = C.CDLL(os.path.join(ROOT, "paper_1505_06707_gb300", "_lib", "libaluprobe.so"))
     lib.alu_fma_rate.argtypes = [C.c_int, C.c_int, C.POINTER(C.c_double), C.POINTER(C.c_double)]
@@ -126,6 +108,11 @@ def alu_probe(iters=4096):
         rc = lib.alu_fma_rate(f64, it, C.byref(fl), C.byref(ms))
         out[name + "_tflops"] = fl.value / 1e12 if rc == 0 else None
         out[name + "_ms_per_launch"] = ms.value if rc == 0 else None
+    lib.alu_int_rate.argtypes = lib.alu_fma_rate.argtypes
+    for name, what in (("mad_wide", 0), ("add64", 1), ("mad_wide_add64", 2)):
+        ops, ms = C.c_double(), C.c_double()
+        rc = lib.alu_int_rate(what, iters, C.byref(ops), C.byref(ms))
+        out[name + "_tops"] = ops.value / 1e12 if rc == 0 else None
     return out
 
 
@@ -839,12 +826,12 @@ def measure_w2(S, torch, dev, args, prec_name, steps, warmup, world=1, with_e2e=
 
 
 # DRAM bytes (read + write) per launch of the complex128 N = 16384 group
-# kernel, from an ncu capture of 69 instances x 16 steps (29.30 MB) scaled by
+# kernel, from an ncu capture of 69 instances x 16 steps (24.03 MB) scaled by
 # the instance count: each instance's 256 KB state is read and written back
 # once per launch and stays in L2 between steps (the tables are shared).
 # Valid while the kernel sources hash to src_sha1.
-TRAFFIC_C128 = {"src_sha1": "a55f0e092028fe20c4774a2cfdc64a50d55e9298",
-                "per_instance": (25108992 + 4186368) / 69}
+TRAFFIC_C128 = {"src_sha1": "f6c331958ca0a1fdc2e8a8f7ab8e5fccaf328800",
+                "per_instance": (19851264 + 4177152) / 69}
 
 
 def roofline_w2(torch, dev, m, prec_name):
