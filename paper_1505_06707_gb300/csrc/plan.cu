@@ -1113,8 +1113,9 @@ int soft_plan::ensure_side() {
 }
 
 // The schedule autotuner of a batch plan: one chunk of 16 steps on a constant,
-// non-zero state (as autotune_size: a zero one is not a step's usual work) with the persistent kernel and with one kernel per size group
-// (each timed after a warm-up run); the faster is kept.
+// non-zero state (as autotune_size: a zero one is not a step's usual work) with
+// the persistent kernel and with one kernel per size group (each timed after a
+// warm-up run); the faster is kept.
 int soft_plan::time_schedules() {
     int rc = ensure_side();
     if (rc) return rc;
